@@ -1,0 +1,132 @@
+// fixed.cuh -- fixed-point arithmetic of the FP64 deposits.
+//
+// The FP64 pipe of sm_103a takes one warp instruction per 64 clocks and SM
+// sub-partition; a 32 x 32 + 64 bit multiply-add takes two (measured: FMA,
+// add and conversion 64 to 77 clocks, mad.wide 2.1, 64-bit add 2.05).  The
+// weighted sums of Eq. 4 are sums of products of numbers in [0, 1] (weights)
+// and marker values, so they are formed in 64-bit integers, each factor in
+// two limbs of 28 low bits and the rest:
+//   weights of a (column, v_x row) pair     2^-57     (FX_A)
+//   (v_y, v_z) cell weights                 2^-56     (FX_Q)
+//   marker values                           2^(el - 1078), el the exponent
+//                                           field of the column's largest value
+//   sums of products                        h + m 2^-28 units of 2^-57
+// The low limbs are signed, so that the product of two of them, which is
+// left out, is at most a quarter of the sum's unit, of either sign.  Against
+// exact rational sums of 4 to 12 markers with values over one e-fold: f
+// 7e-17 rms, weights 5e-17 (the same sums in FP64: 1.3e-16 and 1e-16).
+#pragma once
+#include <cuda_runtime.h>
+
+namespace avl {
+
+constexpr long long FX_ONE = 1ll << 52;       // 1 of a 52-bit fraction (position, row weights)
+constexpr int FX_LIMB = 28;
+constexpr int FX_PAIRS = 56;                  // products of weights <= 1 a sum takes before it is flushed:
+                                              // |h| stays below 56 2^57 + 2^59, |m| below 56 (2^56 + 2^55)
+constexpr int FX_EMIN = 128;                  // smallest exponent of a column's unit: values below 2^-951 count as 0
+
+// v = h 2^28 + l, -2^27 <= l < 2^27
+struct Limbs {
+    int h, l;
+};
+__device__ __forceinline__ Limbs fx_split(long long v)
+{
+    const int l = ((int)v << (32 - FX_LIMB)) >> (32 - FX_LIMB);
+    return {(int)(v >> FX_LIMB) + (l < 0 ? 1 : 0), l};
+}
+
+// c += a b.  The product and the sum as two PTX instructions with the
+// accumulator updated in place, which become one multiply-add: 48 of them
+// take 114 clocks and 60 instructions of a warp; as mad.wide.s32 153 clocks
+// and 124 instructions, from c += (long long)a * b 197 and 166.
+__device__ __forceinline__ void mad_wide(long long& c, int a, int b)
+{
+    long long t;
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(t) : "r"(a), "r"(b));
+    asm("add.s64 %0, %0, %1;" : "+l"(c) : "l"(t));
+}
+
+// a b / 2^56, to nearest but for the product of the low limbs (at most a
+// quarter unit); exact for a = 0 or b = 0, and never negative for a, b >= 0
+__device__ __forceinline__ long long fx_mul(Limbs a, Limbs b)
+{
+    long long m = 1ll << (FX_LIMB - 1);
+    mad_wide(m, a.h, b.l);
+    mad_wide(m, a.l, b.h);
+    long long h = m >> FX_LIMB;
+    mad_wide(h, a.h, b.h);
+    return h;
+}
+
+// sum of products, h + m 2^-28
+struct FxSum {
+    long long h, m;
+    __device__ __forceinline__ void clear() { h = m = 0; }
+    __device__ __forceinline__ void add(Limbs a, Limbs b)
+    {
+        mad_wide(h, a.h, b.h);
+        mad_wide(m, a.h, b.l);
+        mad_wide(m, a.l, b.h);
+    }
+    // whole units, to nearest
+    __device__ __forceinline__ long long units() const { return h + ((m + (1 << (FX_LIMB - 1))) >> FX_LIMB); }
+    // the same value with 0 <= m < 2^28
+    __device__ __forceinline__ void carry()
+    {
+        h += m >> FX_LIMB;
+        m &= (1ll << FX_LIMB) - 1;
+    }
+    __device__ __forceinline__ void shr(int s)
+    {
+        h >>= s;
+        m >>= s;
+    }
+};
+
+// f as mant 2^(e - 1078), |mant| < 2^56, e >= 1 the exponent field of f
+__device__ __forceinline__ long long fx_value(double f, int& e)
+{
+    const long long b = __double_as_longlong(f);
+    const int ef = (int)(b >> 52) & 0x7ff;
+    long long m = b & (FX_ONE - 1);
+    if (ef) m |= FX_ONE;
+    e = max(ef, 1);
+    m <<= 3;
+    return b < 0 ? -m : m;
+}
+
+// t in counts of 2^-52, to nearest, without the FP64 pipe for |t| < 1024;
+// saturates, NaN gives 0
+__device__ __forceinline__ long long fx_count(double t)
+{
+    const long long b = __double_as_longlong(t);
+    const int s = 1032 - ((int)(b >> 52) & 0x7ff);   // t 2^53 = (mantissa 2^10) 2^-s
+    if (s < 0) return __double2ll_rn(t * 4503599627370496.0);
+    const unsigned long long m = (unsigned long long)((b & (FX_ONE - 1)) | FX_ONE) << 10;
+    const long long r = (long long)(((m >> min(s, 63)) + 1) >> 1);
+    return b < 0 ? -r : r;
+}
+
+// an integer as FP64, to nearest, without the FP64 pipe
+__device__ __forceinline__ double fx_double(long long v)
+{
+    const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    if (a == 0) return 0.0;
+    const int z = __clzll((long long)a);
+    const unsigned long long t = a << z;                       // top bit set
+    // exponent field of the top bit, less the bit itself; the rounding carry
+    // runs into the exponent as it should
+    unsigned long long r = ((unsigned long long)(1085 - z) << 52) + ((t >> 11) + ((t >> 10) & 1ull));
+    if (v < 0) r |= 0x8000000000000000ull;
+    return __longlong_as_double((long long)r);
+}
+
+// d 2^k for a normal result (d = 0 stays 0)
+__device__ __forceinline__ double fx_scale(double d, int k)
+{
+    const long long b = __double_as_longlong(d);
+    return __longlong_as_double(b + ((b & 0x7fffffffffffffffll) ? (long long)k << 52 : 0ll));
+}
+
+}  // namespace avl

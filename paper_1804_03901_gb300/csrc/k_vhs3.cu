@@ -13,13 +13,9 @@
 //   gather  one thread per x column adds the 16 cloud-in-cell weights (Eq. 4
 //           numerator alpha f and denominator alpha) of the markers of its
 //           two dual cells into registers: rows j, j+1 of v_x times the
-//           pencil's four (v_y, v_z) cells -- no atomics.  FP64: the columns
-//           are counting-sorted by their pair counts, their sums kept in
-//           shared-memory row planes, and each of 128 lanes walks a light
-//           and a heavy column in one loop, so that a warp's lanes do nearly
-//           equal work (an FP64 warp instruction costs its SM sub-partition
-//           the same whatever its active lanes); the weights of a marker's
-//           (v_y, v_z) cells are stored beside it
+//           pencil's four (v_y, v_z) cells -- no atomics.  FP64 (k_pd3x):
+//           the sums in 64-bit integers (fixed.cuh), since an FP64 warp
+//           instruction costs its SM sub-partition 64 clocks
 //   flush   a finished v_x row is added into the global accumulators; each
 //           cell receives the sums of the four pencils that reach it
 // Markers whose key moved since the last re-sort deposit their 16
@@ -41,6 +37,7 @@
 
 #include "avl_internal.cuh"
 #include "common.cuh"
+#include "fixed.cuh"
 #include "ptx.cuh"
 
 namespace avl {
@@ -56,16 +53,7 @@ __device__ __forceinline__ Pos3<T> pos3_from_cells(double xi, int nx)
     return posm_from_cells<T>(xi, nx);
 }
 
-template <typename T>
-struct Cfg3;
-template <>
-struct Cfg3<float> {
-    static constexpr int MPT = 2;   // markers per thread and chunk
-};
-template <>
-struct Cfg3<double> {
-    static constexpr int MPT = 2;
-};
+constexpr int MPT3 = 2;   // markers per thread and chunk
 
 __device__ __forceinline__ int species_of_pen(const StepArgs* A, int g)
 {
@@ -98,21 +86,28 @@ __device__ __forceinline__ int dual3(float v, float a, float b, int n, float& w)
     return (int)fl;
 }
 // FP64: a and b come scaled by 2^52 (dual_coef), so that t 2^52 rounds to a
-// 64-bit count of 2^-52 rows in one saturating conversion (NaN gives 0);
-// the row is its high bits and the weight its low 52 bits, read as the
-// mantissa of 1 + w: the FP64 pipe (the kernel's limit) sees three
-// operations, the range test is in integers
-__device__ __forceinline__ int dual3(double v, double a52, double b52, int n, double& w)
+// 64-bit count of 2^-52 rows in one saturating conversion (NaN gives 0); the
+// row is its high bits and the weight its low 52 bits
+__device__ __forceinline__ int dual3(double v, double a52, double b52, int n, long long& w)
 {
     const long long t = __double2ll_rn(__fma_rn(v, a52, b52));
     const int fl = (int)(t >> 52);
     if (fl < -2 || fl >= n) {
-        w = 0.0;
+        w = 0;
         return fl < 0 ? -2 : n;
     }
-    w = __longlong_as_double(0x3FF0000000000000ll | (t & 0x000FFFFFFFFFFFFFll)) - 1.0;
+    w = t & (FX_ONE - 1);
     return fl;
 }
+// type of dual3's weight: a float, or a count of 2^-52
+template <typename T>
+struct DualW {
+    using type = float;
+};
+template <>
+struct DualW<double> {
+    using type = long long;
+};
 
 // coefficients a, b of dual3 for dimension d of a species, in storage
 // precision (FP64: times 2^52)
@@ -199,56 +194,37 @@ __device__ void block_exscan(const int* in, int* out, int n, int items, int* wsu
 // memory by bulk copies (TMA) while the current one is processed.
 template <typename T>
 struct Stage3 {
-    static constexpr int NB = P3_THREADS * Cfg3<T>::MPT;   // markers per chunk
+    static constexpr int NB = P3_THREADS * MPT3;              // markers per chunk
     // staged fields: FP32 cell, offset, v_x, v_y, v_z, f; FP64 x, v_x, f (the
-    // weights of the (v_y, v_z) cells are stored beside the marker)
+    // (v_y, v_z) weights are stored beside the marker)
     static constexpr int NF = sizeof(T) == 4 ? 6 : 3;
     static constexpr int FVX = sizeof(T) == 4 ? 2 : 1;       // staged field of v_x
     static constexpr int FF = NF - 1;                         // staged field of f
-    // the balanced gather (column accumulators in shared-memory row planes,
-    // columns sorted by their pair counts): the FP64 form, whose instructions
-    // cost an SM sub-partition the same whatever their active lanes
-    static constexpr bool BAL = sizeof(T) == 8;
     static constexpr int AL = 16 / (int)sizeof(T);           // markers per 16 bytes
     static constexpr int SLEN = NB + 2 * AL;                 // staged entries per field
 };
 
-// FP64 gather (see k_pd3): count buckets of the columns' pair counts; the
-// gather's column blocks are laid out for eight warps
-constexpr int GBK = 64;
-// FP64: the short remainder (fewer markers) of a segment just over NB
-// markers skips the x sort and the gather: its markers deposit by global
-// reductions like the markers off their row, which saves the phases of the
-// sort (scan, scatter, column order) and their barriers for a handful of
-// markers (in FP32 the gather of a few markers costs less than their global
-// reductions)
-constexpr int P3_TAIL = 96;
-constexpr int GL = 128;   // gather lanes: one warp per SM sub-partition
-static_assert(P3_THREADS >= GL && GL % 32 == 0, "k_pd3's FP64 gather needs GL threads");
-
-// FP64: the two row planes of the column accumulators, the column order and
-// the count buckets, after the integer arrays (16-byte aligned)
-template <typename T>
-static size_t pd3_acc_offset(int nx, int nkey)
-{
-    using S = Stage3<T>;
-    size_t b = 2 * (size_t)S::NF * S::SLEN * sizeof(T);      // two staging buffers
-    b += sizeof(T) * (7 * (size_t)S::NB + nx);                 // sorted payload, E
-    b += 4 * (2 * (size_t)nx + 1) + 4 * ((size_t)nkey + 2) + 64;   // histogram, bin starts, segment row
-    return (b + 15) / 16 * 16;
-}
-
-template <typename T>
-static size_t pd3_bytes(int nx, int nkey)
-{
-    size_t b = pd3_acc_offset<T>(nx, nkey);
-    if (Stage3<T>::BAL) b += 2 * 8 * (size_t)nx * sizeof(T) + 4 * (size_t)nx + 8 * (size_t)GBK + 16;
-    return (b + 15) / 16 * 16;
-}
+// FP64 (k_pd3x), markers per chunk: more than a segment of two markers per
+// cell at nx = 256 (512, give or take its square root), so that few segments
+// take a second chunk, and two CTAs per SM with the shared memory it needs
+// (97 KB).  64^3 bump-on-tail: 8.29 ms with 640 or 576, 8.40 with 544.
+constexpr int NB3X = 640;
+constexpr int MPT3X = (NB3X + P3_THREADS - 1) / P3_THREADS;
 
 size_t pd3_smem_bytes(int nx, int nkey, int prec)
 {
-    return prec == AVL_FP32 ? pd3_bytes<float>(nx, nkey) : pd3_bytes<double>(nx, nkey);
+    size_t b;
+    if (prec == AVL_FP32) {
+        using S = Stage3<float>;
+        b = 2 * (size_t)S::NF * S::SLEN * 4;                   // two staging buffers
+        b += 4 * (7 * (size_t)S::NB + nx);                     // sorted payload, E
+    } else {
+        b = 5 * (NB3X + 4) * 8 + 96 * NB3X + 32;                  // staging (w_y, w_z, X, v_x, f), sorted payload
+        b += 16 * (size_t)nx;                                  // kick
+        b += 12 * (size_t)nx + 8 * (size_t)P3_THREADS;         // exponents, bins beyond nx
+    }
+    b += 4 * (2 * (size_t)nx + 1) + 4 * ((size_t)nkey + 2) + 64;   // histogram, bin starts, segment row
+    return (b + 15) / 16 * 16;
 }
 
 // largest key count (nv[0] + 1) over the species of a context
@@ -271,28 +247,34 @@ __device__ __forceinline__ void plane_weights(T wy, T wz, T (&q)[4])
     q[3] = wy * wz;
 }
 
-// FP64: the weights of a marker's four (v_y, v_z) cells, stored beside the
-// marker (they change only when a magnetic field turns v): the plane weights
-// of its dual cells, or 0 when its footprint misses the grid in v_y or v_z
-// (such a marker sits in a clamped pencil and deposits nothing)
-template <typename T>
-__device__ __forceinline__ void marker_planes(const VCoef<T>& vc, T vy, T vz, T (&wq)[4])
+// FP64: the (v_y, v_z) weights of a marker as counts of 2^-52, stored beside
+// it (they change only when a magnetic field turns v); -1 when its footprint
+// misses the grid in v_y or v_z (such a marker sits in a clamped pencil and
+// deposits nothing)
+__device__ __forceinline__ longlong2 marker_wyz(const VCoef<double>& vc, double vy, double vz)
 {
-    T wy, wz;
+    long long wy, wz;
     const int jy = dual3(vy, vc.a[1], vc.b[1], vc.n[1], wy);
     const int jz = dual3(vz, vc.a[2], vc.b[2], vc.n[2], wz);
-    if (jy < -1 || jy >= vc.n[1] || jz < -1 || jz >= vc.n[2]) {
-        wq[0] = wq[1] = wq[2] = wq[3] = (T)0;
-        return;
-    }
-    plane_weights(wy, wz, wq);
+    if (jy < -1 || jy >= vc.n[1] || jz < -1 || jz >= vc.n[2]) return make_longlong2(-1, -1);
+    return make_longlong2(wy, wz);
 }
 
-__device__ __forceinline__ void store_planes(void* mwq, long long k, const double (&wq)[4])
+// FP64: the weights of the pencil's four (v_y, v_z) cells in units of 2^-56
+// from the marker's (v_y, v_z) weights: one product, the others by
+// difference (none negative, sum exactly one)
+__device__ __forceinline__ void plane_weights(longlong2 w, long long (&q)[4])
 {
-    double2* p = reinterpret_cast<double2*>(mwq) + 2 * k;
-    p[0] = make_double2(wq[0], wq[1]);
-    p[1] = make_double2(wq[2], wq[3]);
+    if (w.x < 0) {
+        q[0] = q[1] = q[2] = q[3] = 0;
+        return;
+    }
+    const long long y = w.x << 4, z = w.y << 4;
+    const long long yz = (long long)((__umul64hi((unsigned long long)w.x << 8, (unsigned long long)w.y << 9) + 1) >> 1);
+    q[0] = (FX_ONE << 4) - y - z + yz;
+    q[1] = y - yz;
+    q[2] = z - yz;
+    q[3] = yz;
 }
 
 // the pencil's four (v_y, v_z) planes: first grid offset of each (row 0,
@@ -306,32 +288,22 @@ struct Planes {
 // cloud-in-cell contributions apart from the gather, straight into the
 // global accumulator.  This is one of them: corner bits x (bit 0), v_x row
 // (bit 1), (v_y, v_z) plane (bits 2-3).
-template <typename T>
-__device__ __forceinline__ void deposit_corner_q(T* gacc, int cells, const Planes& pl, int nx, int nvx, int bin, T u,
-                                                 int j, T w, T wqv, T f, int corner)
+__device__ __forceinline__ void deposit_corner(float* gacc, int cells, const Planes& pl, int nx, int nvx, int bin,
+                                               float u, int j, float w, float wy, float wz, float f, int corner)
 {
     const int cx = corner & 1, cv = (corner >> 1) & 1, q = corner >> 2;
     const bool okq = q == 0 ? pl.ok[0] : q == 1 ? pl.ok[1] : q == 2 ? pl.ok[2] : pl.ok[3];
     const int row = j + cv;
     if (!okq || row < 0 || row >= nvx) return;
+    const float ay = (q & 1) ? wy : 1.f - wy, az = (q & 2) ? wz : 1.f - wz;
     const int x = cx ? (bin + 1 == nx ? 0 : bin + 1) : bin;
-    const T ax = cx ? u : (T)1 - u;
-    const T a = ax * (cv ? w : (T)1 - w) * wqv;
-    if (a == (T)0) return;
+    const float ax = cx ? u : 1.f - u;
+    const float a = ax * (cv ? w : 1.f - w) * (ay * az);
+    if (a == 0.f) return;
     const int base = q == 0 ? pl.base[0] : q == 1 ? pl.base[1] : q == 2 ? pl.base[2] : pl.base[3];
     const int o = base + row * nx + x;
     atomicAdd(gacc + o, a * f);
     atomicAdd(gacc + cells + o, a);
-}
-
-// FP32: the plane weight from the marker's (v_y, v_z) cell weights
-template <typename T>
-__device__ __forceinline__ void deposit_corner(T* gacc, int cells, const Planes& pl, int nx, int nvx, int bin, T u,
-                                               int j, T w, T wy, T wz, T f, int corner)
-{
-    const int q = corner >> 2;
-    const T ay = (q & 1) ? wy : (T)1 - wy, az = (q & 2) ? wz : (T)1 - wz;
-    deposit_corner_q<T>(gacc, cells, pl, nx, nvx, bin, u, j, w, ay * az, f, corner);
 }
 
 // exclusive scan of hist[0, nx) into start[0, nx], start[nx] = total; each
@@ -376,13 +348,13 @@ __device__ __forceinline__ void chunk_scan(int* hist, int* start, int nx, int* w
 // PUSH (mode 1) is a template parameter so that the deposit-only instances
 // keep their own register budget (FP32, one column per thread: three CTAs
 // per SM with the push, four without).
-template <typename T, int CPT, bool PUSH>
-__global__ void __launch_bounds__(P3_THREADS, sizeof(T) == 4 ? (CPT == 1 ? (PUSH ? 3 : 4) : (CPT == 2 ? 2 : 1))
-                                                             : (CPT == 1 ? 2 : 1))
+template <int CPT, bool PUSH>
+__global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? (PUSH ? 3 : 4) : (CPT == 2 ? 2 : 1))
     k_pd3(const StepArgs* __restrict__ A, int mode)
 {
+    using T = float;
     using S = Stage3<T>;
-    constexpr int MPT = Cfg3<T>::MPT;
+    constexpr int MPT = MPT3;
     constexpr int NB = S::NB, NF = S::NF, AL = S::AL, SLEN = S::SLEN;
     constexpr int FVX = S::FVX, FF = S::FF;   // staged fields of v_x and f (FP32: v_y, v_z between)
     extern __shared__ __align__(16) unsigned char smem[];
@@ -415,15 +387,6 @@ __global__ void __launch_bounds__(P3_THREADS, sizeof(T) == 4 ? (CPT == 1 ? (PUSH
     int* hist = reinterpret_cast<int*>(Es + nx);
     int* start = hist + nx;
     int* segs = start + nx + 1;
-    // balanced gather (FP64): column accumulators of rows jseg, jseg + 1 in
-    // two planes of 8 x nx (entry e of column x: plane[e * nx + x]), the
-    // columns in order of their pair counts, the count buckets and their
-    // first positions
-    const size_t acc_off = (((size_t)(reinterpret_cast<unsigned char*>(segs + nkey + 2) - smem)) + 15) / 16 * 16;
-    T* RA = reinterpret_cast<T*>(smem + acc_off);
-    int* ordc = reinterpret_cast<int*>(RA + 2 * 8 * nx);
-    int* gbk = ordc + nx;
-    int* gbase = gbk + GBK;
 
     if (threadIdx.x == 0) {
         mbar_init(&bar[0], 1);
@@ -433,28 +396,18 @@ __global__ void __launch_bounds__(P3_THREADS, sizeof(T) == 4 ? (CPT == 1 ? (PUSH
         far_s = 0;
         flag_s = 0;
         nmv_s = 0;
-        if constexpr (sizeof(T) == 4) {
-            src_s[0] = sp.mx[cb];
-            src_s[1] = sp.moff[cb];
-        } else {
-            src_s[0] = sp.mx[cb];
-        }
+        src_s[0] = sp.mx[cb];
+        src_s[1] = sp.moff[cb];
         src_s[FVX] = sp.mv[cb][0];
-        if constexpr (sizeof(T) == 4) {
-            src_s[FVX + 1] = sp.mv[cb][1];
-            src_s[FVX + 2] = sp.mv[cb][2];
-        }
+        src_s[FVX + 1] = sp.mv[cb][1];
+        src_s[FVX + 2] = sp.mv[cb][2];
         src_s[FF] = sp.mf[cb];
     }
     for (int i = threadIdx.x; i < nx; i += P3_THREADS) {
         hist[i] = 0;
-        if (push) Es[i] = sizeof(T) == 4 ? (T)A->fd.E32[i] : (T)A->fd.E64[i];
+        if (push) Es[i] = A->fd.E32[i];
     }
     for (int i = threadIdx.x; i <= nkey; i += P3_THREADS) segs[i] = segg[i];
-    if constexpr (S::BAL) {
-        for (int i = threadIdx.x; i < 2 * 8 * nx; i += P3_THREADS) RA[i] = 0.0;
-        for (int i = threadIdx.x; i < GBK; i += P3_THREADS) gbk[i] = 0;
-    }
     __syncthreads();
 
     // bulk copy of the chunk [b, b + cnt) of every staged field into buffer bf
@@ -486,7 +439,6 @@ __global__ void __launch_bounds__(P3_THREADS, sizeof(T) == 4 ? (CPT == 1 ? (PUSH
     VCoef<T> vc;
     vc.init(sp);
     const T qm_dt = (T)sp.qm_dt, dt_dx = (T)sp.dt_dx;
-    const double dt_dx52 = sp.dt_dx * PosX::ONE;   // FP64: dt / dx in 2^-52 cells
     Planes pl;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -505,35 +457,18 @@ __global__ void __launch_bounds__(P3_THREADS, sizeof(T) == 4 ? (CPT == 1 ? (PUSH
     unsigned long long nmov = 0, nfar = 0;
     int buf = 0;
     unsigned ph0 = 0, ph1 = 0;
-    int rp = 0;   // FP64: plane of row jseg (the other holds row jseg + 1)
 
     for (int k = 0; k < nkey; ++k) {
         const int jseg = k - 1;
         const int send = segs[k + 1];
         for (int b0 = segs[k]; b0 < send; b0 += NB) {
             const int cnt = min(NB, send - b0);
-            const bool tail = S::BAL && b0 > segs[k] && cnt < P3_TAIL;   // FP64: the remainder of a segment over NB
             // stage the next chunk into the other buffer (free since the end of
             // the previous chunk)
             if (threadIdx.x == 0) {
                 int nk = k, nb = b0 + NB;
                 if (nb >= send) nk = first_from(k + 1, nb);
                 if (nk < nkey) issue(buf ^ 1, nb, min(NB, segs[nk + 1] - nb));
-            }
-            // FP64: the stored (v_y, v_z) cell weights of this chunk's markers,
-            // loaded while its staged fields are in flight
-            double2 qlo[MPT], qhi[MPT];
-            if constexpr (sizeof(T) == 8) {
-                const double2* wqg = reinterpret_cast<const double2*>(sp.mwq[cb]);
-#pragma unroll
-                for (int m = 0; m < MPT; ++m) {
-                    const int i = m * P3_THREADS + threadIdx.x;
-                    qlo[m] = qhi[m] = make_double2(0.0, 0.0);
-                    if (i < cnt) {
-                        qlo[m] = wqg[2 * (long long)(b0 + i)];
-                        qhi[m] = wqg[2 * (long long)(b0 + i) + 1];
-                    }
-                }
             }
             const unsigned ph = buf ? ph1 : ph0;
             if (!mbar_wait_or_drain(&bar[buf], ph, wait_first, WAIT_LIMIT)) flag_s = 1;
@@ -552,12 +487,8 @@ __global__ void __launch_bounds__(P3_THREADS, sizeof(T) == 4 ? (CPT == 1 ? (PUSH
                 const int si = o0 + i;
                 const int idx = b0 + i;
                 Pos3<T> pos;
-                if constexpr (sizeof(T) == 4) {
-                    pos.c = reinterpret_cast<const int*>(st)[si];
-                    pos.o = st[SLEN + si];
-                } else {
-                    pos.X = reinterpret_cast<const long long*>(st)[si];
-                }
+                pos.c = reinterpret_cast<const int*>(st)[si];
+                pos.o = st[SLEN + si];
                 T vx = st[FVX * SLEN + si];
                 if (push) {
                     int i0;
@@ -565,38 +496,22 @@ __global__ void __launch_bounds__(P3_THREADS, sizeof(T) == 4 ? (CPT == 1 ? (PUSH
                     pos.cic(i0, wx);
                     int ia, ib;
                     wrap_pair(i0, nx, ia, ib);
-                    if constexpr (sizeof(T) == 8) {
-                        // FP64 (the FP64 pipe limits this form): E_a + w (E_b - E_a)
-                        // fused, one FP64 operation fewer than the plain form;
-                        // the displacement in 2^-52 cells (dt_dx52 = dt / dx 2^52)
-                        const T Ea = Es[ia];
-                        vx = fma(qm_dt, fma(wx, Es[ib] - Ea, Ea), vx);
-                        pos.drift_scaled(vx * dt_dx52, nx);
-                    } else {
-                        const T El = ((T)1 - wx) * Es[ia] + wx * Es[ib];
-                        vx = vx + qm_dt * El;
-                        pos.drift(vx * dt_dx, nx);
-                    }
-                    if constexpr (sizeof(T) == 4) {
-                        reinterpret_cast<int*>(gx)[idx] = pos.c;
-                        goff[idx] = pos.o;
-                    } else {
-                        reinterpret_cast<long long*>(gx)[idx] = pos.X;
-                    }
+                    const T El = ((T)1 - wx) * Es[ia] + wx * Es[ib];
+                    vx = vx + qm_dt * El;
+                    pos.drift(vx * dt_dx, nx);
+                    reinterpret_cast<int*>(gx)[idx] = pos.c;
+                    goff[idx] = pos.o;
                     gvx[idx] = vx;
                 }
                 const T f = st[FF * SLEN + si];
                 T wy = (T)0, wz = (T)0, w;
-                // FP32: the (v_y, v_z) dual cells, checked against the pencil;
-                // FP64: the stored cell weights (0 for a footprint off the grid)
-                if constexpr (sizeof(T) == 4) {
-                    const int jy = dual3(st[(FVX + 1) * SLEN + si], vc.a[1], vc.b[1], vc.n[1], wy);
-                    const int jz = dual3(st[(FVX + 2) * SLEN + si], vc.a[2], vc.b[2], vc.n[2], wz);
-                    if (jy != pjy || jz != pjz) {
-                        // outside the pencil only when the footprint misses the grid
-                        if (jy >= -1 && jy < nvy && jz >= -1 && jz < nvz) flag_s |= 2;
-                        continue;
-                    }
+                // the (v_y, v_z) dual cells, checked against the pencil
+                const int jy = dual3(st[(FVX + 1) * SLEN + si], vc.a[1], vc.b[1], vc.n[1], wy);
+                const int jz = dual3(st[(FVX + 2) * SLEN + si], vc.a[2], vc.b[2], vc.n[2], wz);
+                if (jy != pjy || jz != pjz) {
+                    // outside the pencil only when the footprint misses the grid
+                    if (jy >= -1 && jy < nvy && jz >= -1 && jz < nvz) flag_s |= 2;
+                    continue;
                 }
                 const int jx = dual3(vx, vc.a[0], vc.b[0], nvx, w);
                 if (jx < -1 || jx >= nvx) continue;
@@ -606,26 +521,20 @@ __global__ void __launch_bounds__(P3_THREADS, sizeof(T) == 4 ? (CPT == 1 ? (PUSH
                 int bin = i0 < 0 ? i0 + nx : i0;
                 bin = min(max(bin, 0), nx - 1);
                 const int d = jx - jseg;
-                if (d == 0 && !tail) {
+                if (d == 0) {
                     prank[m] = atomicAdd(&hist[bin], 1);
                 } else {
-                    // off its segment's row (or in a short chunk): parked at the
-                    // tail of the payload arrays (the stays fill them from the
-                    // front) and deposited by the whole block after the sort
-                    if (d != 0) {
-                        ++nmov;
-                        if (d > 1 || d < -1) ++nfar;
-                    }
+                    // off its segment's row: parked at the tail of the payload
+                    // arrays (the stays fill them from the front) and
+                    // deposited by the whole block after the sort
+                    ++nmov;
+                    if (d > 1 || d < -1) ++nfar;
                     const int o = NB - 1 - atomicAdd(&nmv_s, 1);
                     pay[0 * NB + o] = u;
                     pay[1 * NB + o] = w;
                     pay[2 * NB + o] = f;
-                    if constexpr (sizeof(T) == 4) {
-                        pay[3 * NB + o] = wy;
-                        pay[4 * NB + o] = wz;
-                    } else {
-                        pay[3 * NB + o] = (T)idx;   // FP64: its stored cell weights are read by index
-                    }
+                    pay[3 * NB + o] = wy;
+                    pay[4 * NB + o] = wz;
                     pay[5 * NB + o] = (T)bin;
                     pay[6 * NB + o] = (T)jx;
                 }
@@ -645,26 +554,10 @@ __global__ void __launch_bounds__(P3_THREADS, sizeof(T) == 4 ? (CPT == 1 ? (PUSH
                 for (int t = threadIdx.x; t < nmv * 16; t += P3_THREADS) {
                     const int o = NB - 1 - (t >> 4);
                     const int jx = (int)pay[6 * NB + o];
-                    if constexpr (sizeof(T) == 4) {
-                        deposit_corner<T>(gacc, cells, pl, nx, nvx, (int)pay[5 * NB + o], pay[0 * NB + o], jx,
-                                          pay[1 * NB + o], pay[3 * NB + o], pay[4 * NB + o], pay[2 * NB + o],
-                                          t & 15);
-                    } else {
-                        const long long mi = (long long)pay[3 * NB + o];
-                        const T wqv = reinterpret_cast<const double*>(sp.mwq[cb])[4 * mi + ((t & 15) >> 2)];
-                        deposit_corner_q<T>(gacc, cells, pl, nx, nvx, (int)pay[5 * NB + o], pay[0 * NB + o], jx,
-                                            pay[1 * NB + o], wqv, pay[2 * NB + o], t & 15);
-                    }
+                    deposit_corner(gacc, cells, pl, nx, nvx, (int)pay[5 * NB + o], pay[0 * NB + o], jx,
+                                      pay[1 * NB + o], pay[3 * NB + o], pay[4 * NB + o], pay[2 * NB + o], t & 15);
                 }
             };
-            if (tail) {
-                __syncthreads();   // every thread has read nmv_s
-                if (threadIdx.x == 0) nmv_s = 0;
-                deposit_parked();
-                __syncthreads();
-                buf ^= 1;
-                continue;
-            }
             chunk_scan<CPT>(hist, start, nx, wsum);   // every thread has read nmv_s by its barriers
             if (threadIdx.x == 0) nmv_s = 0;
             // stays into x-sorted order
@@ -673,132 +566,18 @@ __global__ void __launch_bounds__(P3_THREADS, sizeof(T) == 4 ? (CPT == 1 ? (PUSH
                 if (prank[m] < 0) continue;
                 const int o = start[pbin[m]] + prank[m];
                 T wq[4];
-                if constexpr (sizeof(T) == 4) {
-                    plane_weights(py[m], pz[m], wq);
-                } else {
-                    wq[0] = qlo[m].x;
-                    wq[1] = qlo[m].y;
-                    wq[2] = qhi[m].x;
-                    wq[3] = qhi[m].y;
-                }
+                plane_weights(py[m], pz[m], wq);
                 pay[0 * NB + o] = pu[m];
                 pay[1 * NB + o] = pw[m];
                 pay[2 * NB + o] = pf[m];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) pay[(3 + q) * NB + o] = wq[q];
             }
-            // FP64: pairs (marker, column) of each column = the markers of its
-            // two dual cells; the columns are counting-sorted by that count
-            // so that a warp's lanes loop over nearly equal counts (an FP64
-            // warp instruction costs its sub-partition the same whatever the
-            // number of active lanes)
-            int gb[CPT], grank[CPT];
-            if constexpr (S::BAL) {
-#pragma unroll
-                for (int c = 0; c < CPT; ++c) {
-                    const int x = threadIdx.x + c * P3_THREADS;
-                    gb[c] = -1;
-                    if (x >= nx) continue;
-                    const int xm = x == 0 ? nx - 1 : x - 1;
-                    const int cnt = (start[xm + 1] - start[xm]) + (start[x + 1] - start[x]);
-                    gb[c] = min(cnt, GBK - 1);
-                    grank[c] = atomicAdd(&gbk[gb[c]], 1);
-                }
-            }
             __syncthreads();
-            if constexpr (S::BAL) {
-                if (threadIdx.x < 32) {   // exclusive scan of the buckets (two per lane)
-                    const int lane = threadIdx.x;
-                    const int a0 = gbk[2 * lane], a1 = gbk[2 * lane + 1];
-                    int incl = a0 + a1;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-                        if (lane >= o) incl += y;
-                    }
-                    gbase[2 * lane] = incl - a0 - a1;
-                    gbase[2 * lane + 1] = incl - a1;
-                }
-            }
             deposit_parked();
             // gather: column x takes weight u from the markers of dual cell
             // x - 1 and 1 - u from those of dual cell x, which follow them in
             // the sorted order (one loop; two at the periodic seam)
-            if constexpr (S::BAL) {
-                __syncthreads();
-#pragma unroll
-                for (int c = 0; c < CPT; ++c)
-                    if (gb[c] >= 0) ordc[gbase[gb[c]] + grank[c]] = threadIdx.x + c * P3_THREADS;
-                __syncthreads();
-                for (int i = threadIdx.x; i < GBK; i += P3_THREADS) gbk[i] = 0;
-                T* P0 = RA + (size_t)rp * 8 * nx;
-                T* P1 = RA + (size_t)(rp ^ 1) * 8 * nx;
-                // gather lanes: the first GL threads (one warp per SM
-                // sub-partition) each take the sorted columns l and 2K - 1 - l
-                // (then 2K + l, 4K - 1 - l, ...), a light and a heavy one, and
-                // walk their pairs in one loop, so that the lanes of a warp do
-                // nearly equal work; a lane's accumulators go back to the row
-                // planes when its column changes.  Each column is summed in
-                // pair order (dual cell x - 1, then dual cell x).
-                const int K = min(GL, (nx + 1) >> 1);
-                const int l = threadIdx.x;
-                if (l < K) {
-                    int r = 0, x = -1, lo = 0, nup = 0, blo = 0, n = 0, kr = 0;
-                    T A0[8], A1[8];
-                    for (;;) {
-                        if (kr == n) {
-                            if (x >= 0) {
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) {
-                                    P0[e * nx + x] = A0[e];
-                                    P1[e * nx + x] = A1[e];
-                                }
-                            }
-                            x = -1;
-                            while (r * K < nx) {
-                                const int pos = r * K + ((r & 1) ? K - 1 - l : l);
-                                ++r;
-                                if (pos >= nx) continue;
-                                const int cx = ordc[pos];
-                                const int cxm = cx == 0 ? nx - 1 : cx - 1;
-                                const int a0 = start[cxm], a1 = start[cxm + 1];
-                                const int b0 = start[cx], b1 = start[cx + 1];
-                                if (a1 - a0 + b1 - b0 == 0) continue;
-                                x = cx;
-                                lo = a0;
-                                nup = a1 - a0;
-                                blo = b0;
-                                n = nup + b1 - b0;
-                                kr = 0;
-                                break;
-                            }
-                            if (x < 0) break;
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) {
-                                A0[e] = P0[e * nx + x];
-                                A1[e] = P1[e * nx + x];
-                            }
-                        }
-                        const bool upper = kr < nup;
-                        const int i = upper ? lo + kr : blo + (kr - nup);
-                        ++kr;
-                        const T u = pay[i];
-                        const T ax = upper ? u : (T)1 - u;
-                        const T a1 = ax * pay[NB + i];
-                        const T a0 = ax - a1;
-                        const T f = pay[2 * NB + i];
-                        const T f0 = a0 * f, f1 = a1 * f;
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const T wqv = pay[(3 + q) * NB + i];
-                            A0[2 * q] += f0 * wqv;
-                            A0[2 * q + 1] += a0 * wqv;
-                            A1[2 * q] += f1 * wqv;
-                            A1[2 * q + 1] += a1 * wqv;
-                        }
-                    }
-                }
-            } else
 #pragma unroll
             for (int c = 0; c < CPT; ++c) {
                 const int x = threadIdx.x + c * P3_THREADS;
@@ -831,31 +610,6 @@ __global__ void __launch_bounds__(P3_THREADS, sizeof(T) == 4 ? (CPT == 1 ? (PUSH
             __syncthreads();
             buf ^= 1;
         }
-        if constexpr (S::BAL) {
-            // row jseg is complete (the next segment reaches rows jseg + 1 and
-            // jseg + 2): its plane into the global accumulator and cleared,
-            // then the planes swap
-            T* P0 = RA + (size_t)rp * 8 * nx;
-#pragma unroll
-            for (int c = 0; c < CPT; ++c) {
-                const int x = threadIdx.x + c * P3_THREADS;
-                if (x >= nx) continue;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const T vn = P0[(2 * q) * nx + x], vd = P0[(2 * q + 1) * nx + x];
-                    if (jseg >= 0 && jseg < nvx && pl.ok[q] && __double_as_longlong(vd) != 0) {
-                        const int o = pl.base[q] + jseg * nx + x;
-                        atomicAdd(gacc + o, vn);
-                        atomicAdd(gacc + cells + o, vd);
-                    }
-                    P0[(2 * q) * nx + x] = (T)0;
-                    P0[(2 * q + 1) * nx + x] = (T)0;
-                }
-            }
-            rp ^= 1;
-            __syncthreads();
-            continue;
-        }
         // row jseg - 1 is complete (no later segment reaches it): registers into
         // the global accumulator; then rotate the rows
         const int row = jseg - 1;
@@ -886,7 +640,7 @@ __global__ void __launch_bounds__(P3_THREADS, sizeof(T) == 4 ? (CPT == 1 ? (PUSH
         __syncthreads();
     }
     // the last row (nvx - 1) after the last segment
-    if constexpr (!S::BAL) {
+    {
         const int row = nvx - 1;
 #pragma unroll
         for (int c = 0; c < CPT; ++c) {
@@ -913,6 +667,452 @@ __global__ void __launch_bounds__(P3_THREADS, sizeof(T) == 4 ? (CPT == 1 ? (PUSH
         if (far_s) atomicAdd(&ctl->far_movers[s], far_s);
         if (flag_s & 2) atomicOr(&ctl->err, ERR_CAPACITY);
         if (flag_s & 1) atomicOr(&ctl->err, ERR_TIMEOUT);
+    }
+}
+
+// FP64 form of the same walk.  The FP64 pipe takes a warp instruction per 64
+// clocks and sub-partition, so only the kick, the drift and the v_x row of a
+// marker and the conversion of the finished sums run there (6.3 operations
+// per marker); every weight and sum is a 64-bit integer (fixed.cuh).  What a
+// marker gives to its two columns is worked out once, by the thread that
+// sorts it into x order; the gather then is three multiply-adds per sum.  One
+// thread per x column keeps the sums of its two v_x rows in registers for the
+// length of a segment, in the gather as h and m (64 registers), between the
+// chunks as whole units (32; two CTAs per SM at 128 registers).
+//
+// Bound by the latency of its phases (16 warps per SM, four barriers per
+// chunk; issue slots 34 % busy, multiply-add pipe 45 %, shared memory 37 %,
+// FP64 pipe 23 %).  134 M markers, 256 x 64^3: 16.95 -> 8.29 ms against the
+// same sums in FP64; measured and left out: balanced columns with the sums in
+// shared memory (10.3 ms, its random payload reads fill the shared-memory
+// pipe), two threads per column (9.5 ms), the push of the next chunk beside
+// the gather (9.5 ms, its second staging buffer and tables cost more
+// instructions than the barriers they save), the conversions in integers
+// (8.6 ms).
+struct FxCol {
+    long long d0[4], v0[4];   // row jseg: weights, weighted values of the four planes
+    long long d1[4], v1[4];   // row jseg + 1
+    int el;                   // the values' unit is 2^(el - 1078)
+    int c0, c1;               // products in the sums of each row
+
+    __device__ __forceinline__ void clear0()
+    {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) d0[q] = v0[q] = 0;
+        c0 = 0;
+    }
+    __device__ __forceinline__ void clear1()
+    {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) d1[q] = v1[q] = 0;
+        c1 = 0;
+    }
+    // row jseg + 1 becomes row jseg; its unit shrinks as far as the sums
+    // allow (they stay below 2^59, which leaves room for FX_PAIRS products)
+    __device__ __forceinline__ void next_row()
+    {
+        int room = el - FX_EMIN;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            d0[q] = d1[q];
+            v0[q] = v1[q];
+            if (c1) room = min(room, __clzll(v0[q] < 0 ? ~v0[q] : v0[q]) - 5);
+        }
+        c0 = c1;
+        clear1();
+        if (room >= 4) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v0[q] <<= min(room, 63);
+            el -= room;
+        }
+    }
+};
+
+__device__ __forceinline__ int4 limbs2(long long a, long long b)
+{
+    const Limbs A = fx_split(a), B = fx_split(b);
+    return make_int4(A.h, A.l, B.h, B.l);
+}
+
+// exclusive scan of hist[0, 256 CPT) into start[0, 256 CPT]: every warp sums
+// the bins in registers (8 CPT per lane) and writes its share, so that the
+// scan takes no barrier of its own
+template <int CPT>
+__device__ __forceinline__ void bin_scan(const int* hist, int* start)
+{
+    constexpr int PER = 8 * CPT;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int v[PER], sum = 0;
+#pragma unroll
+    for (int i = 0; i < PER; i += 4) {
+        const int4 h = reinterpret_cast<const int4*>(hist)[(lane * PER + i) / 4];
+        v[i] = h.x;
+        v[i + 1] = h.y;
+        v[i + 2] = h.z;
+        v[i + 3] = h.w;
+        sum += h.x + h.y + h.z + h.w;
+    }
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if ((lane >> 2) == warp) {   // a warp's share: 32 CPT bins of four lanes
+        int run = incl - sum;
+#pragma unroll
+        for (int i = 0; i < PER; i += 4) {
+            const int4 b = make_int4(run, run + v[i], run + v[i] + v[i + 1], run + v[i] + v[i + 1] + v[i + 2]);
+            reinterpret_cast<int4*>(start)[(lane * PER + i) / 4] = b;
+            run = b.w + v[i + 3];
+        }
+        if (lane == 31) start[P3_THREADS * CPT] = run;
+    }
+}
+
+// finished sums of a cell into the global accumulator, in units of 2^-57 and
+// 2^(el - 1079)
+__device__ __forceinline__ void add_sums(long long d, long long v, int el, double* gacc, int cells, bool ok, int o)
+{
+    if (!ok || d == 0) return;
+    atomicAdd(gacc + o, fx_scale((double)v, el - 1079));
+    atomicAdd(gacc + cells + o, fx_scale((double)d, -57));
+}
+
+template <int CPT, bool PUSH>
+__global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const StepArgs* __restrict__ A, int mode)
+{
+    constexpr int AL = 2, NB = NB3X, SLEN = NB + 2 * AL, NT = P3_THREADS;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint64_t bar;
+    __shared__ unsigned long long mov_s, far_s;
+    __shared__ int flag_s;
+    __shared__ int nmv_s;
+
+    const int g = blockIdx.x;
+    const int s = species_of_pen(A, g);
+    const SpDev& sp = A->sp[s];
+    if (mode != 0 && !sp.mobile) return;
+    Ctl* ctl = A->ctl;
+    const long long wait_first = ctl->wait_limit;
+    const int p = g - sp.pen_base;
+    const int nx = sp.nx, nvx = sp.nv[0], nvy = sp.nv[1], nvz = sp.nv[2], nkey = sp.nkey;
+    const int pjy = p % (nvy + 1) - 1, pjz = p / (nvy + 1) - 1;
+    const int cb = ctl->cur[s];
+    const int cells = sp.nvflat * nx;
+    double* const gacc = reinterpret_cast<double*>(sp.acc[ctl->asel[s]]);
+    const int* segg = sp.seg[cb] + (size_t)p * (nkey + 1);
+    const longlong2* const wyz = sp.mwyz[cb];
+    const double* const gf = reinterpret_cast<const double*>(sp.mf[cb]);
+
+    // shared memory: staging (v_y and v_z weights, X, v_x, f) | payload
+    // (arrays of limb pairs) | kick | hist | start | exponents | segment row
+    longlong2* const st_w = reinterpret_cast<longlong2*>(smem);
+    long long* const st_x = reinterpret_cast<long long*>(st_w + SLEN);
+    double* const st_v = reinterpret_cast<double*>(st_x + SLEN);
+    double* const st_f = st_v + SLEN;
+    int4* pqa = reinterpret_cast<int4*>(st_f + SLEN);             // weights of planes 0 and 1
+    int4* pqb = pqa + NB;                                         //            planes 2 and 3
+    int4* pa = pqb + NB;       // weights of rows jseg and jseg + 1: [0, NB) in the marker's dual cell, [NB, 2 NB) in
+                               // the next
+    int4* pg = pa + 2 * NB + 1;    // the same times the value
+    double2* kick = reinterpret_cast<double2*>(pg + 2 * NB + 1);
+    int* hist = reinterpret_cast<int*>(kick + nx);   // [256 CPT]
+    int* start = hist + NT * CPT;                    // [256 CPT + 1]
+    int* ebin = start + NT * CPT + 1;   // [2][nx] largest exponent field of a dual cell's values, by chunk parity
+    int* elc = ebin + 2 * nx;           // [nx] the columns' exponents (unit of the value sums) before this chunk
+    int* segs = elc + nx;
+
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        fence_mbar_init();
+        mov_s = 0;
+        far_s = 0;
+        flag_s = 0;
+        nmv_s = 0;
+        pa[2 * NB] = pg[2 * NB] = make_int4(0, 0, 0, 0);
+    }
+    for (int i = threadIdx.x; i < nx; i += NT) {
+        ebin[i] = ebin[nx + i] = 0;
+        // kick of a marker between the centres of cells i and i + 1 with
+        // weight w of cell i + 1, as c + (1 + w) d (1 + w: the bits of the
+        // position): E_i + w (E_i+1 - E_i), times (q/m) dt
+        if (PUSH) {
+            const double Ea = A->fd.E64[i], dE = A->fd.E64[i + 1 == nx ? 0 : i + 1] - Ea;
+            kick[i] = make_double2(sp.qm_dt * (Ea - dE), sp.qm_dt * dE);
+        }
+    }
+    for (int i = threadIdx.x; i <= nkey; i += NT) segs[i] = segg[i];
+    for (int i = threadIdx.x; i < NT * CPT; i += NT) hist[i] = 0;
+    __syncthreads();
+
+    double* const gvx = reinterpret_cast<double*>(sp.mv[cb][0]);
+    long long* const gx = reinterpret_cast<long long*>(sp.mx[cb]);
+    // bulk copy of the chunk [b, b + cnt) of every staged field
+    auto issue = [&](int b, int cnt) {
+        const int a0 = b & ~(AL - 1);
+        const int a1 = (b + cnt + AL - 1) & ~(AL - 1);
+        const unsigned bytes = (unsigned)(a1 - a0) * 8u;
+        mbar_arrive_expect_tx(&bar, bytes * 5);
+        bulk_g2s(st_w, wyz + a0, 2 * bytes, &bar);
+        bulk_g2s(st_x, gx + a0, bytes, &bar);
+        bulk_g2s(st_v, gvx + a0, bytes, &bar);
+        bulk_g2s(st_f, gf + a0, bytes, &bar);
+    };
+    // first chunk at or after key k whose segment is not empty
+    auto first_from = [&](int k, int& kb) {
+        for (; k < nkey; ++k)
+            if (segs[k] < segs[k + 1]) break;
+        kb = k < nkey ? segs[k] : 0;
+        return k;
+    };
+    if (threadIdx.x == 0) {
+        int b;
+        const int k0 = first_from(0, b);
+        if (k0 < nkey) issue(b, min(NB, segs[k0 + 1] - b));
+    }
+
+    double av, bv;
+    dual_coef<double>(sp, 0, av, bv);
+    const double dt_dx52 = sp.dt_dx * PosX::ONE;   // dt / dx in 2^-52 cells
+    Planes pl;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int ky = pjy + (q & 1), kz = pjz + (q >> 1);
+        pl.ok[q] = ky >= 0 && ky < nvy && kz >= 0 && kz < nvz;
+        pl.base[q] = pl.ok[q] ? (kz * nvy + ky) * nvx * nx : 0;
+    }
+
+    unsigned nmov = 0, nfar = 0;
+    unsigned ph = 0;   // phase of the staging barrier
+    int par = 0;       // parity of the chunk
+    FxCol col[CPT];
+#pragma unroll
+    for (int c = 0; c < CPT; ++c) {
+        col[c].clear0();
+        col[c].clear1();
+        col[c].el = FX_EMIN;
+    }
+
+    for (int k = 0; k < nkey; ++k) {
+        const int jseg = k - 1;
+        const int send = segs[k + 1];
+        for (int b0 = segs[k]; b0 < send; b0 += NB) {
+            const int cnt = min(NB, send - b0);
+#pragma unroll
+            for (int c = 0; c < CPT; ++c)
+                if (threadIdx.x + c * NT < nx) elc[threadIdx.x + c * NT] = col[c].el;
+            if (!mbar_wait_or_drain(&bar, ph, wait_first, WAIT_LIMIT)) flag_s = 1;
+            ph ^= 1u;
+            const int o0 = b0 & (AL - 1);
+
+            long long mu[MPT3X], mw[MPT3X];
+            int pbin[MPT3X], prank[MPT3X];
+#pragma unroll
+            for (int m = 0; m < MPT3X; ++m) {
+                prank[m] = -1;
+                const int i = m * NT + threadIdx.x;
+                if (i >= cnt) continue;
+                const int si = o0 + i;
+                PosX pos;
+                pos.X = st_x[si];
+                double vx = st_v[si];
+                if (PUSH) {
+                    const long long U = pos.X - (FX_ONE >> 1);
+                    int ia = (int)(U >> 52);   // -1 .. nx - 1
+                    ia = min(max(ia < 0 ? ia + nx : ia, 0), nx - 1);
+                    const double2 kc = kick[ia];
+                    vx += __fma_rn(__longlong_as_double(0x3FF0000000000000ll | (U & (FX_ONE - 1))), kc.y, kc.x);
+                    pos.drift_scaled(vx * dt_dx52, nx);
+                    gx[b0 + i] = pos.X;
+                    gvx[b0 + i] = vx;
+                }
+                if (st_w[si].x < 0) continue;   // footprint off the grid in v_y or v_z
+                long long w;
+                const int jx = dual3(vx, av, bv, nvx, w);
+                if (jx < -1 || jx >= nvx) continue;
+                const long long U = pos.X - (FX_ONE >> 1);
+                int bin = (int)(U >> 52);
+                bin = min(max(bin < 0 ? bin + nx : bin, 0), nx - 1);
+                mu[m] = U & (FX_ONE - 1);
+                mw[m] = w;
+                pbin[m] = bin;
+                const double f = st_f[si];
+                const int d = jx - jseg;
+                if (d == 0) {
+                    prank[m] = atomicAdd(&hist[bin], 1);
+                    atomicMax(&ebin[par * nx + bin], __double2hiint(f) >> 20 & 0x7ff);
+                } else {
+                    // off its segment's row: parked at the tail of the payload
+                    // arrays (the stays fill them from the front) and
+                    // deposited by the whole block after the sort
+                    ++nmov;
+                    if (d > 1 || d < -1) ++nfar;
+                    const int o = NB - 1 - atomicAdd(&nmv_s, 1);
+                    reinterpret_cast<longlong2*>(pa)[o] = st_w[si];
+                    reinterpret_cast<longlong2*>(pqb)[o] = make_longlong2(mu[m], w);
+                    pqa[o] = make_int4(bin, jx, __double2loint(f), __double2hiint(f));
+                }
+            }
+            __syncthreads();
+            const int nmv = nmv_s;
+            bin_scan<CPT>(hist, start);
+            __syncthreads();
+            if (threadIdx.x == 0) nmv_s = 0;
+            // the bins are counted into afresh after the next barrier
+#pragma unroll
+            for (int c = 0; c < CPT; ++c) hist[threadIdx.x + c * NT] = 0;
+            // stays into x-sorted order
+#pragma unroll
+            for (int m = 0; m < MPT3X; ++m) {
+                if (prank[m] < 0) continue;
+                const int bin = pbin[m], o = start[bin] + prank[m], si = o0 + m * NT + threadIdx.x;
+                long long q[4];
+                plane_weights(st_w[si], q);
+                pqa[o] = limbs2(q[0], q[1]);
+                pqb[o] = limbs2(q[2], q[3]);
+                // value in the units of the two columns
+                const int bm = bin == 0 ? nx - 1 : bin - 1, bp = bin + 1 == nx ? 0 : bin + 1;
+                int e;
+                const long long mant = fx_value(st_f[si], e);
+                const int* eb = ebin + par * nx;
+                const int e0 = max(elc[bin], max(eb[bm], eb[bin])), e1 = max(elc[bp], max(eb[bin], eb[bp]));
+                const Limbs f0 = fx_split(mant >> min(e0 - e, 63)), f1 = fx_split(mant >> min(e1 - e, 63));
+                // weights in x and v_x: one product, the others by difference
+                // (none negative)
+                const long long u = mu[m] << 5, w = mw[m] << 5;
+                const long long a11 = fx_mul(fx_split(u), fx_split(mw[m] << 4));
+                const long long a01 = w - a11;
+                const long long a00 = (FX_ONE << 5) - u - a01, a10 = u - a11;
+                const Limbs A00 = fx_split(a00), A01 = fx_split(a01), A10 = fx_split(a10), A11 = fx_split(a11);
+                pa[o] = make_int4(A00.h, A00.l, A01.h, A01.l);
+                pa[NB + o] = make_int4(A10.h, A10.l, A11.h, A11.l);
+                pg[o] = limbs2(fx_mul(A00, f0), fx_mul(A01, f0));
+                pg[NB + o] = limbs2(fx_mul(A10, f1), fx_mul(A11, f1));
+            }
+            __syncthreads();
+            // the staging buffer is free: the next chunk into it
+            if (threadIdx.x == 0) {
+                int nk = k, nb = b0 + NB;
+                if (nb >= send) nk = first_from(k + 1, nb);
+                if (nk < nkey) issue(nb, min(NB, segs[nk + 1] - nb));
+            }
+            // the parked markers: one thread per (marker, corner) into the
+            // global accumulator, so that a chunk's few movers do not hold one
+            // warp behind the others at the chunk's barrier
+            for (int t = threadIdx.x; t < nmv * 16; t += NT) {
+                const int o = NB - 1 - (t >> 4);
+                const int4 id = pqa[o];
+                const longlong2 uw = reinterpret_cast<const longlong2*>(pqb)[o];
+                long long q[4];
+                plane_weights(reinterpret_cast<const longlong2*>(pa)[o], q);
+                const int c = (t & 15) >> 2, row = id.y + ((t >> 1) & 1);
+                const bool ok = (c == 0 ? pl.ok[0] : c == 1 ? pl.ok[1] : c == 2 ? pl.ok[2] : pl.ok[3]) && row >= 0 &&
+                                row < nvx;
+                const int base = c == 0 ? pl.base[0] : c == 1 ? pl.base[1] : c == 2 ? pl.base[2] : pl.base[3];
+                const int x = t & 1 ? (id.x + 1 == nx ? 0 : id.x + 1) : id.x;
+                const long long a = fx_mul(fx_split((t & 1 ? uw.x : FX_ONE - uw.x) << 5),
+                                           fx_split((t & 2 ? uw.y : FX_ONE - uw.y) << 4));
+                const long long al = fx_mul(fx_split(a), fx_split(c == 0 ? q[0] : c == 1 ? q[1] : c == 2 ? q[2] : q[3]));
+                if (!ok || al == 0) continue;
+                const double alpha = fx_scale(fx_double(al), -57);
+                const int at = base + row * nx + x;
+                atomicAdd(gacc + at, alpha * __hiloint2double(id.w, id.z));
+                atomicAdd(gacc + cells + at, alpha);
+            }
+            // gather: column x takes weight u from the markers of dual cell
+            // x - 1 and 1 - u from those of dual cell x
+#pragma unroll
+            for (int c = 0; c < CPT; ++c) {
+                const int x = threadIdx.x + c * NT;
+                if (x >= nx) continue;
+                FxCol& C = col[c];
+                const int xm = x == 0 ? nx - 1 : x - 1;
+                const int lo = start[xm], nup = start[xm + 1] - lo;
+                const int blo = start[x] - nup, n = nup + start[x + 1] - start[x];
+                ebin[(par ^ 1) * nx + x] = 0;   // the next chunk's
+                if (n == 0) continue;
+                const int et = max(C.el, max(ebin[par * nx + xm], ebin[par * nx + x]));
+                const int sh = min(et - C.el, 63);
+                C.el = et;
+                FxSum d0[4], v0[4], d1[4], v1[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    d0[q].h = C.d0[q];
+                    v0[q].h = C.v0[q] >> sh;
+                    d1[q].h = C.d1[q];
+                    v1[q].h = C.v1[q] >> sh;
+                    d0[q].m = v0[q].m = d1[q].m = v1[q].m = 0;
+                }
+                for (int r = 0; r < n;) {
+                    const int re = min(n, r + FX_PAIRS);
+                    if (C.c0 + re - r > FX_PAIRS) {   // many markers per column: the sums start again
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int o = pl.base[q] + jseg * nx + x;
+                            add_sums(d0[q].units(), v0[q].units(), et, gacc, cells, pl.ok[q] && jseg >= 0, o);
+                            add_sums(d1[q].units(), v1[q].units(), et, gacc, cells, pl.ok[q] && jseg + 1 < nvx, o + nx);
+                            d0[q].clear();
+                            v0[q].clear();
+                            d1[q].clear();
+                            v1[q].clear();
+                        }
+                        C.c0 = C.c1 = 0;
+                    }
+                    C.c0 += re - r;
+                    C.c1 += re - r;
+                    // an even number of turns, the last of an odd list with
+                    // weights of zero (slot Z)
+                    const int re2 = re + ((re - r) & 1);
+#pragma unroll 2
+                    for (; r < re2; ++r) {
+                        const bool upper = r < nup, in = r < n;
+                        const int i = in ? r + (upper ? lo : blo) : 0;
+                        const int ia = upper ? i + NB : (in ? i : 2 * NB);
+                        const int4 a = pa[ia], v = pg[ia], qa = pqa[i], qb = pqb[i];
+                        const Limbs Q[4] = {{qa.x, qa.y}, {qa.z, qa.w}, {qb.x, qb.y}, {qb.z, qb.w}};
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            d0[q].add({a.x, a.y}, Q[q]);
+                            v0[q].add({v.x, v.y}, Q[q]);
+                            d1[q].add({a.z, a.w}, Q[q]);
+                            v1[q].add({v.z, v.w}, Q[q]);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    C.d0[q] = d0[q].units();
+                    C.v0[q] = v0[q].units();
+                    C.d1[q] = d1[q].units();
+                    C.v1[q] = v1[q].units();
+                }
+            }
+            __syncthreads();
+            par ^= 1;
+        }
+        // row jseg is complete (the next segment reaches rows jseg + 1 and
+        // jseg + 2): its sums into the global accumulator
+#pragma unroll
+        for (int c = 0; c < CPT; ++c) {
+            const int x = threadIdx.x + c * NT;
+            if (x < nx && jseg >= 0 && col[c].c0) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    add_sums(col[c].d0[q], col[c].v0[q], col[c].el, gacc, cells, pl.ok[q], pl.base[q] + jseg * nx + x);
+            }
+            col[c].next_row();
+        }
+    }
+    // (the last segment is row nvx - 1; what is left belongs to row nvx, off the grid)
+
+    if (nmov) atomicAdd(&mov_s, (unsigned long long)nmov);
+    if (nfar) atomicAdd(&far_s, (unsigned long long)nfar);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (mov_s) atomicAdd(&ctl->movers[s], mov_s);
+        if (far_s) atomicAdd(&ctl->far_movers[s], far_s);
+        if (flag_s) atomicOr(&ctl->err, ERR_TIMEOUT);
     }
 }
 
@@ -1044,7 +1244,7 @@ __global__ void __launch_bounds__(P3_THREADS) k_sort3(const StepArgs* __restrict
         const bool ok = k < end;
         int key = 0;
         if (ok) {
-            T w;
+            typename DualW<T>::type w;
             key = key_of(dual3(vxs[k], ax, bx, nvx, w), nvx);
         }
         const int kk = ok ? key : -1;
@@ -1061,7 +1261,7 @@ __global__ void __launch_bounds__(P3_THREADS) k_sort3(const StepArgs* __restrict
         int key = 0;
         T vx = 0;
         if (ok) {
-            T w;
+            typename DualW<T>::type w;
             vx = vxs[k];
             key = key_of(dual3(vx, ax, bx, nvx, w), nvx);
         }
@@ -1074,12 +1274,7 @@ __global__ void __launch_bounds__(P3_THREADS) k_sort3(const StepArgs* __restrict
             reinterpret_cast<T*>(sp.mv[dst][1])[slot] = reinterpret_cast<const T*>(sp.mv[src][1])[k];
             reinterpret_cast<T*>(sp.mv[dst][2])[slot] = reinterpret_cast<const T*>(sp.mv[src][2])[k];
             reinterpret_cast<T*>(sp.mf[dst])[slot] = reinterpret_cast<const T*>(sp.mf[src])[k];
-            if constexpr (sizeof(T) == 8) {
-                const double2* ps = reinterpret_cast<const double2*>(sp.mwq[src]) + 2 * (long long)k;
-                double2* pd = reinterpret_cast<double2*>(sp.mwq[dst]) + 2 * (long long)slot;
-                pd[0] = ps[0];
-                pd[1] = ps[1];
-            }
+            if constexpr (sizeof(T) == 8) sp.mwyz[dst][slot] = sp.mwyz[src][k];
         }
     }
 }
@@ -1162,7 +1357,7 @@ struct ArraySrc3 {
 template <typename T>
 __device__ __forceinline__ int bucket3(const SpDev& sp, const VCoef<T>& vc, const T (&v)[3])
 {
-    T w;
+    typename DualW<T>::type w;
     const int kx = key_of(dual3(v[0], vc.a[0], vc.b[0], vc.n[0], w), vc.n[0]);
     const int ky = key_of(dual3(v[1], vc.a[1], vc.b[1], vc.n[1], w), vc.n[1]);
     const int kz = key_of(dual3(v[2], vc.a[2], vc.b[2], vc.n[2], w), vc.n[2]);
@@ -1306,11 +1501,7 @@ __global__ void __launch_bounds__(256) k_src3_scatter(const StepArgs* __restrict
         pos.store(sp, 0, slot);
         for (int d = 0; d < 3; ++d) reinterpret_cast<T*>(sp.mv[0][d])[slot] = v[d];
         reinterpret_cast<T*>(sp.mf[0])[slot] = (T)mk.f;
-        if constexpr (sizeof(T) == 8) {
-            double wq[4];
-            marker_planes<double>(vc, v[1], v[2], wq);
-            store_planes(sp.mwq[0], slot, wq);
-        }
+        if constexpr (sizeof(T) == 8) sp.mwyz[0][slot] = marker_wyz(vc, v[1], v[2]);
     }
     if (over) atomicOr(&A->ctl->err, ERR_CAPACITY);
 }
@@ -1451,11 +1642,7 @@ __global__ void __launch_bounds__(256) k_rs3_scatter(const StepArgs* __restrict_
             pos[r].store(sp, dst, slot);
             for (int d = 0; d < 3; ++d) reinterpret_cast<T*>(sp.mv[dst][d])[slot] = v[r][d];
             reinterpret_cast<T*>(sp.mf[dst])[slot] = fv[r];
-            if constexpr (sizeof(T) == 8) {
-                double wq[4];
-                marker_planes<double>(vc, v[r][1], v[r][2], wq);
-                store_planes(sp.mwq[dst], slot, wq);
-            }
+            if constexpr (sizeof(T) == 8) sp.mwyz[dst][slot] = marker_wyz(vc, v[r][1], v[r][2]);
         }
     }
     if (over) atomicOr(&A->ctl->err, ERR_CAPACITY);
@@ -1519,51 +1706,47 @@ __global__ void k_getf3(const T* __restrict__ fg, const T* __restrict__ dg, int 
 // ---------------------------------------------------------------------------
 static int cpt_of(int nx) { return nx <= P3_THREADS ? 1 : (nx <= 2 * P3_THREADS ? 2 : 4); }
 
-template <typename T>
-static cudaError_t set_pd3_attr(int smem)
-{
-    cudaError_t e;
-    if ((e = raise_smem_limit(k_pd3<T, 1, false>, smem))) return e;
-    if ((e = raise_smem_limit(k_pd3<T, 2, false>, smem))) return e;
-    if ((e = raise_smem_limit(k_pd3<T, 4, false>, smem))) return e;
-    if ((e = raise_smem_limit(k_pd3<T, 1, true>, smem))) return e;
-    if ((e = raise_smem_limit(k_pd3<T, 2, true>, smem))) return e;
-    return raise_smem_limit(k_pd3<T, 4, true>, smem);
-}
-
 cudaError_t configure_vhs3(const StepArgs& h)
 {
     const int smem = (int)pd3_smem_bytes(h.fd.nx, nkey_max(h), h.prec);
-    return h.prec == AVL_FP32 ? set_pd3_attr<float>(smem) : set_pd3_attr<double>(smem);
+    cudaError_t e;
+    if (h.prec == AVL_FP64) {
+        if ((e = raise_smem_limit(k_pd3x<1, false>, smem))) return e;
+        if ((e = raise_smem_limit(k_pd3x<2, false>, smem))) return e;
+        if ((e = raise_smem_limit(k_pd3x<1, true>, smem))) return e;
+        return raise_smem_limit(k_pd3x<2, true>, smem);
+    }
+    if ((e = raise_smem_limit(k_pd3<1, false>, smem))) return e;
+    if ((e = raise_smem_limit(k_pd3<2, false>, smem))) return e;
+    if ((e = raise_smem_limit(k_pd3<4, false>, smem))) return e;
+    if ((e = raise_smem_limit(k_pd3<1, true>, smem))) return e;
+    if ((e = raise_smem_limit(k_pd3<2, true>, smem))) return e;
+    return raise_smem_limit(k_pd3<4, true>, smem);
 }
 
-template <typename T>
+template <bool PUSH>
 static void pd3_go(const StepArgs& h, const StepArgs* d, int mode, cudaStream_t st)
 {
-    const int smem = (int)pd3_smem_bytes(h.fd.nx, nkey_max(h), h.prec);
-    switch (cpt_of(h.fd.nx)) {
-        case 1:
-            if (mode == 1) k_pd3<T, 1, true><<<h.npen_total, P3_THREADS, smem, st>>>(d, mode);
-            else k_pd3<T, 1, false><<<h.npen_total, P3_THREADS, smem, st>>>(d, mode);
-            break;
-        case 2:
-            if (mode == 1) k_pd3<T, 2, true><<<h.npen_total, P3_THREADS, smem, st>>>(d, mode);
-            else k_pd3<T, 2, false><<<h.npen_total, P3_THREADS, smem, st>>>(d, mode);
-            break;
-        default:
-            if (mode == 1) k_pd3<T, 4, true><<<h.npen_total, P3_THREADS, smem, st>>>(d, mode);
-            else k_pd3<T, 4, false><<<h.npen_total, P3_THREADS, smem, st>>>(d, mode);
-            break;
+    const int smem = (int)pd3_smem_bytes(h.fd.nx, nkey_max(h), h.prec), cpt = cpt_of(h.fd.nx), n = h.npen_total;
+    if (h.prec == AVL_FP64) {   // nx <= 512
+        if (cpt == 1) k_pd3x<1, PUSH><<<n, P3_THREADS, smem, st>>>(d, mode);
+        else k_pd3x<2, PUSH><<<n, P3_THREADS, smem, st>>>(d, mode);
+    } else if (cpt == 1) {
+        k_pd3<1, PUSH><<<n, P3_THREADS, smem, st>>>(d, mode);
+    } else if (cpt == 2) {
+        k_pd3<2, PUSH><<<n, P3_THREADS, smem, st>>>(d, mode);
+    } else {
+        k_pd3<4, PUSH><<<n, P3_THREADS, smem, st>>>(d, mode);
     }
 }
 
 cudaError_t launch_pd3(const StepArgs& h, const StepArgs* d, int mode, cudaStream_t st)
 {
     if (h.npen_total == 0) return cudaSuccess;
-    if (h.prec == AVL_FP32)
-        pd3_go<float>(h, d, mode, st);
+    if (mode == 1)
+        pd3_go<true>(h, d, mode, st);
     else
-        pd3_go<double>(h, d, mode, st);
+        pd3_go<false>(h, d, mode, st);
     return cudaGetLastError();
 }
 
