@@ -50,10 +50,9 @@ constexpr int FIN_THREADS = 256;    // finalize block
 constexpr int FIN_XB = 16;          // x columns per finalize block
 constexpr int FIELD_THREADS = 512;  // Poisson cluster block
 constexpr int FIELD_CLUSTER = 8;    // CTAs in the Poisson cluster
-// table of the FP64 entropy logarithm (log_tab): one entry per 1/2048 of the
+// table of the FP64 entropy logarithm (fx_log): one entry per 1/2048 of the
 // mantissa interval [1, 2)
-constexpr int LOG_TAB_BITS = 11;
-constexpr int LOG_TAB_N = 1 << LOG_TAB_BITS;
+constexpr int LOG_TAB_N = 2048;
 constexpr long long WAIT_LIMIT = 1ll << 22;   // bounded mbarrier polls: the default limit of a first wait
                                               // (Ctl::wait_limit) and the limit of the drain that follows
                                               // a first wait that gave up
@@ -145,7 +144,7 @@ struct FieldDev {
     const double* gmul;        // cP kappa / K^2 for m <= nx/2 (0 at m = 0 and Nyquist)
     const double* green;       // nx <= GREEN_MAX: G of E = G (circulant) rho, else null
     double* diag;              // 3 + 3 ns
-    const double2* logtab;     // [LOG_TAB_N] (log c_j, 1 / c_j) of the FP64 entropy logarithm (log_tab)
+    const longlong2* logtab;   // [LOG_TAB_N] (2^62 / c_j, 2^53 log c_j) of the FP64 entropy logarithm (fx_log)
     double* hist;              // field history for marker refinement: [hist_cap][nx] FP64, or null;
                                // slot k holds E of the state after step hist_origin + k
     int hist_cap;
@@ -305,6 +304,6 @@ cudaError_t launch_poisson_dense(const double* rho, double* E, int nx, const dou
 cudaError_t launch_poisson(const double* rho, double* E, int nx, const double2* tw, const double* gmul,
                            cudaStream_t st);
 // table of the FP64 entropy logarithm: tab[j] = (log c_j, 1 / c_j), c_j = 1 + (j + 1/2) / 128
-cudaError_t init_log_table(double2* tab, cudaStream_t st);
+cudaError_t init_log_table(longlong2* tab, cudaStream_t st);
 
 }  // namespace avl

@@ -129,4 +129,69 @@ __device__ __forceinline__ double fx_scale(double d, int k)
     return __longlong_as_double(b + ((b & 0x7fffffffffffffffll) ? (long long)k << 52 : 0ll));
 }
 
+// n / d for a normal d > 0, in integers: a 24-bit reciprocal of d's mantissa
+// from the FP32 approximation, one Newton-Raphson step to 30 bits, the
+// quotient's first 29 bits, and one correction by the exact remainder
+// (P. Markstein, "Computation of elementary functions on the IBM RISC
+// System/6000 processor", IBM J. Res. Dev. 34, 1990, the same scheme in
+// floating point).  Within 0.52 units in the last place (0.6 % of quotients
+// are not the nearest).  Operands or quotients that are not normal numbers
+// take the division operator.
+__device__ __forceinline__ double fx_div(double n, double d)
+{
+    const long long bn = __double_as_longlong(n), bd = __double_as_longlong(d);
+    const int en = (int)(bn >> 52) & 0x7ff, ed = (int)(bd >> 52);
+    int ex = en - ed + 1023;
+    if (en == 0 || en == 0x7ff || ed <= 0 || ed >= 0x7ff || ex < 2 || ex > 0x7fd) return n / d;
+    const unsigned long long N = (unsigned long long)((bn & (FX_ONE - 1)) | FX_ONE);
+    const unsigned long long D = (unsigned long long)((bd & (FX_ONE - 1)) | FX_ONE);
+    // 1 / (D 2^-52) in (1/2, 1]: R0 2^-24, then R1 2^-31
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__int_as_float(0x3f800000 | (int)((D >> 29) & 0x7fffff))));
+    const int R0 = (__float_as_int(fminf(r, 0.99999994f)) & 0x7fffff) | 0x800000;
+    const unsigned Dh = (unsigned)(D >> 21);
+    const int e = (int)(((1ll << 55) - (long long)((unsigned long long)Dh * (unsigned)R0)) >> 23);
+    const unsigned R1 = ((unsigned)R0 << 7) + (unsigned)(int)(((long long)R0 * e) >> 25);
+    const unsigned Q0 = __umulhi((unsigned)(N >> 21), R1);                                  // 2^-30
+    const long long rem = (long long)((N << 30) - (unsigned long long)Q0 * D);               // 2^-82, exact
+    long long Q = ((long long)Q0 << 32) + (((long long)(int)(rem >> 24) * (int)(R1 >> 1)) >> 26);   // 2^-62
+    if (Q < (1ll << 62)) {
+        Q <<= 1;
+        --ex;
+    }
+    const long long M = (long long)(((unsigned long long)Q + 512ull) >> 10);   // (Q may be just below 2^63)
+    return __longlong_as_double((((long long)ex << 52) + (M - FX_ONE)) | (bn & (long long)0x8000000000000000ull));
+}
+
+// log f for a positive f: table-driven argument reduction (P. T. P. Tang,
+// "Table-driven implementation of the logarithm function in IEEE
+// floating-point arithmetic", ACM TOMS 16, 1990) in integers.  With
+// f = 2^e m, m in [1, 2), and c_j = 1 + (j + 1/2) / 2048 the centre of the
+// 1/2048 interval that holds m, log f = e ln 2 + log c_j + log1p(r),
+// r = m / c_j - 1 (|r| < 2^-12), log1p by its series to r^4, the cubic and
+// quartic terms (below 2^-37) in FP32.  tab[j] = (2^62 / c_j, 2^53 log c_j);
+// the sum is in units of 2^-53, good to two of them.  Subnormal f take the
+// library's function.
+__device__ __forceinline__ double fx_log(double f, const longlong2* __restrict__ tab)
+{
+    const long long b = __double_as_longlong(f);
+    if (b < 0x0010000000000000ll) return log(f);
+    const int e = (int)(b >> 52) - 1023;
+    const longlong2 t = __ldg(tab + (int)((b >> 41) & 2047));
+    const unsigned Mh = (unsigned)((b >> 32) & 0xfffff) | 0x100000, Ml = (unsigned)b;
+    const unsigned Ih = (unsigned)(t.x >> 32), Il = (unsigned)t.x;
+    const unsigned long long mid =
+        (unsigned long long)Mh * Il + (unsigned long long)Ml * Ih + (unsigned long long)__umulhi(Ml, Il);
+    // r in units of 2^-72, and of 2^-42
+    const long long T = ((long long)((unsigned long long)Mh * Ih - (1ull << 50)) << 22) + (long long)(mid >> 10);
+    const int Th = (int)((T + (1ll << 29)) >> 30);
+    const float rs = (float)Th * 2.2737367544323206e-13f;   // 2^-42
+    const int cu = __float2int_rn((rs * rs) * (rs * 9007199254740992.0f) * (1.f / 3.f - 0.25f * rs));
+    const int sq = (int)(((long long)Th * Th + (1ll << 31)) >> 32);   // r^2 / 2
+    // e ln 2 (2^63 ln 2 in two words)
+    const long long el2 = (long long)e * (0x58b90bfbll << 22) + (((long long)e * 0xe8e7bcd6ll + 512) >> 10);
+    const long long L = el2 + t.y + ((T + (1ll << 18)) >> 19) - sq + cu;
+    return fx_scale(fx_double(L), -53);
+}
+
 }  // namespace avl

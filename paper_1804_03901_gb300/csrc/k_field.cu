@@ -720,16 +720,19 @@ cudaError_t launch_field_batch(const BatchMap* bm, int nrun, int smem, int count
     return cudaGetLastError();
 }
 
-__global__ void k_log_table(double2* tab)
+__global__ void k_log_table(longlong2* tab)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < LOG_TAB_N) {
-        const double c = 1.0 + ((double)j + 0.5) / (double)LOG_TAB_N;
-        tab[j] = make_double2(log(c), 1.0 / c);
+        const double c = 1.0 + ((double)j + 0.5) / (double)LOG_TAB_N;   // exact
+        // 2^62 / c, c = 2^-12 (4096 + 2 j + 1)
+        const unsigned long long den = 4096ull + 2ull * j + 1ull, q = (1ull << 63) / den, r = (1ull << 63) - q * den;
+        const unsigned long long inv = (q << 11) + ((r << 11) + den / 2) / den;   // 2^74 / den
+        tab[j] = make_longlong2((long long)inv, __double2ll_rn(log(c) * 9007199254740992.0));
     }
 }
 
-cudaError_t init_log_table(double2* tab, cudaStream_t st)
+cudaError_t init_log_table(longlong2* tab, cudaStream_t st)
 {
     k_log_table<<<(LOG_TAB_N + 255) / 256, 256, 0, st>>>(tab);
     return cudaGetLastError();

@@ -47,6 +47,7 @@ def test_fixed_point_sums(nx, nv, n, values, B):
             sim.step(1)
             orc.step(1)
         got, den = sim.get_f(0, with_n=True)
-        for a, b in ((got, orc.f[0]), (den, orc.den[0])):
+        # W_kin, N and the entropy (table logarithm, units of 2^-53)
+        for a, b in ((got, orc.f[0]), (den, orc.den[0]), (sim.get_diag()[3:], orc.diag()[3:])):
             assert np.linalg.norm(a - b) < TOL * np.linalg.norm(b), (step, np.linalg.norm(a - b) / np.linalg.norm(b))
     sim.close()
