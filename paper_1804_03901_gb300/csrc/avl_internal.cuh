@@ -60,7 +60,8 @@ constexpr int P3_THREADS = 256;     // 1d3v pencil block (one thread per x colum
 constexpr int FIN3_X = 32;          // 1d3v finalize: x columns per block
 constexpr int FIN3_R = 8;           //                row lanes per block
 constexpr int NV3_MAX = 1024;       // 1d3v: largest nv[0] (key histogram of a pencil in shared memory)
-constexpr int GREEN_MAX = 1024;     // largest nx solved by the circulant product (adjoint engine)
+constexpr int GREEN_MAX = 1024;     // largest nx solved by the circulant product (adjoint engine; steps on a
+                                    // grid that is no power of two)
 
 // elements of one deposit-window plane (numerator, denominator or reference)
 // of a 1d1v chunk: Wmax rows x nx columns, padded to a multiple of 4 so that

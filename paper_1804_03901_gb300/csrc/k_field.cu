@@ -231,6 +231,24 @@ __device__ __forceinline__ int best_cover_warp(int2 h, int wk)
     return __reduce_max_sync(0xffffffffu, best);
 }
 
+// E = G rho (circulant, G odd in i - j) on the columns [xlo, xhi) by a CTA of
+// the cluster: r holds rho less a constant, which the product removes (k = 0)
+// and which would otherwise only bring its rounding; E is CTA 0's.  A warp
+// per output, lanes over j.
+__device__ void dense_slice(const double* r, const double* __restrict__ G, double* E, int nx, int xlo, int xhi)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int i = xlo + warp; i < xhi; i += FIELD_THREADS / 32) {
+        double acc = 0.0;
+        for (int j = lane; j < nx; j += 32) {
+            const int d = i - j;
+            acc = fma(__ldg(G + (d < 0 ? d + nx : d)), r[j], acc);
+        }
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+        if (lane == 0) E[i] = acc;
+    }
+}
+
 constexpr int FIELD_DECIDE = FIELD_CLUSTER - 2;   // CTAs 1 .. FIELD_DECIDE decide the re-sorts
 constexpr int FIELD_DIAG = FIELD_CLUSTER - 1;     // the last CTA sums the diagnostics
 
@@ -409,6 +427,24 @@ __global__ void __cluster_dims__(FIELD_CLUSTER, 1, 1) __launch_bounds__(FIELD_TH
         }
     }
     cluster.sync();
+    // Grids that are no power of two (and small enough for the Green's
+    // function table): the product spread over CTAs 1 .. 7 in place of CTA
+    // 0's direct transforms, whose 2 nx^2 FP64 operations one SM takes (nx =
+    // 300: 112 -> 20 us for the kernel, nx = 100: 52 -> 17 us; a power of two
+    // takes the FFT, 18 us at 64 and 27 us at 512).
+    const bool dense = !fd.pow2 && fd.green != nullptr;
+    if (dense) {
+        if (rank != 0) {
+            for (int j = threadIdx.x; j < nx; j += FIELD_THREADS) rho_s[j] = rho0[j] - rho0[0];
+            __syncthreads();
+            const int slice = (nx + FIELD_CLUSTER - 2) / (FIELD_CLUSTER - 1);
+            double* E0 = cluster.map_shared_rank(reinterpret_cast<double*>(work), 0);
+            dense_slice(rho_s, fd.green, E0, nx, (rank - 1) * slice, min(nx, rank * slice));
+        } else {
+            for (int x = threadIdx.x; x < nx; x += FIELD_THREADS) fd.rho[x] = rho_s[x];
+        }
+        cluster.sync();
+    }
     if (rank != 0) {
         if (rank == FIELD_DIAG) diag_sums(A, cluster.map_shared_rank(dfin, 0));
         if (count_step) resort_work(A, rank, reinterpret_cast<int*>(smem));
@@ -417,7 +453,8 @@ __global__ void __cluster_dims__(FIELD_CLUSTER, 1, 1) __launch_bounds__(FIELD_TH
     }
 
     // --- CTA 0: Poisson --------------------------------------------------
-    for (int x = threadIdx.x; x < nx; x += FIELD_THREADS) fd.rho[x] = rho_s[x];
+    if (!dense)
+        for (int x = threadIdx.x; x < nx; x += FIELD_THREADS) fd.rho[x] = rho_s[x];
     // per-species constants of the shift tables: loads issued before the
     // solve, their values used after it
     double qm_dt = 0.0, inv_dv = 0.0;
@@ -429,7 +466,12 @@ __global__ void __cluster_dims__(FIELD_CLUSTER, 1, 1) __launch_bounds__(FIELD_TH
         inv_dv = sp.inv_dv[0];
         shsel = A->ctl->shsel[threadIdx.x];
     }
-    poisson_spectral(rho_s, work, staged ? tw_s : fd.tw, staged ? gm_s : nullptr, nx, fd.pow2, fd.tw, fd.gmul);
+    if (dense) {
+        for (int x = threadIdx.x; x < nx; x += FIELD_THREADS) rho_s[x] = reinterpret_cast<const double*>(work)[x];
+        __syncthreads();
+    } else {
+        poisson_spectral(rho_s, work, staged ? tw_s : fd.tw, staged ? gm_s : nullptr, nx, fd.pow2, fd.tw, fd.gmul);
+    }
     if (threadIdx.x < A->ns) {
         shf_s[threadIdx.x] = mobile ? (float)(qm_dt * inv_dv) : 0.f;
         tgt_s[threadIdx.x] = count_step ? 1 - shsel : shsel;
