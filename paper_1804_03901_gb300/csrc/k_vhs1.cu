@@ -55,9 +55,25 @@ __device__ __forceinline__ int key_rel(float dv, int kb, float inv_dv, int nv)
 {
     return clampi(kb + (int)floorf(__fmaf_rn(dv, inv_dv, -0.5f)), 0, nv - 1);
 }
+// FP64: row relative to the reference and weight of the next row, a count of
+// 2^-52, from t as a 64-bit count of 2^-52 rows (beyond 1023 rows, which that
+// does not hold, from its floor)
+__device__ __forceinline__ int vrow_rel(double dv, double inv_dv, long long& w)
+{
+    const double t = __fma_rn(dv, inv_dv, -0.5);
+    if (((__double2hiint(t) >> 20) & 0x7ff) < 1033) {   // |t| < 1024
+        const long long n = fx_count(t);
+        w = n & (FX_ONE - 1);
+        return (int)(n >> 52);
+    }
+    const double ft = floor(t);
+    w = fx_count(t - ft);
+    return (int)ft;
+}
 __device__ __forceinline__ int key_rel(double dv, int kb, double inv_dv, int nv)
 {
-    return clampi(kb + (int)floor(__fma_rn(dv, inv_dv, -0.5)), 0, nv - 1);
+    long long w;
+    return clampi(kb + vrow_rel(dv, inv_dv, w), 0, nv - 1);
 }
 __device__ __forceinline__ int key_abs(double v, double vmin, double inv_dv, int nv)
 {
@@ -154,10 +170,8 @@ __device__ __forceinline__ void wrap_pair_in(int i0, int nx, int& ia, int& ib)
 
 // numerator and denominator contributions of a run of markers that share the
 // same four cells (lower corner i0, j0)
-template <typename T>
-struct Run;
-
-// FP32: a run holds at most MPT markers, summed in registers; the run sums
+//
+// A run holds at most MPT markers, summed in registers; the run sums
 // are added into the window with plain FP32 shared-memory reductions.  The
 // window's numerator plane holds deviations from a reference value per
 // cell, sum alpha (f_l - f_ref), with f_ref the cell's f of the previous
@@ -172,8 +186,7 @@ struct Run;
 // with f itself; the rounding of the denominator enters f only through
 // (f - f_ref) as well.  Runs outside the window carry absolute values into
 // the FP64 overflow grids.
-template <>
-struct Run<float> {
+struct Run {
     int i0, j0;
     float r;
     float nh[4], dh[4];
@@ -209,38 +222,6 @@ struct Run<float> {
     __device__ __forceinline__ double den(int k) const { return (double)dh[k]; }
 };
 
-template <>
-struct Run<double> {
-    int i0, j0;
-    double nh[4], dh[4];
-    __device__ __forceinline__ void reset(int i, int j)
-    {
-        i0 = i;
-        j0 = j;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) nh[k] = dh[k] = 0.0;
-    }
-    __device__ __forceinline__ void add(const double (&a)[4], double f, bool)
-    {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            nh[k] += a[k] * f;
-            dh[k] += a[k];
-        }
-    }
-    // window planes: num, den
-    __device__ __forceinline__ void to_window(double* win, int plane, const int (&cell)[4], const double*) const
-    {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            atomicAdd(win + cell[k], nh[k]);
-            atomicAdd(win + plane + cell[k], dh[k]);
-        }
-    }
-    __device__ __forceinline__ double num(int k) const { return nh[k]; }
-    __device__ __forceinline__ double den(int k) const { return dh[k]; }
-};
-
 // the rare out-of-window path: FP64 global atomics into the overflow grids;
 // each row written is tagged with the step (tag), so that the finalize reads
 // and clears only the rows of this step's overflow
@@ -269,9 +250,8 @@ __device__ __forceinline__ void flush_overflow(int ia, int ib, int j0, int nx, i
 // flush a run into the window or, if one of its rows falls outside, into the
 // FP64 overflow grids; window row of grid row j at column x = j - sh[x] - row0.
 // Returns true for the overflow path.
-template <typename T>
-__device__ __forceinline__ bool flush_run(const Run<T>& r, T* win, int plane, int row0, int W, int nx, int nv,
-                                          const int* sh, const T* fref, double* ovf_num, double* ovf_den,
+__device__ __forceinline__ bool flush_run(const Run& r, float* win, int plane, int row0, int W, int nx, int nv,
+                                          const int* sh, const float* fref, double* ovf_num, double* ovf_den,
                                           int* ovf_tag, int tag)
 {
     if (r.j0 + 1 < 0 || r.j0 >= nv) return false;   // footprint entirely off the velocity grid
@@ -538,12 +518,11 @@ __global__ void __launch_bounds__(PD_THREADS) k_rs1(const StepArgs* __restrict__
 // same footprint summed in registers first) and written back in place, and
 // its new key is counted into cnt[1 - hsel] for the next step.  On a re-sort
 // step the markers are read from the buffer k_rs1 has just written.
-// FP64: one CTA per SM with the registers the push and deposit need (at two
-// CTAs, 64 registers, it spills).
-template <typename T, bool BATCH, bool PUSH>
-__global__ void __launch_bounds__(PD_THREADS, sizeof(T) == 8 ? 1 : 2) k_pd1(const StepArgs* __restrict__ A0,
+template <bool BATCH, bool PUSH>
+__global__ void __launch_bounds__(PD_THREADS, 2) k_pd1(const StepArgs* __restrict__ A0,
                                                        const BatchMap* __restrict__ bm)
 {
+    using T = float;
     constexpr int mode = PUSH ? 1 : 0;
     extern __shared__ __align__(128) unsigned char smem[];
     int g = blockIdx.x;
@@ -574,7 +553,7 @@ __global__ void __launch_bounds__(PD_THREADS, sizeof(T) == 8 ? 1 : 2) k_pd1(cons
     const int plane = win_plane(W, nx);
     const size_t win_bytes = (size_t)2 * sizeof(T) * plane;
 
-    const T* Eg = (sizeof(T) == 4) ? reinterpret_cast<const T*>(A->fd.E32) : reinterpret_cast<const T*>(A->fd.E64);
+    const T* Eg = A->fd.E32;
     const bool use_bulk = push && ((nx * sizeof(T)) % 16 == 0);
     if (threadIdx.x == 0) {
         misc[0] = 0;
@@ -616,10 +595,10 @@ __global__ void __launch_bounds__(PD_THREADS, sizeof(T) == 8 ? 1 : 2) k_pd1(cons
     const int row0 = misc[2];
 
     T* win = reinterpret_cast<T*>(winb);
-    // FP32: the reference plane, f of the previous reconstruction at every
+    // the reference plane, f of the previous reconstruction at every
     // window cell (grid row wr + row0 + shs[x] of column x; 0 off the grid)
     T* fref = win + 2 * plane;
-    if constexpr (sizeof(T) == 4) {
+    {
         // eight rows' loads in flight per thread before their stores
         constexpr int RB = 8;
         const float* fprev = reinterpret_cast<const float*>(sp.fgrid);
@@ -643,8 +622,6 @@ __global__ void __launch_bounds__(PD_THREADS, sizeof(T) == 8 ? 1 : 2) k_pd1(cons
     const T qm_dt = (T)sp.qm_dt;
     const T dt_dx = (T)sp.dt_dx;
     const T vref_dtdx = (T)((sp.vmin[0] + (double)kb * sp.dv[0]) * sp.dt_dx);
-    // FP64: the displacement in 2^-52 cells (fixed-point positions, PosX)
-    const double dt_dx52 = sp.dt_dx * PosX::ONE, vref_dtdx52 = (double)vref_dtdx * PosX::ONE;
     double* ovf_num = sp.ovf;
     double* ovf_den = sp.ovf + (size_t)nv * nx;
     int* ovf_tag = sp.ovf_tag;
@@ -662,24 +639,17 @@ __global__ void __launch_bounds__(PD_THREADS, sizeof(T) == 8 ? 1 : 2) k_pd1(cons
         if (any) {
             loadg(dvp + g0, dv8);
             loadg(fp + g0, f8);
-            if constexpr (sizeof(T) == 4) {
-                int c8[MPT];
-                float o8[MPT];
-                loadg(reinterpret_cast<const int*>(sp.mx[cb]) + g0, c8);
-                loadg(sp.moff[cb] + g0, o8);
+            int c8[MPT];
+            float o8[MPT];
+            loadg(reinterpret_cast<const int*>(sp.mx[cb]) + g0, c8);
+            loadg(sp.moff[cb] + g0, o8);
 #pragma unroll
-                for (int m = 0; m < MPT; ++m) {
-                    pos8[m].c = c8[m];
-                    pos8[m].o = o8[m];
-                }
-            } else {
-                long long x8[MPT];
-                loadg(reinterpret_cast<const long long*>(sp.mx[cb]) + g0, x8);
-#pragma unroll
-                for (int m = 0; m < MPT; ++m) pos8[m].X = x8[m];
+            for (int m = 0; m < MPT; ++m) {
+                pos8[m].c = c8[m];
+                pos8[m].o = o8[m];
             }
         }
-        Run<T> run;
+        Run run;
         run.reset(0x7fffffff, 0);
         bool have = false;
         // one marker of the thread's group: push, footprint, run, key count
@@ -696,10 +666,7 @@ __global__ void __launch_bounds__(PD_THREADS, sizeof(T) == 8 ? 1 : 2) k_pd1(cons
                     wrap_pair_in(i0, nx, ia, ib);
                     const T El = ((T)1 - w) * Es[ia] + w * Es[ib];
                     dv += qm_dt * El;
-                    if constexpr (sizeof(T) == 8)
-                        pos.drift_scaled(__fma_rn(dv, dt_dx52, vref_dtdx52), nx);   // in 2^-52 cells
-                    else
-                        pos.drift(vref_dtdx + dv * dt_dx, nx);
+                    pos.drift(vref_dtdx + dv * dt_dx, nx);
                     dv8[m] = dv;
                 }
                 // cloud-in-cell footprint of the new state (Eq. 4 weights)
@@ -708,11 +675,7 @@ __global__ void __launch_bounds__(PD_THREADS, sizeof(T) == 8 ? 1 : 2) k_pd1(cons
                 pos.cic(i0, wx);
                 // the fused multiply-add of key_rel, so that the footprint row
                 // is the key every other kernel computes from the stored value
-                T t;
-                if constexpr (sizeof(T) == 4)
-                    t = __fmaf_rn(dv, inv_dv, -0.5f);
-                else
-                    t = __fma_rn(dv, inv_dv, -0.5);
+                const T t = __fmaf_rn(dv, inv_dv, -0.5f);
                 const T ft = floor(t);
                 const int j0 = kb + (int)ft;
                 code = rel_code(clampi(j0, 0, nv - 1), kbase);
@@ -720,7 +683,7 @@ __global__ void __launch_bounds__(PD_THREADS, sizeof(T) == 8 ? 1 : 2) k_pd1(cons
                 const bool first = !have || i0 != run.i0 || j0 != run.j0;
                 if (first) {
                     if (have)
-                        n_over += flush_run<T>(run, win, plane, row0, W, nx, nv, shs, fref, ovf_num, ovf_den, ovf_tag,
+                        n_over += flush_run(run, win, plane, row0, W, nx, nv, shs, fref, ovf_num, ovf_den, ovf_tag,
                                                tag)
                                       ? 1u
                                       : 0u;
@@ -736,28 +699,21 @@ __global__ void __launch_bounds__(PD_THREADS, sizeof(T) == 8 ? 1 : 2) k_pd1(cons
 #pragma unroll
         for (int m = 0; m < MPT; ++m) one(m, g0 + m < end);
         if (have)
-            n_over += flush_run<T>(run, win, plane, row0, W, nx, nv, shs, fref, ovf_num, ovf_den, ovf_tag, tag) ? 1u
+            n_over += flush_run(run, win, plane, row0, W, nx, nv, shs, fref, ovf_num, ovf_den, ovf_tag, tag) ? 1u
                                                                                                                 : 0u;
         if (!push) continue;
         // in place: the positions and velocities go back where they came from
         if (any) {
             storeg(dvp + g0, dv8);
-            if constexpr (sizeof(T) == 4) {
-                int c8[MPT];
-                float o8[MPT];
+            int c8[MPT];
+            float o8[MPT];
 #pragma unroll
-                for (int m = 0; m < MPT; ++m) {
-                    c8[m] = pos8[m].c;
-                    o8[m] = pos8[m].o;
-                }
-                storeg(reinterpret_cast<int*>(sp.mx[cb]) + g0, c8);
-                storeg(sp.moff[cb] + g0, o8);
-            } else {
-                long long x8[MPT];
-#pragma unroll
-                for (int m = 0; m < MPT; ++m) x8[m] = pos8[m].X;
-                storeg(reinterpret_cast<long long*>(sp.mx[cb]) + g0, x8);
+            for (int m = 0; m < MPT; ++m) {
+                c8[m] = pos8[m].c;
+                o8[m] = pos8[m].o;
             }
+            storeg(reinterpret_cast<int*>(sp.mx[cb]) + g0, c8);
+            storeg(sp.moff[cb] + g0, o8);
         }
     }
     if (n_over) atomicAdd(&misc[0], (int)n_over);
@@ -769,6 +725,205 @@ __global__ void __launch_bounds__(PD_THREADS, sizeof(T) == 8 ? 1 : 2) k_pd1(cons
         fence_proxy_async_smem();
         unsigned char* dstp = reinterpret_cast<unsigned char*>(sp.partial) + (size_t)c * win_bytes;
         bulk_s2g(dstp, winb, (unsigned)win_bytes);
+        bulk_commit();
+        if (misc[0]) atomicAdd(&ctl->ovf_count[s], (unsigned long long)misc[0]);
+        bulk_wait_all();
+    }
+}
+
+// FP64 form.  The FP64 pipe takes a warp instruction per 64 clocks and
+// sub-partition, and a shared-memory FP64 reduction is a loop around such an
+// addition, so the weights are integers (fixed.cuh) and the denominator of
+// Eq. 4 is summed in the window as 64-bit counts of 2^-wb (wb: what M weights
+// of at most 1 leave of 63 bits), exact sums of the rounded weights.  The
+// numerator takes the same rounded weight times the value, one FP64 product
+// and one FP64 reduction per corner, so that the rounding of a weight enters
+// f only through the spread of the values in a cell.  14 FP64 operations per
+// marker where the same deposit in FP64, with its runs of markers of one
+// footprint summed in registers first, took about 40 (lanes end their runs
+// at different markers, so a warp flushed at every marker all the same):
+// 13.5 M markers, 512 x 6600 cells 1.12 -> 0.63 ms. The conversion of the
+// displacement in integers is worth 5 % (0.66 ms on the FP64 pipe); two CTAs
+// per SM at 64 registers are slower (0.70 ms).
+template <bool BATCH, bool PUSH>
+__global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restrict__ A0,
+                                                        const BatchMap* __restrict__ bm)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    int g = blockIdx.x;
+    const StepArgs* __restrict__ A = A0;
+    if constexpr (BATCH) A = batch_run(A0, bm, bm->pd_base, g);
+    const int s = species_of_chunk(A, g);
+    const SpDev& sp = A->sp[s];
+    if (PUSH && !sp.mobile) return;
+    Ctl* ctl = A->ctl;
+    const int hs = ctl->hsel[s];
+    const int c = g - sp.chunk_base;
+    const int nx = sp.nx, nv = sp.nvflat, W = sp.Wmax;
+    const int cb = (PUSH && ctl->sort_now[s]) ? 1 - ctl->cur[s] : ctl->cur[s];
+    const int n_all = (int)sp.n;
+    const int beg = c * sp.M, end = min((c + 1) * sp.M, n_all);
+    const int kb = sp.KB[cb][c];
+    const int kbase = kb - HIST_R;
+
+    // shared memory: (q/m) dt E | barrier, counters | histograms | row shifts | window
+    const size_t eb = ((size_t)nx * 8 + 15) & ~size_t(15);
+    double* Es = reinterpret_cast<double*>(smem);
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + eb);
+    int* misc = reinterpret_cast<int*>(smem + eb + 16);   // [0] overflow runs, [2] row0
+    int* scnt = reinterpret_cast<int*>(smem + eb + 32);   // next-step histogram
+    int* hcur = scnt + HIST_S;                             // current-key histogram (window placement)
+    int* shs = hcur + HIST_S;                              // per-column row shift (nx)
+    double* win = reinterpret_cast<double*>(smem + eb + 32 + 2 * HIST_S * 4 + ((4 * nx + 15) & ~15));
+    const int plane = win_plane(W, nx);
+    const size_t win_bytes = (size_t)2 * 8 * plane;
+    unsigned long long* wden = reinterpret_cast<unsigned long long*>(win + plane);
+
+    const bool use_bulk = PUSH && nx % 2 == 0;
+    if (threadIdx.x == 0) {
+        misc[0] = 0;
+        if (use_bulk) {
+            mbar_init(bar, 1);
+            fence_mbar_init();
+        }
+    }
+    for (int i = threadIdx.x; i < HIST_S; i += PD_THREADS) {
+        scnt[i] = 0;
+        hcur[i] = sp.cnt[hs][(size_t)c * HIST_S + i];
+    }
+    // window coordinate of a deposit at row j, column x: j - shs[x], which
+    // removes this step's drift
+    const int ssel = ctl->shsel[s];
+    for (int i = threadIdx.x; i < nx; i += PD_THREADS) shs[i] = PUSH ? sp.shift[ssel][i] : 0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const int r0 = best_window(hcur, kbase, W, nullptr);
+        misc[2] = r0;
+        sp.wrow0[c] = r0;
+        if (use_bulk) {
+            mbar_arrive_expect_tx(bar, (unsigned)(nx * 8));
+            bulk_g2s(Es, A->fd.E64, (unsigned)(nx * 8), bar);
+        }
+    }
+    {   // zero the window while the field is in flight
+        float4* w4 = reinterpret_cast<float4*>(win);
+        const int n4 = (int)(win_bytes / 16);
+        for (int i = threadIdx.x; i < n4; i += PD_THREADS) w4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (PUSH && !use_bulk)
+        for (int i = threadIdx.x; i < nx; i += PD_THREADS) Es[i] = A->fd.E64[i];
+    // a first wait that gives up flags the timeout; the copy is drained and
+    // the step goes on (every thread reaches the barrier below)
+    if (use_bulk && !mbar_wait_or_drain(bar, 0, ctl->wait_limit, WAIT_LIMIT))
+        if (threadIdx.x == 0) atomicOr(&ctl->err, ERR_TIMEOUT);
+    __syncthreads();
+    const int row0 = misc[2];
+    if (PUSH) {
+        for (int i = threadIdx.x; i < nx; i += PD_THREADS) Es[i] *= sp.qm_dt;
+        __syncthreads();
+    }
+    const double inv_dv = sp.inv_dv[0];
+    // displacement in cells: (v_ref + dv) dt / dx, v_ref of the chunk's reference row
+    const double dt_dx = sp.dt_dx, vref_dtdx = (sp.vmin[0] + (double)kb * sp.dv[0]) * sp.dt_dx;
+    // bits of the window's weights: M of them, none above 1, stay below 2^62
+    const int wb = 62 - max(32 - __clz(sp.M - 1), 5), wsh = 57 - wb;
+    double* ovf_num = sp.ovf;
+    double* ovf_den = sp.ovf + (size_t)nv * nx;
+    int* ovf_tag = sp.ovf_tag;
+    const int tag = (int)ctl->step + 1;
+    double* dvp = reinterpret_cast<double*>(sp.mv[cb][0]);
+    const double* fp = reinterpret_cast<const double*>(sp.mf[cb]);
+    long long* xp = reinterpret_cast<long long*>(sp.mx[cb]);
+    int* far_next = sp.far_cnt[1 - hs];
+    unsigned n_over = 0;
+
+    for (int base = beg; base < end; base += PD_THREADS * MPT) {
+        const int g0 = base + threadIdx.x * MPT;
+        const bool any = g0 < end;
+        double dv4[MPT], f4[MPT];
+        long long x4[MPT];
+        if (any) {
+            loadg(dvp + g0, dv4);
+            loadg(fp + g0, f4);
+            loadg(xp + g0, x4);
+        }
+#pragma unroll
+        for (int m = 0; m < MPT; ++m) {
+            const bool ok = g0 + m < end;
+            int code = 0;
+            if (ok) {
+                PosX pos;
+                pos.X = x4[m];
+                double dv = dv4[m];
+                if (PUSH) {
+                    int i0, ia, ib;
+                    double w;
+                    pos.cic(i0, w);
+                    wrap_pair_in(i0, nx, ia, ib);
+                    const double Ea = Es[ia];
+                    dv += __fma_rn(w, Es[ib] - Ea, Ea);
+                    pos.wrap((long long)((unsigned long long)pos.X +
+                                         (unsigned long long)fx_count(__fma_rn(dv, dt_dx, vref_dtdx))),
+                             nx);
+                    x4[m] = pos.X;
+                    dv4[m] = dv;
+                }
+                // cloud-in-cell footprint of the new state (Eq. 4 weights); the
+                // row from the fused multiply-add of key_rel
+                const long long U = pos.X - (FX_ONE >> 1);
+                const int i0 = (int)(U >> 52);
+                int ia, ib;
+                wrap_pair_in(i0, nx, ia, ib);
+                long long w52;
+                const int j0 = kb + vrow_rel(dv, inv_dv, w52);
+                code = rel_code(clampi(j0, 0, nv - 1), kbase);
+                if (j0 + 1 >= 0 && j0 < nv) {
+                    // 2^-57: one product, the others by difference
+                    const long long u = (U & (FX_ONE - 1)) << 5, w = w52 << 5;
+                    const long long a3 = fx_mul(fx_split(u), fx_split(w >> 1)), a2 = w - a3, a1 = u - a3;
+                    const long long half = wsh > 0 ? 1ll << (wsh - 1) : 0;
+                    const long long a[4] = {((FX_ONE << 5) - u - a2 + half) >> wsh, (a1 + half) >> wsh,
+                                            (a2 + half) >> wsh, (a3 + half) >> wsh};
+                    const int wa = j0 - shs[ia] - row0, wc = j0 - shs[ib] - row0;
+                    const double f = f4[m];
+                    if (wa >= 0 && wa + 1 < W && wc >= 0 && wc + 1 < W) {
+                        const int cell[4] = {wa * nx + ia, wc * nx + ib, (wa + 1) * nx + ia, (wc + 1) * nx + ib};
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            atomicAdd(wden + cell[k], (unsigned long long)a[k]);
+                            atomicAdd(win + cell[k], fx_scale(fx_double(a[k]), -wb) * f);
+                        }
+                    } else {
+                        double d[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) d[k] = fx_scale(fx_double(a[k]), -wb);
+                        flush_overflow(ia, ib, j0, nx, nv, d[0] * f, d[1] * f, d[2] * f, d[3] * f, d[0], d[1], d[2],
+                                       d[3], ovf_num, ovf_den, ovf_tag, tag);
+                        ++n_over;
+                    }
+                }
+            }
+            // the new key counted for this chunk (next step's window)
+            if (PUSH) hist_add(scnt, far_next, code, ok);
+        }
+        // in place: the positions and velocities go back where they came from
+        if (PUSH && any) {
+            storeg(dvp + g0, dv4);
+            storeg(xp + g0, x4);
+        }
+    }
+    if (n_over) atomicAdd(&misc[0], (int)n_over);
+    __syncthreads();
+    if (PUSH)
+        for (int i = threadIdx.x; i < HIST_S; i += PD_THREADS) sp.cnt[1 - hs][(size_t)c * HIST_S + i] = scnt[i];
+    for (int i = threadIdx.x; i < plane; i += PD_THREADS)
+        win[plane + i] = fx_scale(fx_double((long long)wden[i]), -wb);
+    __syncthreads();
+    // flush the window to this chunk's partial sums with one bulk copy
+    if (threadIdx.x == 0) {
+        fence_proxy_async_smem();
+        unsigned char* dstp = reinterpret_cast<unsigned char*>(sp.partial) + (size_t)c * win_bytes;
+        bulk_s2g(dstp, win, (unsigned)win_bytes);
         bulk_commit();
         if (misc[0]) atomicAdd(&ctl->ovf_count[s], (unsigned long long)misc[0]);
         bulk_wait_all();
@@ -1322,14 +1477,14 @@ cudaError_t launch_pd1_batch(int prec, const BatchMap* bm, int blocks, int smem,
     if (blocks == 0) return cudaSuccess;
     if (prec == AVL_FP32) {
         if (mode == 1)
-            k_pd1<float, true, true><<<blocks, PD_THREADS, smem, st>>>(nullptr, bm);
+            k_pd1<true, true><<<blocks, PD_THREADS, smem, st>>>(nullptr, bm);
         else
-            k_pd1<float, true, false><<<blocks, PD_THREADS, smem, st>>>(nullptr, bm);
+            k_pd1<true, false><<<blocks, PD_THREADS, smem, st>>>(nullptr, bm);
     } else {
         if (mode == 1)
-            k_pd1<double, true, true><<<blocks, PD_THREADS, smem, st>>>(nullptr, bm);
+            k_pd1x<true, true><<<blocks, PD_THREADS, smem, st>>>(nullptr, bm);
         else
-            k_pd1<double, true, false><<<blocks, PD_THREADS, smem, st>>>(nullptr, bm);
+            k_pd1x<true, false><<<blocks, PD_THREADS, smem, st>>>(nullptr, bm);
     }
     return cudaGetLastError();
 }
@@ -1366,19 +1521,19 @@ int pd1_smem_needed(const StepArgs& h) { return max_pd_smem(h); }
 
 // dynamic shared-memory limit of the deposit kernel, set whenever the chunk
 // layout changes (outside any stream capture)
-template <typename T>
-static cudaError_t set_pd1_limit_t(int smem)
-{
-    cudaError_t e;
-    if ((e = raise_smem_limit(k_pd1<T, false, false>, smem))) return e;
-    if ((e = raise_smem_limit(k_pd1<T, false, true>, smem))) return e;
-    if ((e = raise_smem_limit(k_pd1<T, true, false>, smem))) return e;
-    return raise_smem_limit(k_pd1<T, true, true>, smem);
-}
-
 static cudaError_t set_pd1_limit(int prec, int smem)
 {
-    return prec == AVL_FP32 ? set_pd1_limit_t<float>(smem) : set_pd1_limit_t<double>(smem);
+    cudaError_t e;
+    if (prec == AVL_FP64) {
+        if ((e = raise_smem_limit(k_pd1x<false, false>, smem))) return e;
+        if ((e = raise_smem_limit(k_pd1x<false, true>, smem))) return e;
+        if ((e = raise_smem_limit(k_pd1x<true, false>, smem))) return e;
+        return raise_smem_limit(k_pd1x<true, true>, smem);
+    }
+    if ((e = raise_smem_limit(k_pd1<false, false>, smem))) return e;
+    if ((e = raise_smem_limit(k_pd1<false, true>, smem))) return e;
+    if ((e = raise_smem_limit(k_pd1<true, false>, smem))) return e;
+    return raise_smem_limit(k_pd1<true, true>, smem);
 }
 
 cudaError_t configure_vhs1(const StepArgs& h) { return set_pd1_limit(h.prec, max_pd_smem(h)); }
@@ -1406,14 +1561,14 @@ cudaError_t launch_pd1(const StepArgs& h, const StepArgs* d, int mode, cudaStrea
     const int smem = max_pd_smem(h);
     if (h.prec == AVL_FP32) {
         if (mode == 1)
-            k_pd1<float, false, true><<<h.nchunk_total, PD_THREADS, smem, st>>>(d, nullptr);
+            k_pd1<false, true><<<h.nchunk_total, PD_THREADS, smem, st>>>(d, nullptr);
         else
-            k_pd1<float, false, false><<<h.nchunk_total, PD_THREADS, smem, st>>>(d, nullptr);
+            k_pd1<false, false><<<h.nchunk_total, PD_THREADS, smem, st>>>(d, nullptr);
     } else {
         if (mode == 1)
-            k_pd1<double, false, true><<<h.nchunk_total, PD_THREADS, smem, st>>>(d, nullptr);
+            k_pd1x<false, true><<<h.nchunk_total, PD_THREADS, smem, st>>>(d, nullptr);
         else
-            k_pd1<double, false, false><<<h.nchunk_total, PD_THREADS, smem, st>>>(d, nullptr);
+            k_pd1x<false, false><<<h.nchunk_total, PD_THREADS, smem, st>>>(d, nullptr);
     }
     return cudaGetLastError();
 }
