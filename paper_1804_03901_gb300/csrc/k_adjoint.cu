@@ -36,9 +36,26 @@
 
 namespace avl {
 
+constexpr int AD_E_THREADS = 512;        // adjoint deposit block
+constexpr int AD_E_SMEM = 64 * 1024;     // and its copies of the grid
+constexpr int AD_PUSH_NX = 2048;         // largest field an FP32 push stages (8 KB)
+
+// a species' constants in the storage precision, computed once on the host:
+// an FP64 operation or conversion takes an SM's pipe as long as 64 FP32
+// instructions, and every thread would run a dozen of them for its few
+// markers
+template <typename T>
+struct AdjC {
+    T va, vb;        // velocity row: v va + vb
+    T qm_dt, dt_dx;
+    T lt;            // dt dv / dx: lambda_X dx to lambda_V dv
+    double c0;       // (q/m) dt / dv: deposit of lambda_V dv
+};
+
 // device-side view of the engine's buffers
 struct AdjSp {
     long long n;
+    int nv, mobile;
     int lat[2];
     unsigned long long seed;
     double jitter;
@@ -49,15 +66,19 @@ struct AdjSp {
     float* coff;
     void* cv;
     void* f;           // [n] marker values
-    void* lx;          // [n] lambda_X
-    void* lv;          // [n] lambda_V
+    void* lx;          // [n] lambda_X dx
+    void* lv;          // [n] lambda_V dv
     double* mu;        // [n] dJ / df_l
-    void* num;         // [nv][nx][2] deposit accumulator: (numerator, denominator) pairs
-    void* den;         // unused
-    void* hF;          // [K + 1][nv][nx] F = N / D per slot
-    void* hD;          // [K + 1][nv][nx] D per slot
-    void* AB;          // [nv][nx][2] grid adjoint (A, B) of the state being walked back
+    void* num;         // [nx][nv][2] deposit accumulator: (numerator, denominator) pairs
+    void* hF;          // [K + 1][nx][nv] F = N / D per slot
+    void* hD;          // [K + 1][nx][nv] D per slot
+    void* AB;          // [nx][nv][2] grid adjoint (A, B) of the state being walked back
+    void* dE;          // [nx] (q/m) dt dE / dv, dE from cell i to i + 1, of that state
+    AdjC<float> cf;
+    AdjC<double> cd;
 };
+__device__ __forceinline__ const AdjC<float>& adj_c(const AdjSp& a, float) { return a.cf; }
+__device__ __forceinline__ const AdjC<double>& adj_c(const AdjSp& a, double) { return a.cd; }
 
 struct AdjDev {
     int ns, theta_s, K;
@@ -107,23 +128,56 @@ struct APos<double> {
 // velocity dual row j0 and weight w of row j0 + 1 (t = (v - vmin)/dv - 1/2),
 // in the storage precision with one explicit fused multiply-add, so that
 // the deposit and the gather find the same row and weight
-template <typename T>
-__device__ __forceinline__ int vrow(T v, const SpDev& sp, T& w)
+__device__ __forceinline__ int vrow(float v, const AdjC<float>& c, int nv, float& w)
 {
-    const T a = (T)sp.inv_dv[0], b = (T)(-sp.vmin[0] * sp.inv_dv[0] - 0.5);
-    T t;
-    if constexpr (sizeof(T) == 4)
-        t = __fmaf_rn(v, a, b);
-    else
-        t = __fma_rn(v, a, b);
-    if (!(t > (T)-2 && t < (T)(sp.nv[0] + 1))) {
-        w = (T)0;
-        return t > (T)0 ? sp.nv[0] + 1 : -2;
+    const float t = __fmaf_rn(v, c.va, c.vb);
+    if (!(t > -2.f && t < (float)(nv + 1))) {
+        w = 0.f;
+        return t > 0.f ? nv + 1 : -2;
     }
-    const T fl = floor(t);
+    const float fl = floorf(t);
     w = t - fl;
     return (int)fl;
 }
+// FP64: the weight as a count of 2^-52, from t as a 64-bit count of 2^-52
+// rows (rows beyond 1023, which that does not hold, from the floor)
+__device__ __forceinline__ int vrow52(double v, const AdjC<double>& c, int nv, long long& w)
+{
+    const double t = __fma_rn(v, c.va, c.vb);
+    int j;
+    if (((__double2hiint(t) >> 20) & 0x7ff) < 1033) {   // |t| < 1024
+        const long long n = fx_count(t);
+        w = n & (FX_ONE - 1);
+        j = (int)(n >> 52);
+    } else {
+        const double fl = floor(t);
+        w = fx_count(t - fl);
+        j = t > 0.0 ? (int)fmin(fl, 1.0e9) : -2;
+    }
+    if (j < -1 || j > nv) {
+        w = 0;
+        return j < 0 ? -2 : nv + 1;
+    }
+    return j;
+}
+__device__ __forceinline__ int vrow(double v, const AdjC<double>& c, int nv, double& w)
+{
+    long long w52;
+    const int j = vrow52(v, c, nv, w52);
+    w = __longlong_as_double(0x3FF0000000000000ll | w52) - 1.0;
+    return j;
+}
+
+template <typename T>
+struct Pair2;
+template <>
+struct Pair2<float> {
+    using type = float2;
+};
+template <>
+struct Pair2<double> {
+    using type = double2;
+};
 
 // (numerator, denominator) of one cell in one reduction: a v2 FP32
 // reduction in the FP32 path, two FP64 ones in the FP64 path
@@ -163,148 +217,240 @@ __global__ void k_ad_init(const StepArgs* __restrict__ A, const AdjDev* __restri
     }
 }
 
-// deposit of the markers of slot `slot` (numerator and denominator of Eq. 4)
-template <typename T>
-__global__ void k_ad_dep(const StepArgs* __restrict__ A, const AdjDev* __restrict__ D, int slot, int all)   // all: the static list
+// Deposit of the markers of slot `slot` (numerator and denominator of Eq. 4).
+// The 32 markers of a warp are neighbours on the creation lattice (a few
+// velocity rows of one column) and stay together, so with the grid stored
+// column by column their reductions fall into a few sectors.  Bound by L2's
+// reductions: 1 M markers 18.5 us (27.5 with the grid stored by rows; with
+// both rows of a column in one 16-byte reduction where it is aligned 25, with
+// a warp's sums formed in shared memory first 36).
+__global__ void __launch_bounds__(256) k_ad_dep(const AdjDev* __restrict__ D, int nx, int slot, int all)   // all: the static list
 {
     const int s = all ? D->stat[blockIdx.y] : D->act[blockIdx.y];
-    const SpDev& sp = A->sp[s];
     const AdjSp& a = D->sp[s];
-    const int nx = sp.nx, nv = sp.nv[0];
-    T* acc = reinterpret_cast<T*>(a.num);
-    const T* f = reinterpret_cast<const T*>(a.f);
-    const T* vv = reinterpret_cast<const T*>(a.hv) + (size_t)slot * a.n;
+    const AdjC<float> C = a.cf;
+    const int nv = a.nv;
+    float* acc = reinterpret_cast<float*>(a.num);
+    const float* f = reinterpret_cast<const float*>(a.f);
+    const float* vv = reinterpret_cast<const float*>(a.hv) + (size_t)slot * a.n;
     for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < a.n; k += (long long)gridDim.x * blockDim.x) {
-        const PosM<T> p = APos<T>::load(a, slot, k);
-        int i0;
-        T wx;
-        p.cic(i0, wx);
-        int ia, ib;
+        int i0, ia, ib;
+        float wx, wv;
+        APos<float>::load(a, slot, k).cic(i0, wx);
         wrap_pair(i0, nx, ia, ib);
-        T wv;
-        const int j0 = vrow(vv[k], sp, wv);
-        const T fl = f[k];
+        const int j0 = vrow(vv[k], C, nv, wv);
+        const float fl = f[k];
 #pragma unroll
-        for (int cv = 0; cv < 2; ++cv) {
-            const int j = j0 + cv;
+        for (int q = 0; q < 4; ++q) {
+            const int j = j0 + (q >> 1);
             if (j < 0 || j >= nv) continue;
-            const T av = cv ? wv : (T)1 - wv;
-            const T a0 = ((T)1 - wx) * av, a1 = wx * av;
-            pair_add(acc + 2 * ((size_t)j * nx + ia), a0 * fl, a0);
-            pair_add(acc + 2 * ((size_t)j * nx + ib), a1 * fl, a1);
+            const float w = (q & 1 ? wx : 1.f - wx) * (q >> 1 ? wv : 1.f - wv);
+            pair_add(acc + 2 * ((size_t)(q & 1 ? ib : ia) * nv + j), w * fl, w);
+        }
+    }
+}
+
+// FP64: a warp sums its contributions in a patch of shared memory (columns x
+// rows around its markers' footprints), weights and sums in integers
+// (fixed.cuh), values in units of the warp's largest, and adds every cell of
+// the patch to the grid: 20 to 60 reductions of (numerator, denominator)
+// where the markers have 128 corners.  Lattice neighbours share footprints in
+// fours; four copies of the patch by lane keep them off one another's words.
+// A warp whose patch does not fit (or with values that are not finite) adds
+// every corner to the grid.  1 M markers: 75 -> 34 us (one copy 54).
+constexpr int AD_PATCH = 160;   // words of a warp's patch and its copies
+__global__ void __launch_bounds__(256, 5) k_ad_depx(const AdjDev* __restrict__ D, int nx, int slot, int all)
+{
+    __shared__ unsigned long long patch_s[8][2 * AD_PATCH];
+    const int s = all ? D->stat[blockIdx.y] : D->act[blockIdx.y];
+    const AdjSp& a = D->sp[s];
+    const AdjC<double> C = a.cd;
+    const int nv = a.nv, lane = threadIdx.x & 31;
+    unsigned long long* Pn = patch_s[threadIdx.x >> 5];
+    unsigned long long* Pd = Pn + AD_PATCH;
+    double* acc = reinterpret_cast<double*>(a.num);
+    const double* f = reinterpret_cast<const double*>(a.f);
+    const double* vv = reinterpret_cast<const double*>(a.hv) + (size_t)slot * a.n;
+    const long long n_pad = (a.n + 31) / 32 * 32;   // whole warps iterate together
+    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n_pad; k += (long long)gridDim.x * blockDim.x) {
+        bool ok = k < a.n;
+        int i0 = 0, j0 = -2, e = 0;
+        long long u = 0, w = 0, mant = 0;
+        double fl = 0.0;
+        if (ok) {
+            const long long U = APos<double>::load(a, slot, k).X - (FX_ONE >> 1);
+            i0 = (int)(U >> 52);
+            u = (U & (FX_ONE - 1)) << 5;
+            j0 = vrow52(vv[k], C, nv, w);
+            w <<= 5;
+            fl = f[k];
+            mant = fx_value(fl, e);
+        }
+        ok = ok && j0 >= -1 && j0 < nv;   // a corner on the grid
+        const unsigned any = __ballot_sync(0xffffffffu, ok);
+        if (!any) continue;
+        const int emax = __reduce_max_sync(0xffffffffu, max(e, FX_EMIN));   // (2047: not finite; sums of 32 take five more)
+        long long c[4];                   // weights of the corners, 2^-57
+        c[3] = fx_mul(fx_split(u), fx_split(w >> 1));
+        c[2] = w - c[3];
+        c[1] = u - c[3];
+        c[0] = (FX_ONE << 5) - u - c[2];
+        // the patch: columns relative to the first marker's (periodic), rows
+        const int ir = __shfl_sync(0xffffffffu, i0, __ffs(any) - 1);
+        int di = i0 - ir;
+        if (2 * di > nx) di -= nx;
+        if (2 * di < -nx) di += nx;
+        const int d0 = __reduce_min_sync(0xffffffffu, ok ? di : 0x3fffffff);
+        const int d1 = __reduce_max_sync(0xffffffffu, ok ? di : -0x3fffffff);
+        const int r0 = __reduce_min_sync(0xffffffffu, ok ? j0 : 0x3fffffff);
+        const int r1 = __reduce_max_sync(0xffffffffu, ok ? j0 : -0x3fffffff);
+        const int W = d1 - d0 + 2, H = r1 - r0 + 2;
+        if (W <= nx && H <= AD_PATCH && W * H <= AD_PATCH && emax < 2040) {
+            const int cs = W * H * 4 <= AD_PATCH ? 2 : 0;   // copies: 1 << cs
+            for (int q = lane; q < (W * H) << cs; q += 32) Pn[q] = Pd[q] = 0;
+            __syncwarp();
+            if (ok) {
+                const Limbs v = fx_split(mant >> min(emax - e, 63));
+                const int at = (di - d0) * H + j0 - r0, lc = lane & ((1 << cs) - 1);
+                const int cell[4] = {at, at + H, at + 1, at + H + 1};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int o = (cell[q] << cs) + lc;
+                    atomicAdd(Pn + o, (unsigned long long)fx_mul(fx_split(c[q]), v));
+                    atomicAdd(Pd + o, (unsigned long long)c[q]);
+                }
+            }
+            __syncwarp();
+            for (int q = lane; q < W * H; q += 32) {
+                long long sn = 0, sd = 0;
+                for (int t = 0; t < 1 << cs; ++t) {
+                    sn += (long long)Pn[(q << cs) + t];
+                    sd += (long long)Pd[(q << cs) + t];
+                }
+                const int col = q / H, j = r0 + q - col * H;
+                int x = ir + d0 + col;
+                x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
+                if (sd != 0 && j >= 0 && j < nv)
+                    pair_add(acc + 2 * ((size_t)x * nv + j), fx_scale(fx_double(sn), emax - 1079),
+                             fx_scale(fx_double(sd), -57));
+            }
+            __syncwarp();
+        } else if (ok) {
+            int ia, ib;
+            wrap_pair(i0, nx, ia, ib);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int j = j0 + (q >> 1);
+                if (j < 0 || j >= nv) continue;
+                const double cd = fx_scale(fx_double(c[q]), -57);
+                pair_add(acc + 2 * ((size_t)(q & 1 ? ib : ia) * nv + j), cd * fl, cd);
+            }
         }
     }
 }
 
 // F = N / D and D into slot `slot`, accumulators cleared; charge per column
-// (Eq. 14) added into rho
+// (Eq. 14) added into rho.  One warp per column and group of rows.
 template <typename T>
 __global__ void __launch_bounds__(256) k_ad_fin(const StepArgs* __restrict__ A, const AdjDev* __restrict__ D, int slot,
                                                 int all)
 {
-    __shared__ double col[8][32];
+    using P = typename Pair2<T>::type;
     const int s = all ? D->stat[blockIdx.y] : D->act[blockIdx.y];
     const SpDev& sp = A->sp[s];
     const AdjSp& a = D->sp[s];
-    const int nx = sp.nx, nv = sp.nv[0];
-    const int x = blockIdx.x * 32 + (threadIdx.x & 31), lr = threadIdx.x >> 5;
+    const int nx = sp.nx, nv = sp.nv[0], lane = threadIdx.x & 31;
+    const int x = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (x >= nx) return;
     const size_t cells = (size_t)nx * nv;
-    const int rg = (nv + gridDim.z - 1) / gridDim.z;   // rows of this block's group
-    const int jb = blockIdx.z * rg, je = min(nv, jb + rg);
-    T* acc = reinterpret_cast<T*>(a.num);
+    P* acc = reinterpret_cast<P*>(a.num);
     T* F = reinterpret_cast<T*>(a.hF) + (size_t)slot * cells;
     T* Dg = reinterpret_cast<T*>(a.hD) + (size_t)slot * cells;
     double r = 0.0;
-    if (x < nx) {
-        for (int j = jb + lr; j < je; j += 8) {
-            const size_t o = (size_t)j * nx + x;
-            const T n0 = acc[2 * o], d0 = acc[2 * o + 1];
-            const T fv = d0 > (T)0 ? n0 / d0 : (T)0;
-            F[o] = fv;
-            Dg[o] = d0;
-            acc[2 * o] = (T)0;
-            acc[2 * o + 1] = (T)0;
-            r += (double)fv;
+    for (int j = blockIdx.z * 32 + lane; j < nv; j += 32 * gridDim.z) {
+        const size_t o = (size_t)x * nv + j;
+        const P nd = acc[o];
+        T fv = (T)0;
+        if constexpr (sizeof(T) == 8) {
+            if (nd.y > 0.0) fv = fx_div(nd.x, nd.y);
+        } else {
+            if (nd.y > 0.f) fv = nd.x / nd.y;
         }
+        F[o] = fv;
+        Dg[o] = nd.y;
+        acc[o] = P{};
+        r += (double)fv;
     }
-    col[lr][threadIdx.x & 31] = r;
-    __syncthreads();
-    if (lr == 0 && x < nx) {
-        double t = 0.0;
-        for (int k = 0; k < 8; ++k) t += col[k][threadIdx.x];
-        atomicAdd(D->rho + x, sp.q * sp.dv[0] * t);
-    }
+    for (int q = 16; q; q >>= 1) r += __shfl_down_sync(0xffffffffu, r, q);
+    if (lane == 0) atomicAdd(D->rho + x, sp.q * sp.dv[0] * r);
 }
 
-// push (Sec. 2) from slot to slot + 1 with the field of slot; immobile
-// species are copied
+// push (Sec. 2) from slot to slot + 1 with the field of slot (`staged`: FP32
+// grids whose field fits a block's shared memory convert it once, not two
+// values per marker); immobile species are copied
 template <typename T>
-__global__ void k_ad_push(const StepArgs* __restrict__ A, const AdjDev* __restrict__ D, int slot)
+__global__ void __launch_bounds__(256) k_ad_push(const AdjDev* __restrict__ D, int nx, int slot, bool staged)
 {
+    extern __shared__ float Es[];
     const int s = D->act[blockIdx.y];
-    const SpDev& sp = A->sp[s];
     const AdjSp& a = D->sp[s];
-    const int nx = sp.nx;
+    const AdjC<T> C = adj_c(a, (T)0);
+    const bool mobile = a.mobile;
     const double* E = D->hE + (size_t)slot * nx;
+    if (staged) {
+        for (int i = threadIdx.x; i < nx; i += blockDim.x) Es[i] = (float)E[i];
+        __syncthreads();
+    }
+    auto field = [&](int i) { return staged ? (T)Es[i] : (T)E[i]; };
     const T* v0 = reinterpret_cast<const T*>(a.hv) + (size_t)slot * a.n;
     T* v1 = reinterpret_cast<T*>(a.hv) + (size_t)(slot + 1) * a.n;
-    const T qm_dt = (T)sp.qm_dt, dt_dx = (T)sp.dt_dx;
     for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < a.n; k += (long long)gridDim.x * blockDim.x) {
         PosM<T> p = APos<T>::load(a, slot, k);
         T v = v0[k];
-        if (sp.mobile) {
+        if (mobile) {
             int i0;
             T w;
             p.cic(i0, w);
             int ia, ib;
             wrap_pair(i0, nx, ia, ib);
-            const T El = ((T)1 - w) * (T)E[ia] + w * (T)E[ib];
-            v = v + qm_dt * El;
-            p.drift(v * dt_dx, nx);
+            const T Ea = field(ia);
+            v = fma(C.qm_dt, fma(w, field(ib) - Ea, Ea), v);
+            if constexpr (sizeof(T) == 8)
+                p.wrap((long long)((unsigned long long)p.X + (unsigned long long)fx_count(v * C.dt_dx)), nx);
+            else
+                p.drift(v * C.dt_dx, nx);
         }
         APos<T>::store(a, slot + 1, k, p);
         v1[k] = v;
     }
 }
 
-// adjoint deposit onto the x grid: e_i += lt (q/m) dt G_i(X) over the mobile
-// markers of slot (lt = lambda_V + dt lambda_X); at the final state e = dx E
-// per-warp partial sums of the adjoint deposit: FP32 in the FP32 path (native
-// shared-memory reductions), FP64 otherwise; one copy per warp keeps the
-// contention within a warp
+// Partial sums in the storage precision, in copies of the grid by lane (the
+// 32 markers of a warp are lattice neighbours and meet in one or two cells;
+// with one copy per warp their reductions ran one after the other: 1 M
+// markers FP64 124 -> 22 us, FP32 36 -> 11), es[i copies + lane mod copies], which also keeps the lanes'
+// banks apart.  The copies are summed in FP64 (FP32: float-float).
 template <typename T>
-struct EAcc {
-    using type = double;
-};
-template <>
-struct EAcc<float> {
-    using type = float;
-};
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_ad_e(const StepArgs* __restrict__ A, const AdjDev* __restrict__ D, int slot,
-                                              int terminal, int copies)
+__global__ void __launch_bounds__(AD_E_THREADS) k_ad_e(const AdjDev* __restrict__ D, int nx, double dx, int slot,
+                                                       int terminal, int copies)
 {
-    using S = typename EAcc<T>::type;
     extern __shared__ __align__(16) unsigned char es_raw[];
-    S* es = reinterpret_cast<S*>(es_raw);   // [8 warps][nx]
+    T* es = reinterpret_cast<T*>(es_raw);   // [nx][copies]
     const int s = D->act[blockIdx.y];
-    const SpDev& sp = A->sp[s];
     const AdjSp& a = D->sp[s];
-    const int nx = sp.nx;
     if (terminal) {
         if (blockIdx.y == 0 && blockIdx.x == 0)
-            for (int i = threadIdx.x; i < nx; i += blockDim.x) D->e[i] = sp.dx * D->hE[(size_t)slot * nx + i];
+            for (int i = threadIdx.x; i < nx; i += blockDim.x) D->e[i] = dx * D->hE[(size_t)slot * nx + i];
         return;
     }
-    if (!sp.mobile) return;
-    for (int i = threadIdx.x; i < copies * nx; i += blockDim.x) es[i] = (S)0;
+    if (!a.mobile) return;
+    for (int i = threadIdx.x; i < copies * nx; i += blockDim.x) es[i] = (T)0;
     __syncthreads();
-    S* ew = copies ? es + ((threadIdx.x >> 5) % copies) * nx : nullptr;
+    const int lc = copies ? (threadIdx.x & (copies - 1)) : 0;
     const T* lx = reinterpret_cast<const T*>(a.lx);
     const T* lv = reinterpret_cast<const T*>(a.lv);
-    const T c0 = (T)sp.qm_dt;
-    const T dt = (T)(sp.dt_dx * sp.dx);
+    const T clt = adj_c(a, (T)0).lt;
+    const double c0 = adj_c(a, (T)0).c0;
     for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < a.n; k += (long long)gridDim.x * blockDim.x) {
         const PosM<T> p = APos<T>::load(a, slot, k);
         int i0;
@@ -312,20 +458,28 @@ __global__ void __launch_bounds__(256) k_ad_e(const StepArgs* __restrict__ A, co
         p.cic(i0, w);
         int ia, ib;
         wrap_pair(i0, nx, ia, ib);
-        const T c = (lv[k] + dt * lx[k]) * c0;
+        const T c = fma(clt, lx[k], lv[k]);
+        const T cb = c * w, ca = c - cb;
         if (copies) {
-            atomicAdd(ew + ia, (S)(c * ((T)1 - w)));
-            atomicAdd(ew + ib, (S)(c * w));
+            atomicAdd(es + ia * copies + lc, ca);
+            atomicAdd(es + ib * copies + lc, cb);
         } else {   // grid too large for shared copies
-            atomicAdd(D->e + ia, (double)(c * ((T)1 - w)));
-            atomicAdd(D->e + ib, (double)(c * w));
+            atomicAdd(D->e + ia, c0 * (double)ca);
+            atomicAdd(D->e + ib, c0 * (double)cb);
         }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < nx && copies; i += blockDim.x) {
-        double t = 0.0;
-        for (int q = 0; q < copies; ++q) t += (double)es[q * nx + i];
-        if (t != 0.0) atomicAdd(D->e + i, t);
+        double t;
+        if constexpr (sizeof(T) == 4) {
+            ff sum{0.f, 0.f};
+            for (int q = 0; q < copies; ++q) ff_add(sum, es[i * copies + ((q + i) & (copies - 1))]);
+            t = (double)sum.hi + (double)sum.lo;
+        } else {
+            t = 0.0;
+            for (int q = 0; q < copies; ++q) t += es[i * copies + ((q + i) & (copies - 1))];
+        }
+        if (t != 0.0) atomicAdd(D->e + i, c0 * t);
     }
 }
 
@@ -337,75 +491,84 @@ __global__ void k_ad_grid(const StepArgs* __restrict__ A, const AdjDev* __restri
     const int s = D->act[blockIdx.y];
     const SpDev& sp = A->sp[s];
     const AdjSp& a = D->sp[s];
-    const int nx = sp.nx;
-    const size_t cells = (size_t)nx * sp.nv[0];
+    const int nx = sp.nx, nv = sp.nv[0];
+    const size_t cells = (size_t)nx * nv;
+    if (blockIdx.x == 0) {
+        const double* E = D->hE + (size_t)slot * nx;
+        const double c = adj_c(a, (T)0).c0;
+        for (int i = threadIdx.x; i < nx; i += blockDim.x)
+            reinterpret_cast<T*>(a.dE)[i] = (T)(c * (E[i + 1 == nx ? 0 : i + 1] - E[i]));
+    }
     const T* F = reinterpret_cast<const T*>(a.hF) + (size_t)slot * cells;
     const T* Dg = reinterpret_cast<const T*>(a.hD) + (size_t)slot * cells;
     T* ab = reinterpret_cast<T*>(a.AB);
     const double psi_c = -sp.q * sp.dv[0];
     for (size_t o = (size_t)blockIdx.x * blockDim.x + threadIdx.x; o < cells; o += (size_t)gridDim.x * blockDim.x) {
         const T d = Dg[o];
-        const T ps = (T)(psi_c * D->tmp[o % nx]);
-        const T A_ = d > (T)0 ? ps / d : (T)0;
+        const T ps = (T)(psi_c * D->tmp[cells >> 32 ? o / nv : (unsigned)o / (unsigned)nv]);
+        T A_;
+        if constexpr (sizeof(T) == 8)
+            A_ = d > (T)0 ? fx_div(ps, d) : (T)0;
+        else
+            A_ = d > (T)0 ? ps / d : (T)0;
         ab[2 * o] = A_;
         ab[2 * o + 1] = A_ * F[o];
     }
 }
 
-// per marker: mu += sum A alpha, lambda update (see the file head)
+// per marker: mu += sum A alpha, lambda update (see the file head; lambda_X
+// times dx and lambda_V times dv, so that no derivative is scaled).  A and
+// A f - B at the four corners (0 off the grid), the weights of rows and
+// columns in turn: 28 operations where the corners one by one took about 50,
+// on the FP64 pipe in the FP64 path.  Weighted sums, not interpolation by
+// differences: A = psi / D is largest where a corner's weight is smallest.
+// 1 M markers: FP64 102 -> 62 us, FP32 26 -> 16.
 template <typename T>
-__global__ void k_ad_gather(const StepArgs* __restrict__ A, const AdjDev* __restrict__ D, int slot, int terminal)
+__global__ void __launch_bounds__(256) k_ad_gather(const AdjDev* __restrict__ D, int nx, int slot, int terminal)
 {
+    using P = typename Pair2<T>::type;
     const int s = D->act[blockIdx.y];
-    const SpDev& sp = A->sp[s];
     const AdjSp& a = D->sp[s];
-    const int nx = sp.nx, nv = sp.nv[0];
-    const T* ab = reinterpret_cast<const T*>(a.AB);
-    const double* E = D->hE + (size_t)slot * nx;
+    const AdjC<T> C = adj_c(a, (T)0);
+    const int nv = a.nv;
+    const bool mobile = a.mobile;
+    const P* ab = reinterpret_cast<const P*>(a.AB);
+    const T* dE = reinterpret_cast<const T*>(a.dE);
     const T* vv = reinterpret_cast<const T*>(a.hv) + (size_t)slot * a.n;
     const T* f = reinterpret_cast<const T*>(a.f);
     T* lx = reinterpret_cast<T*>(a.lx);
     T* lv = reinterpret_cast<T*>(a.lv);
-    const T idx_ = (T)(1.0 / sp.dx), idv = (T)sp.inv_dv[0];
-    const T dt = (T)(sp.dt_dx * sp.dx);
-    const T qm_dt = (T)sp.qm_dt;
     for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < a.n; k += (long long)gridDim.x * blockDim.x) {
         const PosM<T> p = APos<T>::load(a, slot, k);
-        int i0;
-        T wxT;
-        p.cic(i0, wxT);
-        int ia, ib;
+        int i0, ia, ib;
+        T wx, wv;
+        p.cic(i0, wx);
         wrap_pair(i0, nx, ia, ib);
-        T wv;
-        const int j0 = vrow(vv[k], sp, wv);
-        const T wx = wxT, fl = f[k];
-        T m = 0, gx = 0, gv = 0;
-#pragma unroll
-        for (int cv = 0; cv < 2; ++cv) {
-            const int j = j0 + cv;
-            if (j < 0 || j >= nv) continue;
-            const T av = cv ? wv : (T)1 - wv, dav = cv ? idv : -idv;
-#pragma unroll
-            for (int cx = 0; cx < 2; ++cx) {
-                const int i = cx ? ib : ia;
-                const T ax = cx ? wx : (T)1 - wx, dax = cx ? idx_ : -idx_;
-                const size_t o = (size_t)j * nx + i;
-                const T Ac = ab[2 * o], Bc = ab[2 * o + 1];
-                m += Ac * ax * av;
-                const T cc = Ac * fl - Bc;
-                gx += cc * dax * av;
-                gv += cc * ax * dav;
-            }
+        const int j0 = vrow(vv[k], C, nv, wv);
+        const T fl = f[k];
+        P p00{}, p01{}, p10{}, p11{};   // (row, column)
+        if (j0 >= 0 && j0 < nv) {
+            p00 = ab[(size_t)ia * nv + j0];
+            p01 = ab[(size_t)ib * nv + j0];
         }
+        if (j0 + 1 >= 0 && j0 + 1 < nv) {
+            p10 = ab[(size_t)ia * nv + j0 + 1];
+            p11 = ab[(size_t)ib * nv + j0 + 1];
+        }
+        const T ux = (T)1 - wx, uv = (T)1 - wv;
+        const T m = uv * fma(wx, p01.x, ux * p00.x) + wv * fma(wx, p11.x, ux * p10.x);
+        const T c00 = fma(p00.x, fl, -p00.y), c01 = fma(p01.x, fl, -p01.y);
+        const T c10 = fma(p10.x, fl, -p10.y), c11 = fma(p11.x, fl, -p11.y);
+        const T gx = fma(wv, c11 - c10, uv * (c01 - c00));
+        const T gv = fma(wx, c11 - c01, ux * (c10 - c00));
         a.mu[k] += (double)m;
         if (terminal) {
             lx[k] = gx;
             lv[k] = gv;
-        } else if (sp.mobile) {
+        } else if (mobile) {
             const T lxk = lx[k];
-            const T lt = lv[k] + dt * lxk;
-            const T dEdx = (T)(E[ib] - E[ia]) * idx_;
-            lx[k] = lxk + lt * (qm_dt * dEdx) + gx;
+            const T lt = fma(C.lt, lxk, lv[k]);
+            lx[k] = fma(lt, dE[ia], lxk) + gx;
             lv[k] = lt + gv;
         }
     }
@@ -436,17 +599,20 @@ __global__ void __launch_bounds__(256) k_ad_theta(const StepArgs* __restrict__ A
         const double x = ((double)i + ((double)ia + 0.5 + J0) / px) * sp.dx;
         const double v = sp.vmin[0] + ((double)j + ((double)ib + 0.5 + J1) / pv) * sp.dv[0];
         const double mu = a.mu[m];
-        double pert = 1.0;
-        for (int q = 0; q < nm; ++q) pert += f0->amp[q] * cos(2.0 * M_PI * f0->mode[q] * x / L + f0->phase[q]);
-        double B = 0.0;
+        double B = 0.0, Mb[4], tb[4];
         for (int b = 0; b < nb; ++b) {
             const double sd = f0->beam_vth[b][0];
-            const double t = (v - f0->beam_u[b][0]) / sd;
-            const double Mb = f0->beam_n[b] * exp(-0.5 * t * t) / (sqrt(2.0 * M_PI) * sd);
-            B += Mb;
-            acc[nm + b] += mu * pert * Mb * t / sd;
+            tb[b] = (v - f0->beam_u[b][0]) / sd;
+            Mb[b] = f0->beam_n[b] * exp(-0.5 * tb[b] * tb[b]) / (sqrt(2.0 * M_PI) * sd);
+            B += Mb[b];
         }
-        for (int q = 0; q < nm; ++q) acc[q] += mu * B * cos(2.0 * M_PI * f0->mode[q] * x / L + f0->phase[q]);
+        double pert = 1.0;
+        for (int q = 0; q < nm; ++q) {
+            const double c = cos(2.0 * M_PI * f0->mode[q] * x / L + f0->phase[q]);
+            pert += f0->amp[q] * c;
+            acc[q] += mu * B * c;
+        }
+        for (int b = 0; b < nb; ++b) acc[nm + b] += mu * pert * Mb[b] * tb[b] / f0->beam_vth[b][0];
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int t = 0; t < nt; ++t) {
@@ -502,11 +668,11 @@ void adjoint_free(AdjEngine* E)
 
 static int grid_for(long long n) { return (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, 152ll * 8)); }
 
-// row groups of the finalize so that it spreads over the SMs
-static int fin_groups(const AdjEngine* E)
+// blocks of the finalize: eight columns and a group of rows each
+static dim3 fin_grid(const AdjEngine* E, int species)
 {
-    const int xb = (E->nx + 31) / 32;
-    return std::max(1, std::min(64, (2 * 152 + xb - 1) / xb));
+    const int xb = (E->nx + 7) / 8;
+    return dim3(xb, species, std::max(1, std::min(64, (4 * 152 + xb - 1) / xb)));
 }
 
 static long long nmax_active(const AdjEngine* E)
@@ -514,6 +680,16 @@ static long long nmax_active(const AdjEngine* E)
     long long nmax = 0;
     for (int k = 0; k < E->h.nact; ++k) nmax = std::max(nmax, E->n[E->h.act[k]]);
     return nmax;
+}
+
+template <typename T>
+static void launch_dep(const AdjEngine* E, long long nmax, int species, int slot, int all, cudaStream_t st)
+{
+    const dim3 g(grid_for(nmax), species);
+    if constexpr (sizeof(T) == 8)
+        k_ad_depx<<<g, 256, 0, st>>>(E->d, E->nx, slot, all);
+    else
+        k_ad_dep<<<g, 256, 0, st>>>(E->d, E->nx, slot, all);
 }
 
 // the Poisson solve of Eq. 6 (P rho; the backward pass applies it to e):
@@ -531,8 +707,8 @@ static cudaError_t recon_and_field(const StepArgs& h, const StepArgs* dA, AdjEng
 {
     cudaError_t e = cudaMemcpyAsync(E->h.rho, E->h.rho_static, (size_t)E->nx * 8, cudaMemcpyDeviceToDevice, st);
     if (e) return e;
-    k_ad_dep<T><<<dim3(grid_for(nmax_active(E)), E->h.nact), 256, 0, st>>>(dA, E->d, slot, 0);
-    k_ad_fin<T><<<dim3((E->nx + 31) / 32, E->h.nact, fin_groups(E)), 256, 0, st>>>(dA, E->d, slot, 0);
+    launch_dep<T>(E, nmax_active(E), E->h.nact, slot, 0, st);
+    k_ad_fin<T><<<fin_grid(E, E->h.nact), 256, 0, st>>>(dA, E->d, slot, 0);
     if ((e = cudaGetLastError())) return e;
     return solve(h, E->h.rho, E->h.hE + (size_t)slot * E->nx, E->nx, st);
 }
@@ -547,17 +723,18 @@ static cudaError_t static_charge(AdjEngine* E, const StepArgs* dA, cudaStream_t 
     for (int k = 0; k < E->h.nstat; ++k) nmax = std::max(nmax, E->n[E->h.stat[k]]);
     std::swap(E->h.rho, E->h.rho_static);   // k_ad_fin adds into D->rho
     if ((e = cudaMemcpyAsync(E->d, &E->h, sizeof(AdjDev), cudaMemcpyHostToDevice, st))) return e;
-    k_ad_dep<T><<<dim3(grid_for(nmax), E->h.nstat), 256, 0, st>>>(dA, E->d, 0, 1);
-    k_ad_fin<T><<<dim3((E->nx + 31) / 32, E->h.nstat, fin_groups(E)), 256, 0, st>>>(dA, E->d, 0, 1);
+    launch_dep<T>(E, nmax, E->h.nstat, 0, 1, st);
+    k_ad_fin<T><<<fin_grid(E, E->h.nstat), 256, 0, st>>>(dA, E->d, 0, 1);
     if ((e = cudaGetLastError())) return e;
     std::swap(E->h.rho, E->h.rho_static);
     return cudaMemcpyAsync(E->d, &E->h, sizeof(AdjDev), cudaMemcpyHostToDevice, st);
 }
 
 template <typename T>
-static cudaError_t push_slot(AdjEngine* E, const StepArgs* dA, int slot, cudaStream_t st)
+static cudaError_t push_slot(AdjEngine* E, int slot, cudaStream_t st)
 {
-    k_ad_push<T><<<dim3(grid_for(nmax_active(E)), E->h.nact), 256, 0, st>>>(dA, E->d, slot);
+    const bool staged = sizeof(T) == 4 && E->nx <= AD_PUSH_NX;
+    k_ad_push<T><<<dim3(grid_for(nmax_active(E)), E->h.nact), 256, staged ? E->nx * 4 : 0, st>>>(E->d, E->nx, slot, staged);
     return cudaGetLastError();
 }
 
@@ -567,13 +744,17 @@ static cudaError_t back_step(const StepArgs& h, const StepArgs* dA, AdjEngine* E
     const long long nmax = nmax_active(E);
     cudaError_t e = cudaMemsetAsync(E->h.e, 0, (size_t)E->nx * 8, st);
     if (e) return e;
-    const size_t copy_bytes = (size_t)E->nx * sizeof(typename EAcc<T>::type);
-    const int copies = (int)std::min<size_t>(8, (48 * 1024) / copy_bytes);
-    k_ad_e<T><<<dim3(grid_for(nmax), E->h.nact), 256, copies * copy_bytes, st>>>(dA, E->d, slot, terminal, copies);
+    const size_t copy_bytes = (size_t)E->nx * sizeof(T);
+    int copies = 32;
+    while (copies && copies * copy_bytes > AD_E_SMEM) copies >>= 1;
+    if ((e = raise_smem_limit(k_ad_e<T>, (int)(copies * copy_bytes)))) return e;
+    const int blocks = (int)std::min<long long>((nmax + AD_E_THREADS - 1) / AD_E_THREADS, sizeof(T) == 4 ? 304 : 152);
+    k_ad_e<T><<<dim3(blocks, E->h.nact), AD_E_THREADS, copies * copy_bytes, st>>>(E->d, E->nx, h.fd.dx, slot, terminal,
+                                                                                     copies);
     if ((e = cudaGetLastError())) return e;
     if ((e = solve(h, E->h.e, E->h.tmp, E->nx, st))) return e;
     k_ad_grid<T><<<dim3(152 * 2, E->h.nact), 256, 0, st>>>(dA, E->d, slot);
-    k_ad_gather<T><<<dim3(grid_for(nmax), E->h.nact), 256, 0, st>>>(dA, E->d, slot, terminal);
+    k_ad_gather<T><<<dim3(grid_for(nmax), E->h.nact), 256, 0, st>>>(E->d, E->nx, slot, terminal);
     return cudaGetLastError();
 }
 
@@ -584,7 +765,7 @@ static cudaError_t fwd_segment(const StepArgs& h, const StepArgs* dA, AdjEngine*
     cudaError_t e = cudaSuccess;
     for (int j = 0; j < len && !e; ++j) {
         e = recon_and_field<T>(h, dA, E, j, st);
-        if (!e && (push_last || j + 1 < len)) e = push_slot<T>(E, dA, j, st);
+        if (!e && (push_last || j + 1 < len)) e = push_slot<T>(E, j, st);
     }
     return e;
 }
@@ -760,8 +941,8 @@ cudaError_t adjoint_run(AdjEngine** eng, const StepArgs& h, const StepArgs* dA, 
             g(&q.lv, n * pb);
             g((void**)&q.mu, n * 8);
             g(&q.num, 2 * cells * pb);
-            q.den = nullptr;
             g(&q.AB, 2 * cells * pb);
+            g(&q.dE, nx * pb);
             g(&q.hF, (K + 1) * cells * pb);
             g(&q.hD, (K + 1) * cells * pb);
             if (!e) e = cudaMemsetAsync(q.num, 0, 2 * cells * pb, st);
@@ -798,6 +979,20 @@ cudaError_t adjoint_run(AdjEngine** eng, const StepArgs& h, const StepArgs* dA, 
         q.lat[1] = spec.lat[s][1];
         q.seed = spec.seed[s];
         q.jitter = spec.jitter[s];
+        const SpDev& sp = h.sp[s];
+        q.nv = sp.nv[0];
+        q.mobile = sp.mobile;
+        auto consts = [&](auto& c) {
+            using T = decltype(c.va + c.va);
+            c.va = (T)sp.inv_dv[0];
+            c.vb = (T)(-sp.vmin[0] * sp.inv_dv[0] - 0.5);
+            c.qm_dt = (T)sp.qm_dt;
+            c.dt_dx = (T)sp.dt_dx;
+            c.lt = (T)(sp.dt_dx * sp.dv[0]);
+            c.c0 = sp.qm_dt / sp.dv[0];
+        };
+        consts(q.cf);
+        consts(q.cd);
     }
     const int saveK = E->K;
     E->K = K;
