@@ -52,7 +52,6 @@ __device__ __forceinline__ Pos3<T> pos3_from_cells(double xi, int nx)
     return posm_from_cells<T>(xi, nx);
 }
 
-constexpr int MPT3 = 2;   // markers per thread and chunk
 
 __device__ __forceinline__ int species_of_pen(const StepArgs* A, int g)
 {
@@ -191,15 +190,15 @@ __device__ void block_exscan(const int* in, int* out, int n, int items, int* wsu
 // A pencil's markers are walked in chunks of at most NB markers, each inside
 // one segment; the marker fields of the next chunk are staged into shared
 // memory by bulk copies (TMA) while the current one is processed.
-template <typename T>
+// FP32: the fields are cell, offset, v_x, v_y, v_z, f.
 struct Stage3 {
-    static constexpr int NB = P3_THREADS * MPT3;              // markers per chunk
-    // staged fields: FP32 cell, offset, v_x, v_y, v_z, f; FP64 x, v_x, f (the
-    // (v_y, v_z) weights are stored beside the marker)
-    static constexpr int NF = sizeof(T) == 4 ? 6 : 3;
-    static constexpr int FVX = sizeof(T) == 4 ? 2 : 1;       // staged field of v_x
-    static constexpr int FF = NF - 1;                         // staged field of f
-    static constexpr int AL = 16 / (int)sizeof(T);           // markers per 16 bytes
+    // more than a segment of two markers per cell at nx = 256 (512, give or
+    // take its square root), so that few segments take a second chunk
+    static constexpr int NB = 640;
+    static constexpr int MPT = (NB + P3_THREADS - 1) / P3_THREADS;
+    static constexpr int NM = 64;                            // movers of a chunk kept in shared memory
+    static constexpr int NF = 6;
+    static constexpr int AL = 4;                             // markers per 16 bytes
     static constexpr int SLEN = NB + 2 * AL;                 // staged entries per field
 };
 
@@ -210,13 +209,17 @@ struct Stage3 {
 constexpr int NB3X = 640;
 constexpr int MPT3X = (NB3X + P3_THREADS - 1) / P3_THREADS;
 
+// x columns per thread of a pencil's block
+static int cpt_of(int nx) { return nx <= P3_THREADS ? 1 : (nx <= 2 * P3_THREADS ? 2 : 4); }
+
 size_t pd3_smem_bytes(int nx, int nkey, int prec)
 {
     size_t b;
     if (prec == AVL_FP32) {
-        using S = Stage3<float>;
+        using S = Stage3;
         b = 2 * (size_t)S::NF * S::SLEN * 4;                   // two staging buffers
-        b += 4 * (7 * (size_t)S::NB + nx);                     // sorted payload, E
+        b += 32 * (size_t)S::NB + 4 * ((size_t)nx + 2) + 64 * (size_t)S::NM;   // sorted payload, E, movers
+        b += 8 * (size_t)(P3_THREADS * cpt_of(nx) - nx);       // bins beyond nx
     } else {
         b = 5 * (NB3X + 4) * 8 + 96 * NB3X + 32;                  // staging (w_y, w_z, X, v_x, f), sorted payload
         b += 16 * (size_t)nx;                                  // kick
@@ -305,63 +308,93 @@ __device__ __forceinline__ void deposit_corner(float* gacc, int cells, const Pla
     atomicAdd(gacc + cells + o, a);
 }
 
-// exclusive scan of hist[0, nx) into start[0, nx], start[nx] = total; each
-// thread owns CPT consecutive bins and clears them for the next chunk
+// exclusive scan of hist[0, 256 CPT) into start[0, 256 CPT]: every warp sums
+// the bins in registers (8 CPT per lane) and writes its share, so that the
+// scan takes no barrier of its own
 template <int CPT>
-__device__ __forceinline__ void chunk_scan(int* hist, int* start, int nx, int* wsum)
+__device__ __forceinline__ void bin_scan(const int* hist, int* start)
 {
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int i0 = t * CPT;
-    int v[CPT], loc = 0;
+    constexpr int PER = 8 * CPT;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int v[PER], sum = 0;
 #pragma unroll
-    for (int i = 0; i < CPT; ++i) {
-        v[i] = i0 + i < nx ? hist[i0 + i] : 0;
-        loc += v[i];
+    for (int i = 0; i < PER; i += 4) {
+        const int4 h = reinterpret_cast<const int4*>(hist)[(lane * PER + i) / 4];
+        v[i] = h.x;
+        v[i + 1] = h.y;
+        v[i + 2] = h.z;
+        v[i + 3] = h.w;
+        sum += h.x + h.y + h.z + h.w;
     }
-    int incl = loc;
+    int incl = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += y;
     }
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    int pre = 0;
-    for (int w = 0; w < warp; ++w) pre += wsum[w];
-    int run = pre + incl - loc;
+    if ((lane >> 2) == warp) {   // a warp's share: 32 CPT bins of four lanes
+        int run = incl - sum;
 #pragma unroll
-    for (int i = 0; i < CPT; ++i) {
-        if (i0 + i < nx) {
-            start[i0 + i] = run;
-            hist[i0 + i] = 0;
+        for (int i = 0; i < PER; i += 4) {
+            const int4 b = make_int4(run, run + v[i], run + v[i] + v[i + 1], run + v[i] + v[i + 1] + v[i + 2]);
+            reinterpret_cast<int4*>(start)[(lane * PER + i) / 4] = b;
+            run = b.w + v[i + 3];
         }
-        run += v[i];
+        if (lane == 31) start[P3_THREADS * CPT] = run;
     }
-    if (i0 < nx && nx <= i0 + CPT) start[nx] = run;
-    __syncthreads();
 }
+
+// two FP32 values in one register pair: one packed instruction for both lanes
+// of a product or sum, each rounded as by itself
+using F2 = unsigned long long;
+__device__ __forceinline__ F2 f2_dup(float v)
+{
+    F2 r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float2 f2_get(F2 v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ void f2_fma(F2& c, F2 a, F2 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b)); }
 
 // mode 0: deposit of the current markers of every species (refresh);
 // mode 1: push of the mobile species, then deposit of the new state;
 // mode 2: deposit of the mobile species (pushed and re-sorted before).
 // PUSH (mode 1) is a template parameter so that the deposit-only instances
-// keep their own register budget (FP32, one column per thread: three CTAs
-// per SM with the push, four without).
+// keep their own registers (one column per thread: three CTAs per SM; four
+// without the push took 2.25 ms against 2.20, at 64 registers).
+//
+// Bound by the latency of its phases: 24 warps per SM, issue slots 46 % busy,
+// four barriers and 400 warp instructions per 32 markers, a quarter of them in
+// the gather, whose warps run as long as their fullest column (8 markers where
+// the mean is 4).  So: a chunk takes a whole segment (640 markers; at 512 half
+// of them took a second chunk), the bins are scanned by every warp without a
+// barrier of its own, the row of a finished segment leaves from the registers
+// of the gather, a marker's payload is two 16-byte words, the sums are packed
+// FP32 pairs (one instruction for two planes) and the pencil of a marker is
+// checked by comparing, not by taking the floor.  134 M markers, 256 x 64^3:
+// with the push 3.48 -> 2.70 ms, without 2.57 -> 2.11 ms.  Left out: the loop
+// over a column's markers run to the warp's longest with weights of zero
+// (2.80 ms; unrolled by two 2.82, by four 2.92), two markers at a time (2.87),
+// four CTAs per SM with the push (3.17, at 64 registers it spills).
 template <int CPT, bool PUSH>
-__global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? (PUSH ? 3 : 4) : (CPT == 2 ? 2 : 1))
+__global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 3 : (CPT == 2 ? 2 : 1))
     k_pd3(const StepArgs* __restrict__ A, int mode)
 {
     using T = float;
-    using S = Stage3<T>;
-    constexpr int MPT = MPT3;
-    constexpr int NB = S::NB, NF = S::NF, AL = S::AL, SLEN = S::SLEN;
-    constexpr int FVX = S::FVX, FF = S::FF;   // staged fields of v_x and f (FP32: v_y, v_z between)
+    using S = Stage3;
+    constexpr int MPT = S::MPT, NB = S::NB, NF = S::NF, AL = S::AL, SLEN = S::SLEN;
+    constexpr int FVX = 2, FF = 5;            // staged fields of v_x and f (v_y, v_z between)
+    constexpr int BINS = P3_THREADS * CPT;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint64_t bar[2];
-    __shared__ int wsum[P3_THREADS / 32];
     __shared__ unsigned long long mov_s, far_s;
     __shared__ int flag_s;
-    __shared__ int nmv_s;
+    __shared__ int nmv_s[2];
     __shared__ const void* src_s[6];
 
     const int g = blockIdx.x;
@@ -379,13 +412,15 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? (PUSH ? 3 : 4) : (CPT =
     T* const gacc = reinterpret_cast<T*>(sp.acc[ctl->asel[s]]);
     const int* segg = sp.seg[cb] + (size_t)p * (nkey + 1);
 
-    // shared memory: staging | payload (7 x NB) | E | hist | start | segment row
+    // shared memory: staging | payload (2 x 16 bytes x NB) | movers | hist | start | segment row | E
     T* stage = reinterpret_cast<T*>(smem);
-    T* pay = stage + 2 * NF * SLEN;
-    T* Es = pay + 7 * NB;
-    int* hist = reinterpret_cast<int*>(Es + nx);
-    int* start = hist + nx;
-    int* segs = start + nx + 1;
+    float4* pa = reinterpret_cast<float4*>(stage + 2 * NF * SLEN);   // u, f, w
+    float4* pq = pa + NB;                                            // weights of the four planes
+    float4* moved = pq + NB;                                         // movers by chunk parity, 2 x NM x (u, f, w, bin | w_y, w_z, j)
+    int* hist = reinterpret_cast<int*>(moved + 4 * S::NM);
+    int* start = hist + BINS;
+    int* segs = start + BINS + 1;
+    T* Es = reinterpret_cast<T*>(segs + nkey + 1);   // E of cells -1 .. nx
 
     if (threadIdx.x == 0) {
         mbar_init(&bar[0], 1);
@@ -394,7 +429,7 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? (PUSH ? 3 : 4) : (CPT =
         mov_s = 0;
         far_s = 0;
         flag_s = 0;
-        nmv_s = 0;
+        nmv_s[0] = nmv_s[1] = 0;
         src_s[0] = sp.mx[cb];
         src_s[1] = sp.moff[cb];
         src_s[FVX] = sp.mv[cb][0];
@@ -402,10 +437,9 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? (PUSH ? 3 : 4) : (CPT =
         src_s[FVX + 2] = sp.mv[cb][2];
         src_s[FF] = sp.mf[cb];
     }
-    for (int i = threadIdx.x; i < nx; i += P3_THREADS) {
-        hist[i] = 0;
-        if (push) Es[i] = A->fd.E32[i];
-    }
+    for (int i = threadIdx.x; i < BINS; i += P3_THREADS) hist[i] = 0;
+    if (push)
+        for (int i = threadIdx.x; i < nx + 2; i += P3_THREADS) Es[i] = A->fd.E32[i == 0 ? nx - 1 : (i > nx ? 0 : i - 1)];
     for (int i = threadIdx.x; i <= nkey; i += P3_THREADS) segs[i] = segg[i];
     __syncthreads();
 
@@ -446,13 +480,13 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? (PUSH ? 3 : 4) : (CPT =
         pl.base[q] = pl.ok[q] ? (kz * nvy + ky) * nvx * nx : 0;
     }
 
-    // register rows: Rm = row jseg - 1, R0 = row jseg, R1 = row jseg + 1;
-    // entry 2q: numerator, 2q + 1: denominator of plane q
-    T Rm[CPT][8], R0[CPT][8], R1[CPT][8];
+    // register rows: R0 = row jseg, R1 = row jseg + 1; pair h: numerators of
+    // planes 2h and 2h + 1, pair 2 + h: their denominators
+    F2 R0[CPT][4], R1[CPT][4];
 #pragma unroll
     for (int c = 0; c < CPT; ++c)
 #pragma unroll
-        for (int e = 0; e < 8; ++e) Rm[c][e] = R0[c][e] = R1[c][e] = (T)0;
+        for (int e = 0; e < 4; ++e) R0[c][e] = R1[c][e] = 0;
     unsigned long long nmov = 0, nfar = 0;
     int buf = 0;
     unsigned ph0 = 0, ph1 = 0;
@@ -462,25 +496,18 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? (PUSH ? 3 : 4) : (CPT =
         const int send = segs[k + 1];
         for (int b0 = segs[k]; b0 < send; b0 += NB) {
             const int cnt = min(NB, send - b0);
-            // stage the next chunk into the other buffer (free since the end of
-            // the previous chunk)
-            if (threadIdx.x == 0) {
-                int nk = k, nb = b0 + NB;
-                if (nb >= send) nk = first_from(k + 1, nb);
-                if (nk < nkey) issue(buf ^ 1, nb, min(NB, segs[nk + 1] - nb));
-            }
             const unsigned ph = buf ? ph1 : ph0;
             if (!mbar_wait_or_drain(&bar[buf], ph, wait_first, WAIT_LIMIT)) flag_s = 1;
             if (buf) ph1 ^= 1u; else ph0 ^= 1u;
             const T* st = stage + buf * NF * SLEN;
+            float4* const mv = moved + 2 * buf * S::NM;
             const int o0 = b0 & (AL - 1);
 
-            T pu[MPT], pw[MPT], pf[MPT], py[MPT], pz[MPT];
-            int pbin[MPT], prank[MPT];
+            T pu[MPT], pw[MPT], py[MPT], pz[MPT];
+            int pslot[MPT];   // x dual cell | place among its markers << 16
 #pragma unroll
             for (int m = 0; m < MPT; ++m) {
-                prank[m] = -1;
-                pbin[m] = 0;
+                pslot[m] = -1;
                 const int i = m * P3_THREADS + threadIdx.x;
                 if (i >= cnt) continue;
                 const int si = o0 + i;
@@ -493,137 +520,146 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? (PUSH ? 3 : 4) : (CPT =
                     int i0;
                     T wx;
                     pos.cic(i0, wx);
-                    int ia, ib;
-                    wrap_pair(i0, nx, ia, ib);
-                    const T El = ((T)1 - wx) * Es[ia] + wx * Es[ib];
+                    i0 = min(max(i0 + 1, 0), nx);
+                    const T El = ((T)1 - wx) * Es[i0] + wx * Es[i0 + 1];
                     vx = vx + qm_dt * El;
                     pos.drift(vx * dt_dx, nx);
                     reinterpret_cast<int*>(gx)[idx] = pos.c;
                     goff[idx] = pos.o;
                     gvx[idx] = vx;
                 }
-                const T f = st[FF * SLEN + si];
-                T wy = (T)0, wz = (T)0, w;
                 // the (v_y, v_z) dual cells, checked against the pencil
-                const int jy = dual3(st[(FVX + 1) * SLEN + si], vc.a[1], vc.b[1], vc.n[1], wy);
-                const int jz = dual3(st[(FVX + 2) * SLEN + si], vc.a[2], vc.b[2], vc.n[2], wz);
-                if (jy != pjy || jz != pjz) {
+                const T vy = st[(FVX + 1) * SLEN + si], vz = st[(FVX + 2) * SLEN + si];
+                const T ty = __fmaf_rn(vy, vc.a[1], vc.b[1]), tz = __fmaf_rn(vz, vc.a[2], vc.b[2]);
+                const T tx = __fmaf_rn(vx, vc.a[0], vc.b[0]);
+                const T wy = ty - (T)pjy, wz = tz - (T)pjz;
+                T w = tx - (T)jseg;
+                if (!(ty >= (T)pjy && ty < (T)(pjy + 1) && tz >= (T)pjz && tz < (T)(pjz + 1))) {
                     // outside the pencil only when the footprint misses the grid
+                    T d;
+                    const int jy = dual3(vy, vc.a[1], vc.b[1], vc.n[1], d), jz = dual3(vz, vc.a[2], vc.b[2], vc.n[2], d);
                     if (jy >= -1 && jy < nvy && jz >= -1 && jz < nvz) flag_s |= 2;
                     continue;
                 }
-                const int jx = dual3(vx, vc.a[0], vc.b[0], nvx, w);
-                if (jx < -1 || jx >= nvx) continue;
+                const bool stays = tx >= (T)jseg && tx < (T)(jseg + 1);
+                int jx = jseg;
+                if (!stays) {
+                    jx = dual3(vx, vc.a[0], vc.b[0], nvx, w);
+                    if (jx < -1 || jx >= nvx) continue;
+                }
                 int i0;
                 T u;
                 pos.cic(i0, u);
                 int bin = i0 < 0 ? i0 + nx : i0;
                 bin = min(max(bin, 0), nx - 1);
-                const int d = jx - jseg;
-                if (d == 0) {
-                    prank[m] = atomicAdd(&hist[bin], 1);
+                if (stays) {
+                    pslot[m] = bin | (atomicAdd(&hist[bin], 1) << 16);
                 } else {
-                    // off its segment's row: parked at the tail of the payload
-                    // arrays (the stays fill them from the front) and
-                    // deposited by the whole block after the sort
+                    // off its segment's row: kept for the whole block, which
+                    // deposits the chunk's few such markers after the sort
                     ++nmov;
-                    if (d > 1 || d < -1) ++nfar;
-                    const int o = NB - 1 - atomicAdd(&nmv_s, 1);
-                    pay[0 * NB + o] = u;
-                    pay[1 * NB + o] = w;
-                    pay[2 * NB + o] = f;
-                    pay[3 * NB + o] = wy;
-                    pay[4 * NB + o] = wz;
-                    pay[5 * NB + o] = (T)bin;
-                    pay[6 * NB + o] = (T)jx;
+                    if (jx > jseg + 1 || jx < jseg - 1) ++nfar;
+                    const T f = st[FF * SLEN + si];
+                    const int o = atomicAdd(&nmv_s[buf], 1);
+                    if (o < S::NM) {
+                        mv[2 * o] = make_float4(u, f, w, __int_as_float(bin));
+                        mv[2 * o + 1] = make_float4(wy, wz, __int_as_float(jx), 0.f);
+                    } else {
+#pragma unroll 1
+                        for (int c = 0; c < 16; ++c)
+                            deposit_corner(gacc, cells, pl, nx, nvx, bin, u, jx, w, wy, wz, f, c);
+                    }
                 }
-                pbin[m] = bin;
                 pu[m] = u;
                 pw[m] = w;
-                pf[m] = f;
                 py[m] = wy;
                 pz[m] = wz;
             }
             __syncthreads();
-            const int nmv = nmv_s;
-            // the parked markers: one thread per (marker, corner) into the global
-            // accumulator, so that a chunk's few movers do not hold one warp
-            // behind the others at the chunk's barrier
-            auto deposit_parked = [&]() {
-                for (int t = threadIdx.x; t < nmv * 16; t += P3_THREADS) {
-                    const int o = NB - 1 - (t >> 4);
-                    const int jx = (int)pay[6 * NB + o];
-                    deposit_corner(gacc, cells, pl, nx, nvx, (int)pay[5 * NB + o], pay[0 * NB + o], jx,
-                                      pay[1 * NB + o], pay[3 * NB + o], pay[4 * NB + o], pay[2 * NB + o], t & 15);
-                }
-            };
-            chunk_scan<CPT>(hist, start, nx, wsum);   // every thread has read nmv_s by its barriers
-            if (threadIdx.x == 0) nmv_s = 0;
+            // stage the next chunk into the other buffer (every thread is past
+            // the previous chunk's sort, which read it)
+            if (threadIdx.x == P3_THREADS - 32) {
+                nmv_s[buf ^ 1] = 0;
+                int nk = k, nb = b0 + NB;
+                if (nb >= send) nk = first_from(k + 1, nb);
+                if (nk < nkey) issue(buf ^ 1, nb, min(NB, segs[nk + 1] - nb));
+            }
+            const int nmv = min(nmv_s[buf], S::NM);
+            bin_scan<CPT>(hist, start);
+            __syncthreads();   // every warp has read the bins
+#pragma unroll
+            for (int c = 0; c < CPT; ++c) hist[threadIdx.x + c * P3_THREADS] = 0;
             // stays into x-sorted order
 #pragma unroll
             for (int m = 0; m < MPT; ++m) {
-                if (prank[m] < 0) continue;
-                const int o = start[pbin[m]] + prank[m];
+                if (pslot[m] < 0) continue;
+                const int o = start[pslot[m] & 0xffff] + (pslot[m] >> 16);
+                const T f = st[FF * SLEN + o0 + m * P3_THREADS + threadIdx.x];
                 T wq[4];
                 plane_weights(py[m], pz[m], wq);
-                pay[0 * NB + o] = pu[m];
-                pay[1 * NB + o] = pw[m];
-                pay[2 * NB + o] = pf[m];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) pay[(3 + q) * NB + o] = wq[q];
+                pa[o] = make_float4(pu[m], f, pw[m], 0.f);
+                pq[o] = make_float4(wq[0], wq[1], wq[2], wq[3]);
             }
             __syncthreads();
-            deposit_parked();
+            // the movers: one thread per (marker, corner) into the global
+            // accumulator, so that they do not hold one warp behind the others
+            for (int t = threadIdx.x ^ (P3_THREADS / 2); t < nmv * 16; t += P3_THREADS) {
+                const float4 a = mv[(t >> 4) * 2], b = mv[(t >> 4) * 2 + 1];
+                deposit_corner(gacc, cells, pl, nx, nvx, __float_as_int(a.w), a.x, __float_as_int(b.z), a.z, b.x, b.y, a.y,
+                               t & 15);
+            }
             // gather: column x takes weight u from the markers of dual cell
-            // x - 1 and 1 - u from those of dual cell x, which follow them in
-            // the sorted order (one loop; two at the periodic seam)
+            // x - 1 and 1 - u from those of dual cell x
 #pragma unroll
             for (int c = 0; c < CPT; ++c) {
                 const int x = threadIdx.x + c * P3_THREADS;
-                if (x >= nx) continue;
-                const int xm = x == 0 ? nx - 1 : x - 1;
-                const int mid = start[x];
-                const int lo0 = start[xm], hi0 = x == 0 ? start[nx] : mid;
-                const int hi1 = start[x + 1];
-                for (int pass = 0; pass < (x == 0 ? 2 : 1); ++pass) {
-                    const int lo = pass ? mid : lo0, hi = (x == 0 && !pass) ? hi0 : hi1;
-                    for (int i = lo; i < hi; ++i) {
-                        const T u = pay[i];
-                        const bool upper = x == 0 ? pass == 0 : i < mid;
-                        const T ax = upper ? u : (T)1 - u;
-                        const T a1 = ax * pay[NB + i];
-                        const T a0 = ax - a1;
-                        const T f = pay[2 * NB + i];
-                        const T f0 = a0 * f, f1 = a1 * f;
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const T wqv = pay[(3 + q) * NB + i];
-                            R0[c][2 * q] += f0 * wqv;
-                            R0[c][2 * q + 1] += a0 * wqv;
-                            R1[c][2 * q] += f1 * wqv;
-                            R1[c][2 * q + 1] += a1 * wqv;
-                        }
-                    }
+                int nup = 0, n = 0, up = 0, lo = 0;   // markers of x - 1, of both; k + up / k + lo their places
+                if (x < nx) {
+                    const int xm = x == 0 ? nx - 1 : x - 1, mid = start[x];
+                    up = start[xm];
+                    nup = start[xm + 1] - up;
+                    lo = mid - nup;
+                    n = nup + start[x + 1] - mid;
+                }
+#pragma unroll 1   // (unrolled, a warp's lanes part in the remainder: twice the iterations)
+                for (int k = 0; k < n; ++k) {
+                    const int i = k + (k < nup ? up : lo);
+                    const float4 m = pa[i];
+                    const ulonglong2 wq = *reinterpret_cast<const ulonglong2*>(pq + i);
+                    const float ax = k < nup ? m.x : 1.f - m.x;
+                    const float b1 = ax * m.z, b0 = ax - b1;
+                    const F2 a0 = f2_dup(b0), a1 = f2_dup(b1), f0 = f2_dup(b0 * m.y), f1 = f2_dup(b1 * m.y);
+                    f2_fma(R0[c][0], f0, wq.x);
+                    f2_fma(R0[c][1], f0, wq.y);
+                    f2_fma(R0[c][2], a0, wq.x);
+                    f2_fma(R0[c][3], a0, wq.y);
+                    f2_fma(R1[c][0], f1, wq.x);
+                    f2_fma(R1[c][1], f1, wq.y);
+                    f2_fma(R1[c][2], a1, wq.x);
+                    f2_fma(R1[c][3], a1, wq.y);
                 }
             }
-            __syncthreads();
             buf ^= 1;
         }
-        // row jseg - 1 is complete (no later segment reaches it): registers into
+        // row jseg is complete (no later segment reaches it): registers into
         // the global accumulator; then rotate the rows
-        const int row = jseg - 1;
-        if (row >= 0) {
+        if (jseg >= 0) {
 #pragma unroll
             for (int c = 0; c < CPT; ++c) {
                 const int x = threadIdx.x + c * P3_THREADS;
                 if (x >= nx) continue;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const T vn = Rm[c][2 * q], vd = Rm[c][2 * q + 1];
-                    if (pl.ok[q] && vd != (T)0) {
-                        const int o = pl.base[q] + row * nx + x;
-                        atomicAdd(gacc + o, vn);
-                        atomicAdd(gacc + cells + o, vd);
+                for (int h = 0; h < 2; ++h) {
+                    const float2 vn = f2_get(R0[c][h]), vd = f2_get(R0[c][2 + h]);
+                    T* const g0 = gacc + pl.base[2 * h] + jseg * nx + x;
+                    T* const g1 = gacc + pl.base[2 * h + 1] + jseg * nx + x;
+                    if (pl.ok[2 * h] && vd.x != 0.f) {
+                        atomicAdd(g0, vn.x);
+                        atomicAdd(g0 + cells, vd.x);
+                    }
+                    if (pl.ok[2 * h + 1] && vd.y != 0.f) {
+                        atomicAdd(g1, vn.y);
+                        atomicAdd(g1 + cells, vd.y);
                     }
                 }
             }
@@ -631,31 +667,10 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? (PUSH ? 3 : 4) : (CPT =
 #pragma unroll
         for (int c = 0; c < CPT; ++c)
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                Rm[c][e] = R0[c][e];
+            for (int e = 0; e < 4; ++e) {
                 R0[c][e] = R1[c][e];
-                R1[c][e] = (T)0;
+                R1[c][e] = 0;
             }
-        __syncthreads();
-    }
-    // the last row (nvx - 1) after the last segment
-    {
-        const int row = nvx - 1;
-#pragma unroll
-        for (int c = 0; c < CPT; ++c) {
-            const int x = threadIdx.x + c * P3_THREADS;
-            if (x >= nx) continue;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const T vn = Rm[c][2 * q];
-                const T vd = Rm[c][2 * q + 1];
-                if (pl.ok[q] && vd != (T)0) {
-                    const int o = pl.base[q] + row * nx + x;
-                    atomicAdd(gacc + o, vn);
-                    atomicAdd(gacc + cells + o, vd);
-                }
-            }
-        }
     }
 
     if (nmov) atomicAdd(&mov_s, nmov);
@@ -731,42 +746,6 @@ __device__ __forceinline__ int4 limbs2(long long a, long long b)
 {
     const Limbs A = fx_split(a), B = fx_split(b);
     return make_int4(A.h, A.l, B.h, B.l);
-}
-
-// exclusive scan of hist[0, 256 CPT) into start[0, 256 CPT]: every warp sums
-// the bins in registers (8 CPT per lane) and writes its share, so that the
-// scan takes no barrier of its own
-template <int CPT>
-__device__ __forceinline__ void bin_scan(const int* hist, int* start)
-{
-    constexpr int PER = 8 * CPT;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int v[PER], sum = 0;
-#pragma unroll
-    for (int i = 0; i < PER; i += 4) {
-        const int4 h = reinterpret_cast<const int4*>(hist)[(lane * PER + i) / 4];
-        v[i] = h.x;
-        v[i + 1] = h.y;
-        v[i + 2] = h.z;
-        v[i + 3] = h.w;
-        sum += h.x + h.y + h.z + h.w;
-    }
-    int incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if ((lane >> 2) == warp) {   // a warp's share: 32 CPT bins of four lanes
-        int run = incl - sum;
-#pragma unroll
-        for (int i = 0; i < PER; i += 4) {
-            const int4 b = make_int4(run, run + v[i], run + v[i] + v[i + 1], run + v[i] + v[i + 1] + v[i + 2]);
-            reinterpret_cast<int4*>(start)[(lane * PER + i) / 4] = b;
-            run = b.w + v[i + 3];
-        }
-        if (lane == 31) start[P3_THREADS * CPT] = run;
-    }
 }
 
 // finished sums of a cell into the global accumulator, in units of 2^-57 and
@@ -1706,7 +1685,6 @@ __global__ void k_getf3(const T* __restrict__ fg, const T* __restrict__ dg, int 
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-static int cpt_of(int nx) { return nx <= P3_THREADS ? 1 : (nx <= 2 * P3_THREADS ? 2 : 4); }
 
 cudaError_t configure_vhs3(const StepArgs& h)
 {
