@@ -787,15 +787,29 @@ avl_status avl_create(const avl_domain* dom, const avl_species* spec, int32_t ns
         fin_base += sp.nfin;
         const size_t cells = (size_t)nx * sp.nvflat;
         const size_t nvk = (size_t)sp.nvflat;
-        void *pf, *pn, *po, *pr, *pd, *p1, *p2, *p3, *p4, *p5, *p6;
+        void *pf, *pn, *po, *pr, *pd, *p1, *p2, *p3, *p4, *p5, *p6, *pv2;
         if ((e = dalloc(c, &pf, cells * pb, true)) || (e = dalloc(c, &pn, cells * pb, true)) ||
             (e = dalloc(c, &po, 2 * cells * 8 + nvk * 8, true)) || (e = dalloc(c, &pr, (size_t)sp.nrq * nx * 8, true)) ||
             (e = dalloc(c, &pd, (size_t)sp.nfin * 4 * 8, true)) || (e = dalloc(c, &p1, nvk * 4, true)) ||
             (e = dalloc(c, &p2, nvk * 4, true)) || (e = dalloc(c, &p3, (nvk + 1) * 4, true)) ||
             (e = dalloc(c, &p4, nvk * 4, true)) || (e = dalloc(c, &p5, (size_t)nx * 4, true)) ||
-            (e = dalloc(c, &p6, (size_t)nx * 4, true))) {
+            (e = dalloc(c, &p6, (size_t)nx * 4, true)) || (e = dalloc(c, &pv2, nvk * pb, false))) {
             cuda_fail(c, e, "cudaMalloc(species)");
             return bail(AVL_ENOMEM);
+        }
+        sp.v2row = pv2;
+        std::vector<double> v2(nvk);
+        std::vector<float> v2f(nvk);
+        for (int j = 0; j < p.nv[0]; ++j) {
+            const double v = sp.vmin[0] + (j + 0.5) * sp.dv[0];
+            v2[j] = v * v;
+            v2f[j] = (float)v * (float)v;
+        }
+        e = cudaMemcpy(pv2, dom->precision == AVL_FP32 ? (const void*)v2f.data() : (const void*)v2.data(), nvk * pb,
+                       cudaMemcpyHostToDevice);
+        if (e) {
+            cuda_fail(c, e, "cudaMemcpy(v2)");
+            return bail(AVL_ECUDA);
         }
         sp.fgrid = pf;
         sp.ngrid = pn;

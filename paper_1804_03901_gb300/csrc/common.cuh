@@ -197,6 +197,43 @@ struct ff {
 };
 
 __device__ __forceinline__ void ff_add(ff& a, float x) { two_sum_add(a.hi, a.lo, x); }
+__device__ __forceinline__ void ff_add(ff& a, ff b)
+{
+    two_sum_add(a.hi, a.lo, b.hi);
+    a.lo = __fadd_rn(a.lo, b.lo);
+}
+
+// Sums of a finalize block, in the accumulators' own arithmetic (FP32 as
+// float-float): an FP64 addition or conversion costs a warp 64 clocks, and the
+// trees of N, W_kin and S, the conversions before them and v^2 of a row took
+// 31 per warp and row pair (now six additions per block warp, v^2 from a
+// table): k_fin1 at 512 x 1024 FP32 48 -> 33 us, 512 x 6600 FP64 114 -> 90,
+// 64 small runs 423 -> 340, k_fin3 at 100 x 24 x 20 x 18 FP64 53 -> 37.
+__device__ __forceinline__ void acc_add(ff& a, ff b) { ff_add(a, b); }
+__device__ __forceinline__ void acc_add(double& a, double b) { a += b; }
+__device__ __forceinline__ ff acc_xor(ff a, int o)
+{
+    return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
+__device__ __forceinline__ double acc_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+// the warp's sums of a, b and c, in lanes 0, 8 and 16: half the lanes go on
+// with c, a quarter with b, so that three sums take six additions, not 15
+template <typename S>
+__device__ __forceinline__ S warp_sum3(S a, S b, S c)
+{
+    const int lane = threadIdx.x & 31;
+    const bool h = lane & 16, q = lane & 8;
+    S x = h ? c : a, y = h ? S{} : b;
+    acc_add(x, acc_xor(h ? a : c, 16));
+    acc_add(y, acc_xor(h ? b : S{}, 16));
+    S z = q ? y : x;
+    acc_add(z, acc_xor(q ? x : y, 8));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) acc_add(z, acc_xor(z, o));
+    return z;
+}
+__device__ __forceinline__ double acc_value(ff a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double acc_value(double a) { return a; }
 
 template <typename T>
 struct ColAcc;
@@ -211,13 +248,12 @@ struct ColAcc<float> {
         ff_add(w, __fmul_rn(v2, fh));
         if (fh > 0.f) ff_add(ent, __fmul_rn(fh, logf(fh)));
     }
-    __device__ __forceinline__ double r() const { return (double)rho.hi + (double)rho.lo; }
-    __device__ __forceinline__ double wk() const { return (double)w.hi + (double)w.lo; }
-    __device__ __forceinline__ double s() const { return (double)ent.hi + (double)ent.lo; }
+    using Sum = ff;
 };
 
 template <>
 struct ColAcc<double> {
+    using Sum = double;
     double rho = 0.0, w = 0.0, ent = 0.0;
     const longlong2* logtab = nullptr;
     __device__ __forceinline__ void add(double fh, double, double v2)

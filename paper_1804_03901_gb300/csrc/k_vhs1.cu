@@ -1089,8 +1089,9 @@ __global__ void __launch_bounds__(FIN_THREADS, 4) k_fin1(const StepArgs* __restr
                                                       const BatchMap* __restrict__ bm)
 {
     constexpr int RL = FIN_THREADS / FIN_XB;   // row lanes
-    __shared__ double col_red[RL][FIN_XB];
-    __shared__ double red[3][FIN_THREADS / 32];
+    using Sum = typename ColAcc<T>::Sum;
+    __shared__ Sum col_red[RL][FIN_XB];
+    __shared__ Sum red[3][FIN_THREADS / 32];
     __shared__ int clist[FIN_LIST];
     __shared__ int crow[FIN_LIST];
     __shared__ int ncl;
@@ -1159,6 +1160,7 @@ __global__ void __launch_bounds__(FIN_THREADS, 4) k_fin1(const StepArgs* __restr
 
     ColAcc<T> acc;
     if constexpr (sizeof(T) == 8) acc.logtab = A->fd.logtab;
+    const T* v2 = reinterpret_cast<const T*>(sp.v2row);
     // overflow rows, f = num / den, f and n stored, charge and diagnostics
     // (FP32: f_ref = the cell's f of the previous reconstruction, read before
     // it is overwritten; the deposit kernel staged the same value)
@@ -1174,8 +1176,7 @@ __global__ void __launch_bounds__(FIN_THREADS, 4) k_fin1(const StepArgs* __restr
         cs.value(fr, fh, fl, dsum);
         fg[(size_t)j * nx + x] = fh + fl;
         ng[(size_t)j * nx + x] = dsum;
-        const T vj = (T)(sp.vmin[0] + (j + 0.5) * sp.dv[0]);
-        acc.add(fh, fl, vj * vj);
+        acc.add(fh, fl, v2[j]);
     };
     if (xok && use_list) {
         // two rows at a time, the partials of their first WSLOT windows loaded
@@ -1240,39 +1241,25 @@ __global__ void __launch_bounds__(FIN_THREADS, 4) k_fin1(const StepArgs* __restr
         }
     }
     // charge of this species per column, summed over the row lanes in order
-    col_red[lr][col] = acc.r();
+    col_red[lr][col] = acc.rho;
     __syncthreads();
     if (lr == 0 && xok) {
-        double r = 0.0;
-        for (int k = 0; k < RL; ++k) r += col_red[k][col];
-        sp.rho_part[(size_t)rqi * nx + x] = sp.q * sp.dv[0] * r;
+        Sum r = col_red[0][col];
+        for (int k = 1; k < RL; ++k) acc_add(r, col_red[k][col]);
+        sp.rho_part[(size_t)rqi * nx + x] = sp.q * sp.dv[0] * acc_value(r);
     }
     // diagnostics of the block
-    double dN = acc.r(), dW = acc.wk(), dS = acc.s();
-    for (int o = 16; o > 0; o >>= 1) {
-        dN += __shfl_down_sync(0xffffffffu, dN, o);
-        dW += __shfl_down_sync(0xffffffffu, dW, o);
-        dS += __shfl_down_sync(0xffffffffu, dS, o);
-    }
+    const Sum d = warp_sum3(acc.rho, acc.w, acc.ent);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) {
-        red[0][warp] = dN;
-        red[1][warp] = dW;
-        red[2][warp] = dS;
-    }
+    if ((lane & 7) == 0 && lane < 24) red[lane >> 3][warp] = d;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0, bb = 0, cc = 0;
-        for (int w = 0; w < FIN_THREADS / 32; ++w) {
-            a += red[0][w];
-            bb += red[1][w];
-            cc += red[2][w];
-        }
+    if (threadIdx.x < 3) {   // N, W_kin, S
+        const int k = threadIdx.x;
+        Sum a = red[k][0];
+        for (int w = 1; w < FIN_THREADS / 32; ++w) acc_add(a, red[k][w]);
         const double cell = sp.dx * sp.dv[0];
-        sp.dpart[(size_t)blk * 4 + 0] = a * cell;
-        sp.dpart[(size_t)blk * 4 + 1] = 0.5 * sp.m * bb * cell;
-        sp.dpart[(size_t)blk * 4 + 2] = cc * cell;
-        sp.dpart[(size_t)blk * 4 + 3] = 0.0;
+        sp.dpart[(size_t)blk * 4 + k] = acc_value(a) * (k == 1 ? 0.5 * sp.m * cell : cell);
+        if (k == 0) sp.dpart[(size_t)blk * 4 + 3] = 0.0;
     }
 }
 

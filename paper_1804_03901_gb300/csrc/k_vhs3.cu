@@ -1104,8 +1104,9 @@ template <typename T>
 __global__ void __launch_bounds__(FIN3_X * FIN3_R) k_fin3(const StepArgs* __restrict__ A, int all_species)
 {
     constexpr int NT = FIN3_X * FIN3_R;
-    __shared__ double col_red[FIN3_R][FIN3_X];
-    __shared__ double red[3][NT / 32];
+    using Sum = typename ColAcc<T>::Sum;
+    __shared__ Sum col_red[FIN3_R][FIN3_X];
+    __shared__ Sum red[3][NT / 32];
     const int g = blockIdx.x;
     const int s = species_of_fin3(A, g);
     const SpDev& sp = A->sp[s];
@@ -1160,38 +1161,24 @@ __global__ void __launch_bounds__(FIN3_X * FIN3_R) k_fin3(const StepArgs* __rest
         }
     }
     const double dvol = sp.dv[0] * sp.dv[1] * sp.dv[2];
-    col_red[lr][col] = acc.r();
+    col_red[lr][col] = acc.rho;
     __syncthreads();
     if (lr == 0 && xok) {
-        double r = 0.0;
-        for (int k = 0; k < FIN3_R; ++k) r += col_red[k][col];
-        sp.rho_part[(size_t)rqi * nx + x] = sp.q * dvol * r;
+        Sum r = col_red[0][col];
+        for (int k = 1; k < FIN3_R; ++k) acc_add(r, col_red[k][col]);
+        sp.rho_part[(size_t)rqi * nx + x] = sp.q * dvol * acc_value(r);
     }
-    double dN = acc.r(), dW = acc.wk(), dS = acc.s();
-    for (int o = 16; o > 0; o >>= 1) {
-        dN += __shfl_down_sync(0xffffffffu, dN, o);
-        dW += __shfl_down_sync(0xffffffffu, dW, o);
-        dS += __shfl_down_sync(0xffffffffu, dS, o);
-    }
+    const Sum d = warp_sum3(acc.rho, acc.w, acc.ent);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) {
-        red[0][warp] = dN;
-        red[1][warp] = dW;
-        red[2][warp] = dS;
-    }
+    if ((lane & 7) == 0 && lane < 24) red[lane >> 3][warp] = d;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double n0 = 0, w0 = 0, s0 = 0;
-        for (int w = 0; w < NT / 32; ++w) {
-            n0 += red[0][w];
-            w0 += red[1][w];
-            s0 += red[2][w];
-        }
+    if (threadIdx.x < 3) {   // N, W_kin, S
+        const int k = threadIdx.x;
+        Sum t = red[k][0];
+        for (int w = 1; w < NT / 32; ++w) acc_add(t, red[k][w]);
         const double cell = sp.dx * dvol;
-        sp.dpart[(size_t)blk * 4 + 0] = n0 * cell;
-        sp.dpart[(size_t)blk * 4 + 1] = 0.5 * sp.m * w0 * cell;
-        sp.dpart[(size_t)blk * 4 + 2] = s0 * cell;
-        sp.dpart[(size_t)blk * 4 + 3] = 0.0;
+        sp.dpart[(size_t)blk * 4 + k] = acc_value(t) * (k == 1 ? 0.5 * sp.m * cell : cell);
+        if (k == 0) sp.dpart[(size_t)blk * 4 + 3] = 0.0;
     }
 }
 
