@@ -95,8 +95,33 @@ cudaError_t dalloc(avl_ctx* c, void** p, size_t bytes, bool zero)
     return e;
 }
 
+// SpConst of a species for its current grid, time step and magnetic field B
+template <typename T>
+static void fill_const(SpConst<T>& k, const SpDev& sp, const double (&B)[3])
+{
+    const double s = sizeof(T) == 8 ? 4503599627370496.0 : 1.0;
+    double t[3], t2 = 0.0;
+    for (int d = 0; d < 3; ++d) {
+        k.a[d] = (T)(sp.inv_dv[d] * s);
+        k.b[d] = (T)(std::fma(-sp.vmin[d], sp.inv_dv[d], -0.5) * s);
+        t[d] = 0.5 * sp.qm_dt * B[d];
+        t2 = std::fma(t[d], t[d], t2);
+    }
+    k.qm_dt = (T)sp.qm_dt;
+    k.dt_dx = (T)sp.dt_dx;
+    k.ba = (T)(0.5 * sp.qm_dt);
+    for (int d = 0; d < 3; ++d) {
+        k.bt[d] = (T)t[d];
+        k.bs[d] = (T)(2.0 / (1.0 + t2) * t[d]);
+    }
+}
+
 avl_status upload_args(avl_ctx* c)
 {
+    for (int s = 0; s < c->ns; ++s) {
+        fill_const(c->h.sp[s].cf, c->h.sp[s], c->h.fd.B);
+        fill_const(c->h.sp[s].cd, c->h.sp[s], c->h.fd.B);
+    }
     AVL_CUDA(c, cudaMemcpyAsync(c->d_args, &c->h, sizeof(StepArgs), cudaMemcpyHostToDevice, c->st));
     // the host copy must stay unchanged until the copy has run
     AVL_CUDA(c, cudaStreamSynchronize(c->st));

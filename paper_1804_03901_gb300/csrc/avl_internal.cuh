@@ -72,6 +72,18 @@ __host__ __device__ inline int win_plane(int W, int nx) { return (W * nx + 3) & 
 // device-side error bits (Ctl::err)
 enum : int { ERR_TIMEOUT = 1, ERR_NUMERIC = 2, ERR_CAPACITY = 4 };
 
+// a species' constants in the storage precision, filled by the host: every
+// thread of a kernel would take dozens of FP64 operations and conversions for
+// them, 64 clocks of its SM sub-partition each per warp
+template <typename T>
+struct SpConst {
+    T a[3], b[3];              // velocity row t = v a + b (FP64: times 2^52)
+    T qm_dt, dt_dx;
+    // Boris push: a = (q/m) dt / 2, t = a B (tangent of half the rotation
+    // angle along B), s = 2 t / (1 + |t|^2)
+    T ba, bt[3], bs[3];
+};
+
 struct SpDev {
     int nvdim, nx, nv[3], nvflat;
     int mobile;
@@ -80,6 +92,8 @@ struct SpDev {
     double vmin[3], dv[3], inv_dv[3];
     double dx;
     double qm_dt, dt_dx;       // (q/m) dt, dt/dx
+    SpConst<float> cf;
+    SpConst<double> cd;
     // chunks
     int M;                     // markers per chunk (multiple of 64)
     int nchunk;                // chunks (0: no markers)
@@ -124,11 +138,17 @@ struct SpDev {
     int pen_base;              // first global pencil block of this species
     int* seg[2];               // [npen][nkey + 1] first marker of every key, per buffer
     void* acc[2];              // [2][nvflat][nx] numerator, denominator of the deposit
-    void* v2row;               // [nvflat] |v|^2 at the centre of every velocity cell
+    void* v2row;               // [nvflat] |v|^2 at the centre of every velocity cell (storage precision)
     int* kcount;               // [npen * nkey] bucket counts (zero between operations)
     int* kcur;                 // [npen * nkey] slot cursors of a creation or global re-sort
     int* ktile;                // [ceil(npen * nkey / 1024)] bucket counts per scan tile
 };
+template <typename T>
+__host__ __device__ __forceinline__ const SpConst<T>& sp_const(const SpDev& sp)
+{
+    if constexpr (sizeof(T) == 4) return sp.cf;
+    else return sp.cd;
+}
 
 struct FieldDev {
     int nx, pow2, softening, ndiag;

@@ -262,9 +262,6 @@ struct ColAcc<double> {
         w += v2 * fh;
         if (__double_as_longlong(fh) > 0) ent += fh * fx_log(fh, logtab);   // fh > 0 (fh is not a NaN)
     }
-    __device__ __forceinline__ double r() const { return rho; }
-    __device__ __forceinline__ double wk() const { return w; }
-    __device__ __forceinline__ double s() const { return ent; }
 };
 
 // SplitMix64 (Steele, Lea & Flood 2014): output n of the generator seeded

@@ -83,7 +83,7 @@ __device__ __forceinline__ int dual3(float v, float a, float b, int n, float& w)
     w = t - fl;
     return (int)fl;
 }
-// FP64: a and b come scaled by 2^52 (dual_coef), so that t 2^52 rounds to a
+// FP64: a and b come scaled by 2^52, so that t 2^52 rounds to a
 // 64-bit count of 2^-52 rows in one saturating conversion (NaN gives 0); the
 // row is its high bits and the weight its low 52 bits
 __device__ __forceinline__ int dual3(double v, double a52, double b52, int n, long long& w)
@@ -107,24 +107,17 @@ struct DualW<double> {
     using type = long long;
 };
 
-// coefficients a, b of dual3 for dimension d of a species, in storage
-// precision (FP64: times 2^52)
-template <typename T>
-__device__ __forceinline__ void dual_coef(const SpDev& sp, int d, T& a, T& b)
-{
-    const double s = sizeof(T) == 8 ? 4503599627370496.0 : 1.0;
-    a = (T)(sp.inv_dv[d] * s);
-    b = (T)((-sp.vmin[d] * sp.inv_dv[d] - 0.5) * s);
-}
-
+// coefficients a, b of dual3 and cell counts of a species' velocity grid
 template <typename T>
 struct VCoef {
     T a[3], b[3];
     int n[3];
     __device__ __forceinline__ void init(const SpDev& sp)
     {
+        const SpConst<T>& k = sp_const<T>(sp);
         for (int d = 0; d < 3; ++d) {
-            dual_coef<T>(sp, d, a[d], b[d]);
+            a[d] = k.a[d];
+            b[d] = k.b[d];
             n[d] = sp.nv[d];
         }
     }
@@ -369,7 +362,7 @@ __device__ __forceinline__ void f2_fma(F2& c, F2 a, F2 b) { asm("fma.rn.f32x2 %0
 // without the push took 2.25 ms against 2.20, at 64 registers).
 //
 // Bound by the latency of its phases: 24 warps per SM, issue slots 46 % busy,
-// four barriers and 400 warp instructions per 32 markers, a quarter of them in
+// three barriers and 400 warp instructions per 32 markers, a quarter of them in
 // the gather, whose warps run as long as their fullest column (8 markers where
 // the mean is 4).  So: a chunk takes a whole segment (640 markers; at 512 half
 // of them took a second chunk), the bins are scanned by every warp without a
@@ -471,7 +464,7 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 3 : (CPT == 2 ? 2 : 1))
     float* const goff = sp.moff[cb];
     VCoef<T> vc;
     vc.init(sp);
-    const T qm_dt = (T)sp.qm_dt, dt_dx = (T)sp.dt_dx;
+    const T qm_dt = sp.cf.qm_dt, dt_dx = sp.cf.dt_dx;
     Planes pl;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -850,8 +843,7 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
         if (k0 < nkey) issue(b, min(NB, segs[k0 + 1] - b));
     }
 
-    double av, bv;
-    dual_coef<double>(sp, 0, av, bv);
+    const double av = sp.cd.a[0], bv = sp.cd.b[0];
     const double dt_dx52 = sp.dt_dx * PosX::ONE;   // dt / dx in 2^-52 cells
     Planes pl;
 #pragma unroll
@@ -1202,8 +1194,7 @@ __global__ void __launch_bounds__(P3_THREADS) k_sort3(const StepArgs* __restrict
     const int* sg = sp.seg[src] + (size_t)p * (nk + 1);
     int* dg = sp.seg[dst] + (size_t)p * (nk + 1);
     const int beg = sg[0], end = sg[nk];
-    T ax, bx;
-    dual_coef<T>(sp, 0, ax, bx);
+    const T ax = sp_const<T>(sp).a[0], bx = sp_const<T>(sp).b[0];
     const T* vxs = reinterpret_cast<const T*>(sp.mv[src][0]);
     for (int i = threadIdx.x; i < nk + 1; i += P3_THREADS) cnt[i] = 0;
     __syncthreads();
@@ -1330,6 +1321,19 @@ __device__ __forceinline__ int bucket3(const SpDev& sp, const VCoef<T>& vc, cons
     const int ky = key_of(dual3(v[1], vc.a[1], vc.b[1], vc.n[1], w), vc.n[1]);
     const int kz = key_of(dual3(v[2], vc.a[2], vc.b[2], vc.n[2], w), vc.n[2]);
     return (kz * (vc.n[1] + 1) + ky) * sp.nkey + kx;
+}
+
+// the same bucket and, FP64, the (v_y, v_z) weights as marker_wyz has them,
+// from the same conversions
+template <typename T>
+__device__ __forceinline__ int bucket3w(const VCoef<T>& vc, int nkey, const T (&v)[3], longlong2& wyz)
+{
+    typename DualW<T>::type w, wy, wz;
+    const int kx = key_of(dual3(v[0], vc.a[0], vc.b[0], vc.n[0], w), vc.n[0]);
+    const int jy = dual3(v[1], vc.a[1], vc.b[1], vc.n[1], wy), jz = dual3(v[2], vc.a[2], vc.b[2], vc.n[2], wz);
+    if constexpr (sizeof(T) == 8)
+        wyz = jy < -1 || jy >= vc.n[1] || jz < -1 || jz >= vc.n[2] ? make_longlong2(-1, -1) : make_longlong2(wy, wz);
+    return (key_of(jz, vc.n[2]) * (vc.n[1] + 1) + key_of(jy, vc.n[1])) * nkey + kx;
 }
 
 template <typename T, typename Src>
@@ -1477,49 +1481,50 @@ __global__ void __launch_bounds__(256) k_src3_scatter(const StepArgs* __restrict
 // ---------------------------------------------------------------------------
 // static background magnetic field: Boris push and global re-sort
 // ---------------------------------------------------------------------------
-// Boris coefficients of a species (storage precision): a = (q/m) dt / 2,
-// t = a B (tangent of half the rotation angle along B), s = 2 t / (1 + |t|^2)
 template <typename T>
-struct BorisCoef {
-    T a, t[3], s[3];
-    __device__ __forceinline__ void init(const SpDev& sp, const double (&B)[3])
-    {
-        const double a2 = 0.5 * sp.qm_dt;
-        double tt[3], t2 = 0.0;
-        for (int d = 0; d < 3; ++d) {
-            tt[d] = a2 * B[d];
-            t2 += tt[d] * tt[d];
-        }
-        const double f = 2.0 / (1.0 + t2);
-        a = (T)a2;
-        for (int d = 0; d < 3; ++d) {
-            t[d] = (T)tt[d];
-            s[d] = (T)(f * tt[d]);
-        }
-    }
+struct Vec2;
+template <>
+struct Vec2<float> {
+    using type = float2;
+};
+template <>
+struct Vec2<double> {
+    using type = double2;
 };
 
 // Boris push of every marker of species s in buffer cur, written back in
 // place: half kick by E_x at the old position, rotation v- -> v+ about B,
 // half kick, x += v_x dt.  The (pencil, key) bucket of the new velocities,
 // computed from the stored values exactly as the scatter recomputes it, is
-// counted into kcount (one atomic per distinct bucket of a warp).
+// counted into kcount (one atomic per distinct bucket of a warp).  The field
+// is staged as half kicks and their differences: 23 FP64 operations per marker
+// of the FP64 push where it took 28, and its constants come from the host (a
+// thread took 40 for its few markers): 2.6 M markers, 100 x 24 x 20 x 18, push
+// and re-sort 294 -> 234 us.
 template <typename T>
 __global__ void __launch_bounds__(256) k_bpush3(const StepArgs* __restrict__ A, int s)
 {
+    using T2 = typename Vec2<T>::type;
     extern __shared__ __align__(16) unsigned char smem[];
-    T* Es = reinterpret_cast<T*>(smem);
+    T2* Es = reinterpret_cast<T2*>(smem);   // half kick at the centre of cell i and its change to cell i + 1
     const SpDev& sp = A->sp[s];
     const int cb = A->ctl->cur[s];
     const int nx = sp.nx;
-    for (int i = threadIdx.x; i < nx; i += blockDim.x)
-        Es[i] = sizeof(T) == 4 ? (T)A->fd.E32[i] : (T)A->fd.E64[i];
+    const SpConst<T>& k0 = sp_const<T>(sp);
+    struct {
+        T a, t[3], s[3];
+    } bc = {k0.ba, {k0.bt[0], k0.bt[1], k0.bt[2]}, {k0.bs[0], k0.bs[1], k0.bs[2]}};
+    for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+        const int j = i + 1 == nx ? 0 : i + 1;
+        const T e0 = sizeof(T) == 4 ? (T)A->fd.E32[i] : (T)A->fd.E64[i], e1 = sizeof(T) == 4 ? (T)A->fd.E32[j] : (T)A->fd.E64[j];
+        Es[i].x = bc.a * e0;
+        Es[i].y = bc.a * (e1 - e0);
+    }
     __syncthreads();
-    BorisCoef<T> bc;
-    bc.init(sp, A->fd.B);
     VCoef<T> vc;
     vc.init(sp);
-    const T dt_dx = (T)sp.dt_dx;
+    const T dt_dx = k0.dt_dx;
+    const int nkey = sp.nkey;
     T* const g0 = reinterpret_cast<T*>(sp.mv[cb][0]);
     T* const g1 = reinterpret_cast<T*>(sp.mv[cb][1]);
     T* const g2 = reinterpret_cast<T*>(sp.mv[cb][2]);
@@ -1531,23 +1536,27 @@ __global__ void __launch_bounds__(256) k_bpush3(const StepArgs* __restrict__ A, 
         if (ok) {
             Pos3<T> pos;
             pos.load(sp, cb, (int)k);
-            int i0, ia, ib;
+            int i0;
             T wx;
             pos.cic(i0, wx);
-            wrap_pair(i0, nx, ia, ib);
-            const T aE = bc.a * (((T)1 - wx) * Es[ia] + wx * Es[ib]);
+            const T2 e = Es[(unsigned)i0 < (unsigned)nx ? i0 : nx - 1];
+            const T aE = fma(wx, e.y, e.x);
             const T m0 = g0[k] + aE, m1 = g1[k], m2 = g2[k];
             const T p0 = m0 + (m1 * bc.t[2] - m2 * bc.t[1]);
             const T p1 = m1 + (m2 * bc.t[0] - m0 * bc.t[2]);
             const T p2 = m2 + (m0 * bc.t[1] - m1 * bc.t[0]);
             const T v[3] = {m0 + (p1 * bc.s[2] - p2 * bc.s[1]) + aE, m1 + (p2 * bc.s[0] - p0 * bc.s[2]),
                             m2 + (p0 * bc.s[1] - p1 * bc.s[0])};
-            pos.drift(v[0] * dt_dx, nx);
+            if constexpr (sizeof(T) == 8)
+                pos.wrap((long long)((unsigned long long)pos.X + (unsigned long long)fx_count(v[0] * dt_dx)), nx);
+            else
+                pos.drift(v[0] * dt_dx, nx);
             pos.store(sp, cb, (int)k);
             g0[k] = v[0];
             g1[k] = v[1];
             g2[k] = v[2];
-            b = bucket3<T>(sp, vc, v);
+            longlong2 wyz;
+            b = bucket3w<T>(vc, nkey, v, wyz);
         }
         const int kk = ok ? b : -1;
         const unsigned grp = __match_any_sync(0xffffffffu, kk);
@@ -1559,8 +1568,10 @@ __global__ void __launch_bounds__(256) k_bpush3(const StepArgs* __restrict__ A, 
 // of buffer 1 - cur (k_src3_scan has placed the cursors).  A warp takes
 // RS3_ROUNDS x 32 consecutive markers: all loads first, then one slot per
 // round (a match on the bucket and one atomic per distinct bucket, all
-// rounds' atomics in flight together), then the stores.
-constexpr int RS3_ROUNDS = 4;
+// rounds' atomics in flight together), then the stores.  Bound by the latency
+// of its loads and atomics: 134 M FP32 markers, push and re-sort 2.82 ms with
+// four rounds, 2.70 with two (more warps per SM), 2.89 with one.
+constexpr int RS3_ROUNDS = 2;
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_rs3_scatter(const StepArgs* __restrict__ A, int s)
@@ -1574,12 +1585,14 @@ __global__ void __launch_bounds__(256) k_rs3_scatter(const StepArgs* __restrict_
     const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
     const long long n = sp.n;
+    const int nkey = sp.nkey;
     const T* f_src = reinterpret_cast<const T*>(sp.mf[src]);
     bool over = false;
     for (long long w0 = wid * 32 * RS3_ROUNDS; w0 < n; w0 += nw * 32 * RS3_ROUNDS) {
         T v[RS3_ROUNDS][3], fv[RS3_ROUNDS];
         Pos3<T> pos[RS3_ROUNDS];
         int b[RS3_ROUNDS];
+        longlong2 wyz[RS3_ROUNDS];
 #pragma unroll
         for (int r = 0; r < RS3_ROUNDS; ++r) {
             const long long k = w0 + r * 32 + lane;
@@ -1588,7 +1601,7 @@ __global__ void __launch_bounds__(256) k_rs3_scatter(const StepArgs* __restrict_
                 for (int d = 0; d < 3; ++d) v[r][d] = reinterpret_cast<const T*>(sp.mv[src][d])[k];
                 fv[r] = f_src[k];
                 pos[r].load(sp, src, (int)k);
-                b[r] = bucket3<T>(sp, vc, v[r]);
+                b[r] = bucket3w<T>(vc, nkey, v[r], wyz[r]);
             }
         }
         unsigned grp[RS3_ROUNDS];
@@ -1610,7 +1623,7 @@ __global__ void __launch_bounds__(256) k_rs3_scatter(const StepArgs* __restrict_
             pos[r].store(sp, dst, slot);
             for (int d = 0; d < 3; ++d) reinterpret_cast<T*>(sp.mv[dst][d])[slot] = v[r][d];
             reinterpret_cast<T*>(sp.mf[dst])[slot] = fv[r];
-            if constexpr (sizeof(T) == 8) sp.mwyz[dst][slot] = marker_wyz(vc, v[r][1], v[r][2]);
+            if constexpr (sizeof(T) == 8) sp.mwyz[dst][slot] = wyz[r];
         }
     }
     if (over) atomicOr(&A->ctl->err, ERR_CAPACITY);
@@ -1790,9 +1803,9 @@ cudaError_t launch_bpush3(const StepArgs& h, const StepArgs* d, int s, cudaStrea
     if (n == 0) return cudaSuccess;
     const int blocks = marker_blocks(n);
     if (h.prec == AVL_FP32)
-        k_bpush3<float><<<blocks, 256, (size_t)h.sp[s].nx * 4, st>>>(d, s);
+        k_bpush3<float><<<blocks, 256, (size_t)h.sp[s].nx * 8, st>>>(d, s);
     else
-        k_bpush3<double><<<blocks, 256, (size_t)h.sp[s].nx * 8, st>>>(d, s);
+        k_bpush3<double><<<blocks, 256, (size_t)h.sp[s].nx * 16, st>>>(d, s);
     return cudaGetLastError();
 }
 
