@@ -53,17 +53,8 @@ BYTES_PER_MARKER_ALGO = {(1, "fp32"): 20.0, (1, "fp64"): 40.0,    # 1d1v: read x
                          (3, "fp32"): 28.0, (3, "fp64"): 56.0,    # 1d3v: read x, vx, vy, vz, f; write x, vx
                          ("3B", "fp32"): 24.0, ("3B", "fp64"): 40.0}   # deposit only: read x, v, f
 BYTES_PER_MARKER_LAYOUT = {(1, "fp32"): 28.0, (1, "fp64"): 40.0,  # read all fields, write cell, off, dv in place
-                           (3, "fp32"): 36.0, (3, "fp64"): 64.0,  # read all fields, write cell, off, vx in place
+                           (3, "fp32"): 36.0, (3, "fp64"): 56.0,  # read all fields (FP64: X, vx, f and the stored (v_y, v_z) weights), write x, vx in place
                            ("3B", "fp32"): 24.0, ("3B", "fp64"): 40.0}
-# FP64 floating-point operations per marker of the 1d1v push + deposit (an FMA
-# counts 2): field gather (1 - w) E_a + w E_b 4, its CIC weight 2, kick 2,
-# drift 2, new CIC weights in x 2 and v 3, the four corner weights 6, the
-# numerator and denominator sums 12
-FP64_FLOPS_PER_MARKER = {1: 33.0}
-# FP64 FMA lanes per clock per SM on the GB300 (a warp's FP64 instruction
-# holds its SM sub-partition 64 clocks; four sub-partitions): an in-bounds
-# microbenchmark of dependent and independent FMA chains
-FP64_FMA_PER_SM_CLK = 2.0
 KERNEL_DESC = {1: "k_pd1 (gather + push + VHS deposit, written back in place)",
                3: "k_pd3 (gather + push + x-sorted VHS deposit per pencil, in place)",
                "3B": "k_pd3 mode 2 (x-sorted VHS deposit per pencil of the Boris-pushed, re-sorted markers)"}
@@ -205,8 +196,8 @@ def peaks():
     return 6800.0, "fallback"
 
 
-KERNEL_SOURCES = {1: ("k_vhs1.cu", "common.cuh", "resort.cuh", "ptx.cuh", "avl_internal.cuh"),
-                  3: ("k_vhs3.cu", "common.cuh", "avl_internal.cuh")}
+KERNEL_SOURCES = {1: ("k_vhs1.cu", "common.cuh", "fixed.cuh", "resort.cuh", "ptx.cuh", "avl_internal.cuh"),
+                  3: ("k_vhs3.cu", "common.cuh", "fixed.cuh", "avl_internal.cuh")}
 
 
 def kernel_source_hash(nvdim):
@@ -367,19 +358,6 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
-# FP64 floating-point operations per marker of the 1d3v push + deposit k_pd3
-# (an FMA counts 2; the weights of the marker's (v_y, v_z) cells are stored
-# beside it and not recomputed per step)
-def fp64_flops_3d():
-    push = 2 + 4 + 2 + 2          # CIC weight of x, field gather, kick, drift
-    weights = 2 + 3               # new CIC weight of x; dual row and weight of v_x
-    gather = 2 * (5 + 16 * 2)     # per column of the marker (two): ax, a1, a0, a0 f, a1 f; 16 FMAs into the rows
-    return float(push + weights + gather)
-
-
-FP64_FLOPS_PER_MARKER[3] = fp64_flops_3d()
-
-
 def measure(A, w, args, rank, world, local, stream):
     """Device-timed, profiled and end-to-end rates of one precision form of
     the workload, timed from the state after args.start_step (or half the
@@ -471,33 +449,20 @@ def measure(A, w, args, rank, world, local, stream):
     algo, lay = BYTES_PER_MARKER_ALGO[(kind, prec)], BYTES_PER_MARKER_LAYOUT[(kind, prec)]
     achieved = nmark * algo / (pd_ms / 1e3) / 1e9
     traffic_pm = recorded_traffic(w["name"], prec, nvd)
-    names = KERNEL_NAMES[kind]
-    hbm_entry = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
-                 "traffic": traffic_pm * nmark if traffic_pm else None,
-                 "kernel": KERNEL_DESC[kind],
-                 "algorithmic_bytes_per_marker": algo,
-                 "layout_bytes_per_marker": lay,
-                 "frac_layout_bytes": nmark * lay / (pd_ms / 1e3) / 1e9 / hbm,
-                 "peak_kind": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured" else peak_kind,
-                 "kernel_ms_per_step": {k: float(v / args.steps) for k, v in zip(names, kms)},
-                 "kernel_share": {k: float(v / kms.sum()) for k, v in zip(names, kms)}}
-    roofline = hbm_entry
-    if prec == "fp64" and kind in FP64_FLOPS_PER_MARKER:
-        # the FP64 form is bound by the FP64 pipe (a small fraction of the
-        # FP32 rate on this GPU): the same kernel against it
-        props = torch.cuda.get_device_properties(torch.cuda.current_device())
-        mhz = clk.get("sm_max_mhz") or clk.get("sm_mhz") or 2070.0
-        fpeak = FP64_FMA_PER_SM_CLK * 2.0 * props.multi_processor_count * mhz * 1e6 / 1e12
-        fach = nmark * FP64_FLOPS_PER_MARKER[kind] / (pd_ms / 1e3) / 1e12
-        roofline = {"bound": "alu", "achieved": fach, "peak": fpeak, "unit": "TFLOP/s", "frac": fach / fpeak,
-                    "traffic": hbm_entry["traffic"], "kernel": KERNEL_DESC[kind],
-                    "flops_per_marker": FP64_FLOPS_PER_MARKER[kind],
-                    "peak_kind": "FP64 pipe: 2 FMA lanes per clock per SM (in-bounds microbenchmark) x 2 FLOP x "
-                                 "SMs x the sampled maximum SM clock",
-                    "kernel_ms_per_step": hbm_entry["kernel_ms_per_step"],
-                    "kernel_share": hbm_entry["kernel_share"],
-                    "hbm": {k: hbm_entry[k] for k in ("achieved", "peak", "unit", "frac", "algorithmic_bytes_per_marker",
-                                                      "peak_kind")}}
+    # the FP64 push + deposit kernels (sums in 64-bit integers) have their own names
+    pd = {1: "k_pd1", 3: "k_pd3", "3B": "k_pd3"}[kind]
+    names, desc = KERNEL_NAMES[kind], KERNEL_DESC[kind]
+    if prec == "fp64":
+        names, desc = [pd + "x" if k == pd else k for k in names], desc.replace(pd, pd + "x", 1)
+    roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
+                "traffic": traffic_pm * nmark if traffic_pm else None,
+                "kernel": desc,
+                "algorithmic_bytes_per_marker": algo,
+                "layout_bytes_per_marker": lay,
+                "frac_layout_bytes": nmark * lay / (pd_ms / 1e3) / 1e9 / hbm,
+                "peak_kind": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured" else peak_kind,
+                "kernel_ms_per_step": {k: float(v / args.steps) for k, v in zip(names, kms)},
+                "kernel_share": {k: float(v / kms.sum()) for k, v in zip(names, kms)}}
     sim.close()
     return {"value": value, "ms_per_step": ms / args.steps, "dtype": "f32" if prec == "fp32" else "f64",
             "workload": w["name"], "markers": nmark, "start_step": start, "roofline": roofline, "clocks": clk,
