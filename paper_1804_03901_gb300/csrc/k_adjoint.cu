@@ -70,6 +70,7 @@ struct AdjSp {
     void* lv;          // [n] lambda_V dv
     double* mu;        // [n] dJ / df_l
     void* num;         // [nx][nv][2] deposit accumulator: (numerator, denominator) pairs
+    float* fref;       // FP32: [nx][nv] F of the initial state; numerators hold deviations from it
     void* hF;          // [K + 1][nx][nv] F = N / D per slot
     void* hD;          // [K + 1][nx][nv] D per slot
     void* AB;          // [nx][nv][2] grid adjoint (A, B) of the state being walked back
@@ -223,7 +224,8 @@ __global__ void k_ad_init(const StepArgs* __restrict__ A, const AdjDev* __restri
 // column by column their reductions fall into a few sectors.  Bound by L2's
 // reductions: 1 M markers 18.5 us (27.5 with the grid stored by rows; with
 // both rows of a column in one 16-byte reduction where it is aligned 25, with
-// a warp's sums formed in shared memory first 36).
+// a warp's sums formed in shared memory first 36), 19.7 with the numerators as
+// deviations from F_0 (k_ad_fin).
 __global__ void __launch_bounds__(256) k_ad_dep(const AdjDev* __restrict__ D, int nx, int slot, int all)   // all: the static list
 {
     const int s = all ? D->stat[blockIdx.y] : D->act[blockIdx.y];
@@ -232,6 +234,7 @@ __global__ void __launch_bounds__(256) k_ad_dep(const AdjDev* __restrict__ D, in
     const int nv = a.nv;
     float* acc = reinterpret_cast<float*>(a.num);
     const float* f = reinterpret_cast<const float*>(a.f);
+    const float* __restrict__ fref = a.fref;
     const float* vv = reinterpret_cast<const float*>(a.hv) + (size_t)slot * a.n;
     for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < a.n; k += (long long)gridDim.x * blockDim.x) {
         int i0, ia, ib;
@@ -245,7 +248,8 @@ __global__ void __launch_bounds__(256) k_ad_dep(const AdjDev* __restrict__ D, in
             const int j = j0 + (q >> 1);
             if (j < 0 || j >= nv) continue;
             const float w = (q & 1 ? wx : 1.f - wx) * (q >> 1 ? wv : 1.f - wv);
-            pair_add(acc + 2 * ((size_t)(q & 1 ? ib : ia) * nv + j), w * fl, w);
+            const size_t o = (size_t)(q & 1 ? ib : ia) * nv + j;
+            pair_add(acc + 2 * o, w * (fl - fref[o]), w);
         }
     }
 }
@@ -350,7 +354,10 @@ __global__ void __launch_bounds__(256, 5) k_ad_depx(const AdjDev* __restrict__ D
 }
 
 // F = N / D and D into slot `slot`, accumulators cleared; charge per column
-// (Eq. 14) added into rho.  One warp per column and group of rows.
+// (Eq. 14) added into rho.  One warp per column and group of rows.  FP32:
+// N holds sum alpha (f_l - F_0), F_0 the initial state's F, so F = F_0 + N / D
+// (Eq. 4 for any F_0) carries the rounding of f's change and of its spread in
+// a cell only; the charge is summed in float-float before F is rounded.
 template <typename T>
 __global__ void __launch_bounds__(256) k_ad_fin(const StepArgs* __restrict__ A, const AdjDev* __restrict__ D, int slot,
                                                 int all)
@@ -366,21 +373,28 @@ __global__ void __launch_bounds__(256) k_ad_fin(const StepArgs* __restrict__ A, 
     P* acc = reinterpret_cast<P*>(a.num);
     T* F = reinterpret_cast<T*>(a.hF) + (size_t)slot * cells;
     T* Dg = reinterpret_cast<T*>(a.hD) + (size_t)slot * cells;
-    double r = 0.0;
+    using Sum = typename ColAcc<T>::Sum;
+    Sum rs{};
     for (int j = blockIdx.z * 32 + lane; j < nv; j += 32 * gridDim.z) {
         const size_t o = (size_t)x * nv + j;
         const P nd = acc[o];
         T fv = (T)0;
         if constexpr (sizeof(T) == 8) {
             if (nd.y > 0.0) fv = fx_div(nd.x, nd.y);
+            rs += fv;
         } else {
-            if (nd.y > 0.f) fv = nd.x / nd.y;
+            if (nd.y > 0.f) {
+                const float f0 = a.fref[o], q = nd.x / nd.y;
+                ff_add(rs, f0);
+                ff_add(rs, q);
+                fv = f0 + q;
+            }
         }
         F[o] = fv;
         Dg[o] = nd.y;
         acc[o] = P{};
-        r += (double)fv;
     }
+    double r = acc_value(rs);
     for (int q = 16; q; q >>= 1) r += __shfl_down_sync(0xffffffffu, r, q);
     if (lane == 0) atomicAdd(D->rho + x, sp.q * sp.dv[0] * r);
 }
@@ -713,9 +727,15 @@ static cudaError_t recon_and_field(const StepArgs& h, const StepArgs* dA, AdjEng
     return solve(h, E->h.rho, E->h.hE + (size_t)slot * E->nx, E->nx, st);
 }
 
+// FP32: F of slot 0 becomes the reference of the numerators of species s
+static cudaError_t keep_reference(const StepArgs& h, AdjEngine* E, int s, cudaStream_t st)
+{
+    return cudaMemcpyAsync(E->h.sp[s].fref, E->h.sp[s].hF, (size_t)E->nx * h.sp[s].nv[0] * 4, cudaMemcpyDeviceToDevice, st);
+}
+
 // charge of the species that are not stepped (immobile, not theta): once
 template <typename T>
-static cudaError_t static_charge(AdjEngine* E, const StepArgs* dA, cudaStream_t st)
+static cudaError_t static_charge(const StepArgs& h, AdjEngine* E, const StepArgs* dA, cudaStream_t st)
 {
     cudaError_t e = cudaMemsetAsync(E->h.rho_static, 0, (size_t)E->nx * 8, st);
     if (e || E->h.nstat == 0) return e;
@@ -723,9 +743,15 @@ static cudaError_t static_charge(AdjEngine* E, const StepArgs* dA, cudaStream_t 
     for (int k = 0; k < E->h.nstat; ++k) nmax = std::max(nmax, E->n[E->h.stat[k]]);
     std::swap(E->h.rho, E->h.rho_static);   // k_ad_fin adds into D->rho
     if ((e = cudaMemcpyAsync(E->d, &E->h, sizeof(AdjDev), cudaMemcpyHostToDevice, st))) return e;
-    launch_dep<T>(E, nmax, E->h.nstat, 0, 1, st);
-    k_ad_fin<T><<<fin_grid(E, E->h.nstat), 256, 0, st>>>(dA, E->d, 0, 1);
-    if ((e = cudaGetLastError())) return e;
+    for (int pass = sizeof(T) == 4 ? 0 : 1; pass < 2; ++pass) {   // FP32: the reference first
+        launch_dep<T>(E, nmax, E->h.nstat, 0, 1, st);
+        k_ad_fin<T><<<fin_grid(E, E->h.nstat), 256, 0, st>>>(dA, E->d, 0, 1);
+        if ((e = cudaGetLastError())) return e;
+        if (pass) break;
+        for (int k = 0; k < E->h.nstat; ++k)
+            if ((e = keep_reference(h, E, E->h.stat[k], st))) return e;
+        if ((e = cudaMemsetAsync(E->h.rho, 0, (size_t)E->nx * 8, st))) return e;
+    }
     std::swap(E->h.rho, E->h.rho_static);
     return cudaMemcpyAsync(E->d, &E->h, sizeof(AdjDev), cudaMemcpyHostToDevice, st);
 }
@@ -858,7 +884,15 @@ static cudaError_t run(const StepArgs& h, const StepArgs* dA, AdjEngine* E, int 
         k_ad_init<T><<<grid_for(E->n[s]), 256, 0, st>>>(dA, E->d, s);
         if ((e = cudaGetLastError())) return e;
     }
-    if ((e = static_charge<T>(E, dA, st))) return e;
+    if constexpr (sizeof(T) == 4)
+        for (int s = 0; s < E->ns; ++s)
+            if ((e = cudaMemsetAsync(E->h.sp[s].fref, 0, (size_t)E->nx * h.sp[s].nv[0] * 4, st))) return e;
+    if ((e = static_charge<T>(h, E, dA, st))) return e;
+    if constexpr (sizeof(T) == 4) {
+        if ((e = recon_and_field<T>(h, dA, E, 0, st))) return e;
+        for (int k = 0; k < E->h.nact; ++k)
+            if ((e = keep_reference(h, E, E->h.act[k], st))) return e;
+    }
     if ((e = cudaMemsetAsync(E->h.grad, 0, 8 * (64 + 4), st))) return e;
     // forward: segments of K steps; checkpoint c = state c K
     const int nseg = std::max(1, (nsteps + K - 1) / K);
@@ -943,6 +977,8 @@ cudaError_t adjoint_run(AdjEngine** eng, const StepArgs& h, const StepArgs* dA, 
             g(&q.num, 2 * cells * pb);
             g(&q.AB, 2 * cells * pb);
             g(&q.dE, nx * pb);
+            q.fref = nullptr;
+            if (h.prec == AVL_FP32) g((void**)&q.fref, cells * 4);
             g(&q.hF, (K + 1) * cells * pb);
             g(&q.hD, (K + 1) * cells * pb);
             if (!e) e = cudaMemsetAsync(q.num, 0, 2 * cells * pb, st);
