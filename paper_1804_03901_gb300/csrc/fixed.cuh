@@ -9,10 +9,13 @@
 //   weights of a (column, v_x row) pair     2^-57     (FX_A)
 //   (v_y, v_z) cell weights                 2^-56     (FX_Q)
 //   marker values                           2^(el - 1078), el the exponent
-//                                           field of the column's largest value
+//                                           field of the largest value that
+//                                           reaches the row in the column
 //   sums of products                        h + m 2^-28 units of 2^-57
 // The low limbs are signed, so that the product of two of them, which is
-// left out, is at most a quarter of the sum's unit, of either sign.  Against
+// left out, is at most a quarter of the sum's unit, of either sign.  The units
+// are absolute, so what would reach a cell with a small weight only, and values
+// outside FX_EMIN .. FX_EMAX, are summed in FP64 instead (k_pd3x).  Against
 // exact rational sums of 4 to 12 markers with values over one e-fold: f
 // 7e-17 rms, weights 5e-17 (the same sums in FP64: 1.3e-16 and 1e-16).
 #pragma once
@@ -24,7 +27,8 @@ constexpr long long FX_ONE = 1ll << 52;       // 1 of a 52-bit fraction (positio
 constexpr int FX_LIMB = 28;
 constexpr int FX_PAIRS = 56;                  // products of weights <= 1 a sum takes before it is flushed:
                                               // |h| stays below 56 2^57 + 2^59, |m| below 56 (2^56 + 2^55)
-constexpr int FX_EMIN = 128;                  // smallest exponent of a column's unit: values below 2^-951 count as 0
+constexpr int FX_EMIN = 64, FX_EMAX = 2040;   // exponent fields of the values that the sums take: theirs (units of
+                                              // at least 2^-1015, magnitudes below 2^1024) are normal numbers
 
 // v = h 2^28 + l, -2^27 <= l < 2^27
 struct Limbs {
@@ -96,6 +100,9 @@ __device__ __forceinline__ long long fx_value(double f, int& e)
     return b < 0 ? -m : m;
 }
 
+// whether the sums take a value with exponent field e
+__device__ __forceinline__ bool fx_in_range(int e) { return e >= FX_EMIN && e <= FX_EMAX; }
+
 // t in counts of 2^-52, to nearest, without the FP64 pipe for |t| < 1024;
 // saturates, NaN gives 0
 __device__ __forceinline__ long long fx_count(double t)
@@ -121,6 +128,17 @@ __device__ __forceinline__ double fx_double(long long v)
     if (v < 0) r |= 0x8000000000000000ull;
     return __longlong_as_double((long long)r);
 }
+
+// lesser of a weight w (a count of 2^-52) and 1 - w, but 1 for w = 0, whose
+// corner takes nothing (at least 0 and less than 2^-32 below)
+__device__ __forceinline__ float lesser_weight(long long w)
+{
+    const unsigned a = (unsigned)(w >> 20);
+    return w == 0 ? 1.0f : (float)min(a, ~a) * 2.3283064365386963e-10f;   // 2^-32
+}
+
+// FP64 value of the weight of the next row or column, or of this one
+__device__ __forceinline__ double weight_of(long long w, bool next) { return fx_double(next ? w : FX_ONE - w); }
 
 // d 2^k for a normal result (d = 0 stays 0)
 __device__ __forceinline__ double fx_scale(double d, int k)

@@ -216,7 +216,7 @@ size_t pd3_smem_bytes(int nx, int nkey, int prec)
     } else {
         b = 5 * (NB3X + 4) * 8 + 96 * NB3X + 32;                  // staging (w_y, w_z, X, v_x, f), sorted payload
         b += 16 * (size_t)nx;                                  // kick
-        b += 12 * (size_t)nx + 8 * (size_t)P3_THREADS;         // exponents, bins beyond nx
+        b += 16 * (size_t)nx + 8 * (size_t)P3_THREADS;         // exponents, bins beyond nx
     }
     b += 4 * (2 * (size_t)nx + 1) + 4 * ((size_t)nkey + 2) + 64;   // histogram, bin starts, segment row
     return (b + 15) / 16 * 16;
@@ -703,24 +703,16 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 3 : (CPT == 2 ? 2 : 1))
 // a corner below SMALL3 = 2^-20 (0.5 % of markers at random places) is
 // deposited corner by corner with FP64 products instead, like a mover but not
 // counted as one, which leaves f and n within a few 2^-37 of those sums in
-// every cell (134 M markers, 256 x 64^3: the step 9.47 -> 9.71 ms).
+// every cell (134 M markers, 256 x 64^3: the step 9.47 -> 9.71 ms).  For the
+// same reason a row's values have a unit of its own, that of the largest value
+// that reaches the row in the column (one unit for both rows lost a row that
+// followed a much larger one: k_pd3x 8.54 -> 8.79 ms), and a value whose
+// exponent the sums do not hold goes with the small corners.
 constexpr float SMALL3 = 1.0f / (1 << 20);
-
-// lesser of a weight w (a count of 2^-52) and 1 - w, but 1 for w = 0, whose
-// corner takes nothing (at least 0 and less than 2^-32 below)
-__device__ __forceinline__ float lesser_weight(long long w)
-{
-    const unsigned a = (unsigned)(w >> 20);
-    return w == 0 ? 1.0f : (float)min(a, ~a) * 2.3283064365386963e-10f;   // 2^-32
-}
-
-// FP64 value of the weight of the next row or column, or of this one
-__device__ __forceinline__ double weight_of(long long w, bool next) { return fx_double(next ? w : FX_ONE - w); }
 
 struct FxCol {
     long long d0[4], v0[4];   // row jseg: weights, weighted values of the four planes
     long long d1[4], v1[4];   // row jseg + 1
-    int el;                   // the values' unit is 2^(el - 1078)
     int c0, c1;               // products in the sums of each row
 
     __device__ __forceinline__ void clear0()
@@ -735,24 +727,16 @@ struct FxCol {
         for (int q = 0; q < 4; ++q) d1[q] = v1[q] = 0;
         c1 = 0;
     }
-    // row jseg + 1 becomes row jseg; its unit shrinks as far as the sums
-    // allow (they stay below 2^59, which leaves room for FX_PAIRS products)
+    // row jseg + 1 becomes row jseg
     __device__ __forceinline__ void next_row()
     {
-        int room = el - FX_EMIN;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             d0[q] = d1[q];
             v0[q] = v1[q];
-            if (c1) room = min(room, __clzll(v0[q] < 0 ? ~v0[q] : v0[q]) - 5);
         }
         c0 = c1;
         clear1();
-        if (room >= 4) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) v0[q] <<= min(room, 63);
-            el -= room;
-        }
     }
 };
 
@@ -812,8 +796,9 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
     int* hist = reinterpret_cast<int*>(kick + nx);   // [256 CPT]
     int* start = hist + NT * CPT;                    // [256 CPT + 1]
     int* ebin = start + NT * CPT + 1;   // [2][nx] largest exponent field of a dual cell's values, by chunk parity
-    int* elc = ebin + 2 * nx;           // [nx] the columns' exponents (unit of the value sums) before this chunk
-    int* segs = elc + nx;
+    int* elc = ebin + 2 * nx;           // [nx] exponents el of a column's rows jseg (high half) and jseg + 1: their
+                                        // value sums are in units of 2^(el - 1078); [nx] what this chunk adds to them
+    int* segs = elc + 2 * nx;
 
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
@@ -826,6 +811,7 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
     }
     for (int i = threadIdx.x; i < nx; i += NT) {
         ebin[i] = ebin[nx + i] = 0;
+        elc[i] = FX_EMIN << 16 | FX_EMIN;
         // kick of a marker between the centres of cells i and i + 1 with
         // weight w of cell i + 1, as c + (1 + w) d (1 + w: the bits of the
         // position): E_i + w (E_i+1 - E_i), times (q/m) dt
@@ -882,7 +868,6 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
     for (int c = 0; c < CPT; ++c) {
         col[c].clear0();
         col[c].clear1();
-        col[c].el = FX_EMIN;
     }
 
     for (int k = 0; k < nkey; ++k) {
@@ -890,9 +875,6 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
         const int send = segs[k + 1];
         for (int b0 = segs[k]; b0 < send; b0 += NB) {
             const int cnt = min(NB, send - b0);
-#pragma unroll
-            for (int c = 0; c < CPT; ++c)
-                if (threadIdx.x + c * NT < nx) elc[threadIdx.x + c * NT] = col[c].el;
             if (!mbar_wait_or_drain(&bar, ph, wait_first, WAIT_LIMIT)) flag_s = 1;
             ph ^= 1u;
             const int o0 = b0 & (AL - 1);
@@ -930,16 +912,18 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
                 mw[m] = w;
                 pbin[m] = bin;
                 const double f = st_f[si];
+                const int ef = __double2hiint(f) >> 20 & 0x7ff;
                 const int d = jx - jseg;
                 const bool small =
                     lesser_weight(mu[m]) * lesser_weight(w) * (lesser_weight(wyz.x) * lesser_weight(wyz.y)) < SMALL3;
-                if (d == 0 && !small) {
+                if (d == 0 && !small && (fx_in_range(ef) | (((__double2hiint(f) & 0x7fffffff) | __double2loint(f)) == 0))) {
                     prank[m] = atomicAdd(&hist[bin], 1);
-                    atomicMax(&ebin[par * nx + bin], __double2hiint(f) >> 20 & 0x7ff);
+                    atomicMax(&ebin[par * nx + bin], ef);
                 } else {
-                    // off its segment's row, or a small corner: parked at the
-                    // tail of the payload arrays (the stays fill them from the
-                    // front) and deposited by the whole block after the sort
+                    // off its segment's row, a small corner or a value beyond
+                    // the sums' range: parked at the tail of the payload
+                    // arrays (the stays fill them from the front) and
+                    // deposited by the whole block after the sort
                     if (d != 0) ++nmov;
                     if (d > 1 || d < -1) ++nfar;
                     const int o = NB - 1 - atomicAdd(&nmv_s, 1);
@@ -951,6 +935,18 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
             __syncthreads();
             const int nmv = nmv_s;
             bin_scan<CPT>(hist, start);
+            // the columns' units: those of their rows before, or of the
+            // largest value of their two dual cells
+#pragma unroll
+            for (int c = 0; c < CPT; ++c) {
+                const int x = threadIdx.x + c * NT;
+                if (x >= nx) continue;
+                const int et = max(ebin[par * nx + (x == 0 ? nx - 1 : x - 1)], ebin[par * nx + x]);
+                const int el0 = elc[x] >> 16, el1 = elc[x] & 0xffff;
+                ebin[(par ^ 1) * nx + x] = 0;   // the next chunk's
+                elc[nx + x] = min(max(et - el0, 0), 63) << 16 | min(max(et - el1, 0), 63);
+                elc[x] = max(el0, et) << 16 | max(el1, et);
+            }
             __syncthreads();
             if (threadIdx.x == 0) nmv_s = 0;
             // the bins are counted into afresh after the next barrier
@@ -965,13 +961,14 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
                 plane_weights(st_w[si], q);
                 pqa[o] = limbs2(q[0], q[1]);
                 pqb[o] = limbs2(q[2], q[3]);
-                // value in the units of the two columns
-                const int bm = bin == 0 ? nx - 1 : bin - 1, bp = bin + 1 == nx ? 0 : bin + 1;
+                // value in the unit of row jseg + 1 of the two columns; that of
+                // row jseg, which holds the segment before too, is at least it
+                const int bp = bin + 1 == nx ? 0 : bin + 1;
                 int e;
                 const long long mant = fx_value(st_f[si], e);
-                const int* eb = ebin + par * nx;
-                const int e0 = max(elc[bin], max(eb[bm], eb[bin])), e1 = max(elc[bp], max(eb[bin], eb[bp]));
-                const Limbs f0 = fx_split(mant >> min(e0 - e, 63)), f1 = fx_split(mant >> min(e1 - e, 63));
+                const int u0 = elc[bin], u1 = elc[bp];
+                const int l0 = u0 & 0xffff, l1 = u1 & 0xffff, s0 = min((u0 >> 16) - l0, 63), s1 = min((u1 >> 16) - l1, 63);
+                const Limbs f0 = fx_split(mant >> min(l0 - e, 63)), f1 = fx_split(mant >> min(l1 - e, 63));
                 // weights in x and v_x: one product, the others by difference
                 // (none negative)
                 const long long u = mu[m] << 5, w = mw[m] << 5;
@@ -981,8 +978,8 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
                 const Limbs A00 = fx_split(a00), A01 = fx_split(a01), A10 = fx_split(a10), A11 = fx_split(a11);
                 pa[o] = make_int4(A00.h, A00.l, A01.h, A01.l);
                 pa[NB + o] = make_int4(A10.h, A10.l, A11.h, A11.l);
-                pg[o] = limbs2(fx_mul(A00, f0), fx_mul(A01, f0));
-                pg[NB + o] = limbs2(fx_mul(A10, f1), fx_mul(A11, f1));
+                pg[o] = limbs2(fx_mul(A00, f0) >> s0, fx_mul(A01, f0));
+                pg[NB + o] = limbs2(fx_mul(A10, f1) >> s1, fx_mul(A11, f1));
             }
             __syncthreads();
             // the staging buffer is free: the next chunk into it
@@ -1022,18 +1019,15 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
                 const int xm = x == 0 ? nx - 1 : x - 1;
                 const int lo = start[xm], nup = start[xm + 1] - lo;
                 const int blo = start[x] - nup, n = nup + start[x + 1] - start[x];
-                ebin[(par ^ 1) * nx + x] = 0;   // the next chunk's
                 if (n == 0) continue;
-                const int et = max(C.el, max(ebin[par * nx + xm], ebin[par * nx + x]));
-                const int sh = min(et - C.el, 63);
-                C.el = et;
+                const int sh0 = elc[nx + x] >> 16, sh1 = elc[nx + x] & 0xffff;
                 FxSum d0[4], v0[4], d1[4], v1[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     d0[q].h = C.d0[q];
-                    v0[q].h = C.v0[q] >> sh;
+                    v0[q].h = C.v0[q] >> sh0;
                     d1[q].h = C.d1[q];
-                    v1[q].h = C.v1[q] >> sh;
+                    v1[q].h = C.v1[q] >> sh1;
                     d0[q].m = v0[q].m = d1[q].m = v1[q].m = 0;
                 }
                 for (int r = 0; r < n;) {
@@ -1042,8 +1036,8 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             const int o = pl.base[q] + jseg * nx + x;
-                            add_sums(d0[q].units(), v0[q].units(), et, gacc, cells, pl.ok[q] && jseg >= 0, o);
-                            add_sums(d1[q].units(), v1[q].units(), et, gacc, cells, pl.ok[q] && jseg + 1 < nvx, o + nx);
+                            add_sums(d0[q].units(), v0[q].units(), elc[x] >> 16, gacc, cells, pl.ok[q] && jseg >= 0, o);
+                            add_sums(d1[q].units(), v1[q].units(), elc[x] & 0xffff, gacc, cells, pl.ok[q] && jseg + 1 < nvx, o + nx);
                             d0[q].clear();
                             v0[q].clear();
                             d1[q].clear();
@@ -1088,12 +1082,15 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
 #pragma unroll
         for (int c = 0; c < CPT; ++c) {
             const int x = threadIdx.x + c * NT;
-            if (x < nx && jseg >= 0 && col[c].c0) {
+            if (x >= nx) continue;
+            if (jseg >= 0 && col[c].c0) {
+                const int el = elc[x] >> 16;
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                    add_sums(col[c].d0[q], col[c].v0[q], col[c].el, gacc, cells, pl.ok[q], pl.base[q] + jseg * nx + x);
+                    add_sums(col[c].d0[q], col[c].v0[q], el, gacc, cells, pl.ok[q], pl.base[q] + jseg * nx + x);
             }
             col[c].next_row();
+            elc[x] = elc[x] << 16 | FX_EMIN;
         }
     }
     // (the last segment is row nvx - 1; what is left belongs to row nvx, off the grid)

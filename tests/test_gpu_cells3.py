@@ -76,3 +76,48 @@ def test_lone_markers(B):
         # over weights of 1e-6
         compare(sim, orc, 1e-10, 1e-7)
     sim.close()
+
+
+@pytest.mark.parametrize("where", ["vx up", "vx down", "x"])
+@pytest.mark.parametrize("fall", [1e6, 1e18])
+def test_steep_values(where, fall):
+    """f falls by `fall` from one v_x row or one x column to the next."""
+    sim, orc = simulation()
+    rng = np.random.default_rng(5)
+    n = 30000
+    x = dyadic(rng.uniform(0.0, 16.0, n))
+    v = dyadic(np.array([rng.uniform(-8.0, 4.0, n), rng.uniform(-2.0, 2.0, n), rng.uniform(-2.0, 2.0, n)]))
+    at = np.floor(x) if where == "x" else np.floor(v[0]) if where == "vx up" else -np.floor(v[0])
+    f = fall ** (at / 1.0 - at.max()) * rng.uniform(0.5, 2.0, n)
+    sim.set_markers(0, x, v, f)
+    orc.set_markers(0, x, v, f)
+    orc.refresh()
+    # the unit of a column's sums is 2^-56 of the largest value, which reaches the
+    # cell with a weight of at least 2^-20: some 20 markers of 1.5 x 2^-36
+    compare(sim, orc, 1e-9, 1e-10)
+    sim.close()
+
+
+def test_value_range():
+    sim, orc = simulation()
+    k = np.arange(8)
+    x, v = 3 * k + 0.5 + dyadic(0.3), np.array([-20.5 + 3 * k + dyadic(0.4), 0 * k + dyadic(0.3) - 0.5, 0 * k - 0.75])
+    f = np.array([1.0, 1e-305, -3e-300, 1e-290, 1e140, -1e130, 0.0, 1e-60])
+    sim.set_markers(0, x, v, f)
+    orc.set_markers(0, x, v, f)
+    orc.refresh()
+    got, ref, den = sim.get_f(0), orc.f[0], orc.den[0]
+    assert np.all(np.abs(got - ref)[den > 0] <= 1e-12 * np.abs(ref)[den > 0])
+    sim.close()
+
+
+def test_overflow_is_reported():
+    """Five markers whose weighted values add up beyond the range: f is infinite
+    and the call says so."""
+    from paper_1804_03901_gb300 import avl as A
+    sim, _ = simulation()
+    with pytest.raises(A.AvlError) as e:
+        sim.set_markers(0, np.full(5, 4.5), np.full((3, 5), -0.5), np.full(5, 1.7e308))
+        sim.synchronize()
+    assert e.value.status == A.AVL_ENUMERIC
+    sim.close()
