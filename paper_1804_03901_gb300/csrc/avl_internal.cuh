@@ -180,6 +180,7 @@ struct Ctl {
     int sort_next[MAXS];       // decided by the field kernel for the next step
     int hsel[MAXS];            // which cnt / far_cnt buffer holds the current counts
     unsigned long long ovf_count[MAXS];
+    int ovf_used[MAXS];        // 1d1v FP64: the overflow grids were written, by markers of the window too
     unsigned long long ovf_last[MAXS];
     unsigned long long nsort[MAXS];
     unsigned long long uncovered[MAXS];   // markers outside their chunk's best window (decision input)

@@ -15,7 +15,7 @@
 // The low limbs are signed, so that the product of two of them, which is
 // left out, is at most a quarter of the sum's unit, of either sign.  The units
 // are absolute, so what would reach a cell with a small weight only, and values
-// outside FX_EMIN .. FX_EMAX, are summed in FP64 instead (k_pd3x).  Against
+// outside FX_EMIN .. FX_EMAX, are summed in FP64 instead (k_pd3x, k_pd1x).  Against
 // exact rational sums of 4 to 12 markers with values over one e-fold: f
 // 7e-17 rms, weights 5e-17 (the same sums in FP64: 1.3e-16 and 1e-16).
 #pragma once
@@ -116,17 +116,19 @@ __device__ __forceinline__ long long fx_count(double t)
 }
 
 // an integer as FP64, to nearest, without the FP64 pipe
-__device__ __forceinline__ double fx_double(long long v)
+__device__ __forceinline__ double fx_double(unsigned long long a)
 {
-    const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
     if (a == 0) return 0.0;
     const int z = __clzll((long long)a);
     const unsigned long long t = a << z;                       // top bit set
     // exponent field of the top bit, less the bit itself; the rounding carry
     // runs into the exponent as it should
-    unsigned long long r = ((unsigned long long)(1085 - z) << 52) + ((t >> 11) + ((t >> 10) & 1ull));
-    if (v < 0) r |= 0x8000000000000000ull;
-    return __longlong_as_double((long long)r);
+    return __longlong_as_double((long long)(((unsigned long long)(1085 - z) << 52) + ((t >> 11) + ((t >> 10) & 1ull))));
+}
+__device__ __forceinline__ double fx_double(long long v)
+{
+    const long long r = __double_as_longlong(fx_double(v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v));
+    return __longlong_as_double(v < 0 ? r | (long long)0x8000000000000000ull : r);
 }
 
 // lesser of a weight w (a count of 2^-52) and 1 - w, but 1 for w = 0, whose

@@ -605,6 +605,7 @@ __global__ void __cluster_dims__(FIELD_CLUSTER, 1, 1) __launch_bounds__(FIELD_TH
         if (s < ns) {
             ctl->ovf_last[s] = ovf;
             ctl->ovf_count[s] = 0;
+            ctl->ovf_used[s] = 0;
             if (sp_dim == 3) {
                 // 1d3v: the deposit just finalized becomes current, the other
                 // accumulator (cleared by the finalize) takes the next one.

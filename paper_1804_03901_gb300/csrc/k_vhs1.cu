@@ -734,17 +734,24 @@ __global__ void __launch_bounds__(PD_THREADS, 2) k_pd1(const StepArgs* __restric
 // FP64 form.  The FP64 pipe takes a warp instruction per 64 clocks and
 // sub-partition, and a shared-memory FP64 reduction is a loop around such an
 // addition, so the weights are integers (fixed.cuh) and the denominator of
-// Eq. 4 is summed in the window as 64-bit counts of 2^-wb (wb: what M weights
-// of at most 1 leave of 63 bits), exact sums of the rounded weights.  The
-// numerator takes the same rounded weight times the value, one FP64 product
-// and one FP64 reduction per corner, so that the rounding of a weight enters
-// f only through the spread of the values in a cell.  14 FP64 operations per
-// marker where the same deposit in FP64, with its runs of markers of one
+// Eq. 4 is summed in the window as 64-bit counts of 2^-57, exact sums of the
+// rounded weights: a carry out of a word, every 128 weights of 1 at the
+// soonest, goes to the FP64 overflow grid.  The numerator takes the same
+// rounded weight times the value, one FP64 product and one FP64 reduction per
+// corner, so that the rounding of a weight enters f only through the spread of
+// the values in a cell.  A marker with a corner below SMALL1 = 2^-24 (four in
+// a million at random places) goes to the overflow grids as a whole, its
+// weights FP64 products, so that n of a cell that only small weights reach is
+// within 2^-33 too and no cell is lost (at 2^-22 the finalize of 512 x 6600
+// cells reads 26 us more of overflow rows).  14 FP64 operations per marker
+// where the same deposit in FP64, with its runs of markers of one
 // footprint summed in registers first, took about 40 (lanes end their runs
 // at different markers, so a warp flushed at every marker all the same):
-// 13.5 M markers, 512 x 6600 cells 1.12 -> 0.63 ms. The conversion of the
+// 13.5 M markers, 512 x 6600 cells 1.12 -> 0.64 ms. The conversion of the
 // displacement in integers is worth 5 % (0.66 ms on the FP64 pipe); two CTAs
 // per SM at 64 registers are slower (0.70 ms).
+constexpr float SMALL1 = 1.0f / (1 << 24);
+
 template <bool BATCH, bool PUSH>
 __global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restrict__ A0,
                                                         const BatchMap* __restrict__ bm)
@@ -770,7 +777,7 @@ __global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restri
     const size_t eb = ((size_t)nx * 8 + 15) & ~size_t(15);
     double* Es = reinterpret_cast<double*>(smem);
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + eb);
-    int* misc = reinterpret_cast<int*>(smem + eb + 16);   // [0] overflow runs, [2] row0
+    int* misc = reinterpret_cast<int*>(smem + eb + 16);   // [0] overflow runs, [1] overflow grids written, [2] row0
     int* scnt = reinterpret_cast<int*>(smem + eb + 32);   // next-step histogram
     int* hcur = scnt + HIST_S;                             // current-key histogram (window placement)
     int* shs = hcur + HIST_S;                              // per-column row shift (nx)
@@ -781,7 +788,7 @@ __global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restri
 
     const bool use_bulk = PUSH && nx % 2 == 0;
     if (threadIdx.x == 0) {
-        misc[0] = 0;
+        misc[0] = misc[1] = 0;
         if (use_bulk) {
             mbar_init(bar, 1);
             fence_mbar_init();
@@ -825,8 +832,6 @@ __global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restri
     const double inv_dv = sp.inv_dv[0];
     // displacement in cells: (v_ref + dv) dt / dx, v_ref of the chunk's reference row
     const double dt_dx = sp.dt_dx, vref_dtdx = (sp.vmin[0] + (double)kb * sp.dv[0]) * sp.dt_dx;
-    // bits of the window's weights: M of them, none above 1, stay below 2^62
-    const int wb = 62 - max(32 - __clz(sp.M - 1), 5), wsh = 57 - wb;
     double* ovf_num = sp.ovf;
     double* ovf_den = sp.ovf + (size_t)nv * nx;
     int* ovf_tag = sp.ovf_tag;
@@ -878,28 +883,42 @@ __global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restri
                 const int j0 = kb + vrow_rel(dv, inv_dv, w52);
                 code = rel_code(clampi(j0, 0, nv - 1), kbase);
                 if (j0 + 1 >= 0 && j0 < nv) {
-                    // 2^-57: one product, the others by difference
-                    const long long u = (U & (FX_ONE - 1)) << 5, w = w52 << 5;
-                    const long long a3 = fx_mul(fx_split(u), fx_split(w >> 1)), a2 = w - a3, a1 = u - a3;
-                    const long long half = wsh > 0 ? 1ll << (wsh - 1) : 0;
-                    const long long a[4] = {((FX_ONE << 5) - u - a2 + half) >> wsh, (a1 + half) >> wsh,
-                                            (a2 + half) >> wsh, (a3 + half) >> wsh};
                     const int wa = j0 - shs[ia] - row0, wc = j0 - shs[ib] - row0;
                     const double f = f4[m];
-                    if (wa >= 0 && wa + 1 < W && wc >= 0 && wc + 1 < W) {
+                    const long long u52 = U & (FX_ONE - 1);
+                    const bool in = wa >= 0 && wa + 1 < W && wc >= 0 && wc + 1 < W;
+                    if (in && lesser_weight(u52) * lesser_weight(w52) >= SMALL1) {
+                        // 2^-57: one product, the others by difference
+                        const long long u = u52 << 5, w = w52 << 5;
+                        const long long a3 = fx_mul(fx_split(u), fx_split(w >> 1)), a2 = w - a3, a1 = u - a3;
+                        const long long a[4] = {(FX_ONE << 5) - u - a2, a1, a2, a3};
                         const int cell[4] = {wa * nx + ia, wc * nx + ib, (wa + 1) * nx + ia, (wc + 1) * nx + ib};
+                        unsigned long long old[4];
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
-                            atomicAdd(wden + cell[k], (unsigned long long)a[k]);
-                            atomicAdd(win + cell[k], fx_scale(fx_double(a[k]), -wb) * f);
+                            old[k] = atomicAdd(wden + cell[k], (unsigned long long)a[k]);
+                            atomicAdd(win + cell[k], fx_scale(fx_double(a[k]), -57) * f);
+                        }
+                        // a weight carries out of a word only from its last 2^57
+                        if (max(max(old[0], old[1]), max(old[2], old[3])) >> 57 == 127) {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const int j = j0 + (k >> 1);
+                                if (old[k] + (unsigned long long)a[k] >= old[k] || j < 0 || j >= nv) continue;
+                                atomicAdd(ovf_den + (size_t)j * nx + (k & 1 ? ib : ia), 128.0);   // 2^64 counts
+                                ovf_tag[j] = tag;
+                                misc[1] = 1;
+                            }
                         }
                     } else {
                         double d[4];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) d[k] = fx_scale(fx_double(a[k]), -wb);
+                        for (int k = 0; k < 4; ++k)
+                            d[k] = fx_scale(weight_of(u52, k & 1) * weight_of(w52, k & 2), -104);
                         flush_overflow(ia, ib, j0, nx, nv, d[0] * f, d[1] * f, d[2] * f, d[3] * f, d[0], d[1], d[2],
                                        d[3], ovf_num, ovf_den, ovf_tag, tag);
-                        ++n_over;
+                        misc[1] = 1;
+                        if (!in) ++n_over;
                     }
                 }
             }
@@ -917,7 +936,7 @@ __global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restri
     if (PUSH)
         for (int i = threadIdx.x; i < HIST_S; i += PD_THREADS) sp.cnt[1 - hs][(size_t)c * HIST_S + i] = scnt[i];
     for (int i = threadIdx.x; i < plane; i += PD_THREADS)
-        win[plane + i] = fx_scale(fx_double((long long)wden[i]), -wb);
+        win[plane + i] = fx_scale(fx_double(wden[i]), -57);
     __syncthreads();
     // flush the window to this chunk's partial sums with one bulk copy
     if (threadIdx.x == 0) {
@@ -926,6 +945,7 @@ __global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restri
         bulk_s2g(dstp, win, (unsigned)win_bytes);
         bulk_commit();
         if (misc[0]) atomicAdd(&ctl->ovf_count[s], (unsigned long long)misc[0]);
+        if (misc[1]) ctl->ovf_used[s] = 1;
         bulk_wait_all();
     }
 }
@@ -1110,7 +1130,7 @@ __global__ void __launch_bounds__(FIN_THREADS, 4) k_fin1(const StepArgs* __restr
     const bool xok = x < nx;
     const int j0 = rqi * sp.rq, j1 = min(nv, j0 + sp.rq);
     const int plane = win_plane(W, nx);
-    const bool any_ovf = ctl->ovf_count[s] != 0;
+    const bool any_ovf = ctl->ovf_count[s] != 0 || ctl->ovf_used[s] != 0;
     double* ovf_num = sp.ovf;
     double* ovf_den = sp.ovf + (size_t)nv * nx;
     const int* ovf_tag = sp.ovf_tag;
@@ -1164,9 +1184,9 @@ __global__ void __launch_bounds__(FIN_THREADS, 4) k_fin1(const StepArgs* __restr
     // overflow rows, f = num / den, f and n stored, charge and diagnostics
     // (FP32: f_ref = the cell's f of the previous reconstruction, read before
     // it is overwritten; the deposit kernel staged the same value)
-    auto finish = [&](int j, CellSum<T>& cs) {
+    auto finish = [&](int j, int row_tag, CellSum<T>& cs) {
         const T fr = sizeof(T) == 4 ? fg[(size_t)j * nx + x] : (T)0;
-        if (any_ovf && ovf_tag[j] == tag) {
+        if (row_tag == tag) {
             const size_t o = (size_t)j * nx + x;
             cs.add_ovf(ovf_num[o], ovf_den[o], fr);
             ovf_num[o] = 0.0;
@@ -1190,6 +1210,7 @@ __global__ void __launch_bounds__(FIN_THREADS, 4) k_fin1(const StepArgs* __restr
             const int jb = j + RL;
             const bool two = jb < j1;
             const int ra = j - shx, rb = jb - shx;   // rows in window coordinates
+            const int ta = any_ovf ? ovf_tag[j] : 0, tb = any_ovf && two ? ovf_tag[jb] : 0;
             while (lo < nlist && srow[lo] + W <= ra) ++lo;
             int lob = lo;
             while (lob < nlist && srow[lob] + W <= rb) ++lob;
@@ -1218,14 +1239,14 @@ __global__ void __launch_bounds__(FIN_THREADS, 4) k_fin1(const StepArgs* __restr
                 if (oa[k]) ca.add_pair(na[k], da[k]);
             for (int q = lo + WSLOT; q < nlist && srow[q] <= ra; ++q)
                 ca.add_partial(pcol + (size_t)slist[q] * wstride + (size_t)(ra - srow[q]) * nx, plane);
-            finish(j, ca);
+            finish(j, ta, ca);
             if (two) {
 #pragma unroll
                 for (int k = 0; k < WSLOT; ++k)
                     if (ob[k]) cb.add_pair(nb[k], db[k]);
                 for (int q = lob + WSLOT; q < nlist && srow[q] <= rb; ++q)
                     cb.add_partial(pcol + (size_t)slist[q] * wstride + (size_t)(rb - srow[q]) * nx, plane);
-                finish(jb, cb);
+                finish(jb, tb, cb);
             }
             lo = lob;
         }
@@ -1237,7 +1258,7 @@ __global__ void __launch_bounds__(FIN_THREADS, 4) k_fin1(const StepArgs* __restr
                 const int wr = j - shx - sp.wrow0[cc];
                 if (wr >= 0 && wr < W) cs.add_partial(part + (size_t)cc * planes * plane + (size_t)wr * nx + x, plane);
             }
-            finish(j, cs);
+            finish(j, any_ovf ? ovf_tag[j] : 0, cs);
         }
     }
     // charge of this species per column, summed over the row lanes in order
