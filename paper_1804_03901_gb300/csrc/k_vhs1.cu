@@ -852,6 +852,7 @@ __global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restri
             loadg(fp + g0, f4);
             loadg(xp + g0, x4);
         }
+        int pi = 0x7fffffff, pj = 0;   // footprint of the marker before: a run of them counts once
 #pragma unroll
         for (int m = 0; m < MPT; ++m) {
             const bool ok = g0 + m < end;
@@ -882,6 +883,9 @@ __global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restri
                 long long w52;
                 const int j0 = kb + vrow_rel(dv, inv_dv, w52);
                 code = rel_code(clampi(j0, 0, nv - 1), kbase);
+                const bool first = i0 != pi || j0 != pj;
+                pi = i0;
+                pj = j0;
                 if (j0 + 1 >= 0 && j0 < nv) {
                     const int wa = j0 - shs[ia] - row0, wc = j0 - shs[ib] - row0;
                     const double f = f4[m];
@@ -918,7 +922,7 @@ __global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restri
                         flush_overflow(ia, ib, j0, nx, nv, d[0] * f, d[1] * f, d[2] * f, d[3] * f, d[0], d[1], d[2],
                                        d[3], ovf_num, ovf_den, ovf_tag, tag);
                         misc[1] = 1;
-                        if (!in) ++n_over;
+                        if (!in && first) ++n_over;
                     }
                 }
             }

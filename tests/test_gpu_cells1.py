@@ -89,3 +89,21 @@ def test_dense_cells(monkeypatch):
     orc.refresh()
     compare(sim, orc, 1e-9, 1e-9)
     sim.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("kinds,runs", [((0, 0, 0, 0), 1), ((0, 0, 1, 1), 2), ((0, 1, 0, 1), 4)])
+def test_out_of_window_runs(kinds, runs, precision, monkeypatch):
+    """The counter of avl_get_stats: runs of consecutive markers with the same
+    cells that miss their chunk's window, in either precision."""
+    from paper_1804_03901_gb300 import avl as A
+    monkeypatch.setenv("AVL_WMAX", "6")
+    prec = A.AVL_FP64 if precision == "fp64" else A.AVL_FP32
+    sim = A.Simulation(A.make_domain(1, NX, float(NX), 1e-4, precision=prec),
+                       [A.make_species(-1.0, 1.0, (NV,), (VMIN,), (VMAX,))])
+    x = np.concatenate([np.arange(60) + 0.75, 10.75 + 20.0 * np.array(kinds)])
+    v = np.concatenate([np.full(60, VMIN + 20.75), np.full(4, VMIN + 50.75)])
+    sim.set_markers(0, x, v, np.ones(64))
+    sim.step(1)
+    assert sim.get_stats()[0][0] == runs
+    sim.close()
