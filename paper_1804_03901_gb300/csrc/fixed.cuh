@@ -27,8 +27,9 @@ constexpr long long FX_ONE = 1ll << 52;       // 1 of a 52-bit fraction (positio
 constexpr int FX_LIMB = 28;
 constexpr int FX_PAIRS = 56;                  // products of weights <= 1 a sum takes before it is flushed:
                                               // |h| stays below 56 2^57 + 2^59, |m| below 56 (2^56 + 2^55)
-constexpr int FX_EMIN = 64, FX_EMAX = 2040;   // exponent fields of the values that the sums take: theirs (units of
-                                              // at least 2^-1015, magnitudes below 2^1024) are normal numbers
+constexpr int FX_EMIN = 96, FX_EMAX = 2040;   // exponent fields of the values that the sums take: theirs (units of
+                                              // at least 2^-983, magnitudes below 2^1024) are normal numbers, also
+                                              // with 26 bits below the unit
 
 // v = h 2^28 + l, -2^27 <= l < 2^27
 struct Limbs {

@@ -256,97 +256,131 @@ __global__ void __launch_bounds__(256) k_ad_dep(const AdjDev* __restrict__ D, in
 
 // FP64: a warp sums its contributions in a patch of shared memory (columns x
 // rows around its markers' footprints), weights and sums in integers
-// (fixed.cuh), values in units of the warp's largest, and adds every cell of
-// the patch to the grid: 20 to 60 reductions of (numerator, denominator)
-// where the markers have 128 corners.  Lattice neighbours share footprints in
-// fours; four copies of the patch by lane keep them off one another's words.
-// A warp whose patch does not fit (or with values that are not finite) adds
-// every corner to the grid.  1 M markers: 75 -> 34 us (one copy 54).
+// (fixed.cuh), and adds every cell of the patch to the grid: 20 to 60
+// reductions of (numerator, denominator) where the markers have 128 corners.
+// Lattice neighbours share footprints in fours; four copies of the patch by
+// lane keep them off one another's words.  g of a marker (k_ad_gather) has
+// the factor (f - F) / D, so F = N / D must not lose what a small D leaves of
+// it: the numerator takes the denominator's rounded weights, each product
+// whole in two words (2^-57 and 2^-83 of the value's unit), and every cell has
+// its own unit, of the largest value that reaches it.  A marker with a corner
+// below SMALL_AD = 2^-16 (0.07 % of them), with a value beyond the sums' range
+// or in a warp whose patch does not fit adds its corners to the grid in FP64.
+// 1 M markers: 75 -> 39 us (34 with the products rounded to 2^-57 of the warp's
+// largest value; one copy 54; five blocks per SM, 51 registers, 46).
 constexpr int AD_PATCH = 160;   // words of a warp's patch and its copies
-__global__ void __launch_bounds__(256, 5) k_ad_depx(const AdjDev* __restrict__ D, int nx, int slot, int all)
+constexpr int AD_LO = 26;       // bits of the low words: 32 of them stay below 2^31
+constexpr float SMALL_AD = 1.0f / (1 << 16);
+__global__ void __launch_bounds__(256, 4) k_ad_depx(const AdjDev* __restrict__ D, int nx, int slot, int all)
 {
     __shared__ unsigned long long patch_s[8][2 * AD_PATCH];
+    __shared__ unsigned low_s[8][2 * AD_PATCH];
     const int s = all ? D->stat[blockIdx.y] : D->act[blockIdx.y];
     const AdjSp& a = D->sp[s];
     const AdjC<double> C = a.cd;
     const int nv = a.nv, lane = threadIdx.x & 31;
-    unsigned long long* Pn = patch_s[threadIdx.x >> 5];
+    unsigned long long* Pn = patch_s[threadIdx.x >> 5];   // numerators, denominators
     unsigned long long* Pd = Pn + AD_PATCH;
+    unsigned* Pl = low_s[threadIdx.x >> 5];               // low words of the numerators
+    int* Pe = reinterpret_cast<int*>(Pl + AD_PATCH);      // exponents of the units
     double* acc = reinterpret_cast<double*>(a.num);
     const double* f = reinterpret_cast<const double*>(a.f);
     const double* vv = reinterpret_cast<const double*>(a.hv) + (size_t)slot * a.n;
     const long long n_pad = (a.n + 31) / 32 * 32;   // whole warps iterate together
     for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n_pad; k += (long long)gridDim.x * blockDim.x) {
         bool ok = k < a.n;
-        int i0 = 0, j0 = -2, e = 0;
-        long long u = 0, w = 0, mant = 0;
+        int i0 = 0, j0 = -2;
+        long long u = 0, w = 0;   // weights, 2^-52
         double fl = 0.0;
         if (ok) {
             const long long U = APos<double>::load(a, slot, k).X - (FX_ONE >> 1);
             i0 = (int)(U >> 52);
-            u = (U & (FX_ONE - 1)) << 5;
+            u = U & (FX_ONE - 1);
             j0 = vrow52(vv[k], C, nv, w);
-            w <<= 5;
             fl = f[k];
-            mant = fx_value(fl, e);
         }
         ok = ok && j0 >= -1 && j0 < nv;   // a corner on the grid
-        const unsigned any = __ballot_sync(0xffffffffu, ok);
-        if (!any) continue;
-        const int emax = __reduce_max_sync(0xffffffffu, max(e, FX_EMIN));   // (2047: not finite; sums of 32 take five more)
-        long long c[4];                   // weights of the corners, 2^-57
-        c[3] = fx_mul(fx_split(u), fx_split(w >> 1));
-        c[2] = w - c[3];
-        c[1] = u - c[3];
-        c[0] = (FX_ONE << 5) - u - c[2];
-        // the patch: columns relative to the first marker's (periodic), rows
-        const int ir = __shfl_sync(0xffffffffu, i0, __ffs(any) - 1);
-        int di = i0 - ir;
-        if (2 * di > nx) di -= nx;
-        if (2 * di < -nx) di += nx;
-        const int d0 = __reduce_min_sync(0xffffffffu, ok ? di : 0x3fffffff);
-        const int d1 = __reduce_max_sync(0xffffffffu, ok ? di : -0x3fffffff);
-        const int r0 = __reduce_min_sync(0xffffffffu, ok ? j0 : 0x3fffffff);
-        const int r1 = __reduce_max_sync(0xffffffffu, ok ? j0 : -0x3fffffff);
-        const int W = d1 - d0 + 2, H = r1 - r0 + 2;
-        if (W <= nx && H <= AD_PATCH && W * H <= AD_PATCH && emax < 2040) {
-            const int cs = W * H * 4 <= AD_PATCH ? 2 : 0;   // copies: 1 << cs
-            for (int q = lane; q < (W * H) << cs; q += 32) Pn[q] = Pd[q] = 0;
-            __syncwarp();
-            if (ok) {
-                const Limbs v = fx_split(mant >> min(emax - e, 63));
+        int e;
+        const long long mant = fx_value(fl, e);
+        bool pat = ok && lesser_weight(u) * lesser_weight(w) >= SMALL_AD && (fx_in_range(e) || mant == 0);
+        const unsigned any = __ballot_sync(0xffffffffu, pat);
+        if (any) {
+            // the patch: columns relative to the first marker's (periodic), rows
+            const int ir = __shfl_sync(0xffffffffu, i0, __ffs(any) - 1);
+            int di = i0 - ir;
+            if (2 * di > nx) di -= nx;
+            if (2 * di < -nx) di += nx;
+            const int d0 = __reduce_min_sync(0xffffffffu, pat ? di : 0x3fffffff);
+            const int d1 = __reduce_max_sync(0xffffffffu, pat ? di : -0x3fffffff);
+            const int r0 = __reduce_min_sync(0xffffffffu, pat ? j0 : 0x3fffffff);
+            const int r1 = __reduce_max_sync(0xffffffffu, pat ? j0 : -0x3fffffff);
+            const int W = d1 - d0 + 2, H = r1 - r0 + 2;
+            if (W <= nx && H <= AD_PATCH && W * H <= AD_PATCH) {
+                const int cs = W * H * 4 <= AD_PATCH ? 2 : 0;   // copies: 1 << cs
+                for (int q = lane; q < (W * H) << cs; q += 32) {
+                    Pn[q] = Pd[q] = 0;
+                    Pl[q] = 0;
+                    Pe[q] = FX_EMIN;
+                }
+                __syncwarp();
                 const int at = (di - d0) * H + j0 - r0, lc = lane & ((1 << cs) - 1);
                 const int cell[4] = {at, at + H, at + 1, at + H + 1};
+                if (pat) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int o = (cell[q] << cs) + lc;
-                    atomicAdd(Pn + o, (unsigned long long)fx_mul(fx_split(c[q]), v));
-                    atomicAdd(Pd + o, (unsigned long long)c[q]);
+                    for (int q = 0; q < 4; ++q) atomicMax(Pe + cell[q], e);
                 }
-            }
-            __syncwarp();
-            for (int q = lane; q < W * H; q += 32) {
-                long long sn = 0, sd = 0;
-                for (int t = 0; t < 1 << cs; ++t) {
-                    sn += (long long)Pn[(q << cs) + t];
-                    sd += (long long)Pd[(q << cs) + t];
+                __syncwarp();
+                if (pat) {
+                    long long c[4];   // weights of the corners, 2^-57
+                    c[3] = fx_mul(fx_split(u << 5), fx_split(w << 4));
+                    c[2] = (w << 5) - c[3];
+                    c[1] = (u << 5) - c[3];
+                    c[0] = (FX_ONE << 5) - (u << 5) - c[2];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int o = (cell[q] << cs) + lc;
+                        const Limbs A = fx_split(c[q]), v = fx_split(mant >> min(Pe[cell[q]] - e, 63));
+                        long long m = ((long long)A.l * v.l) >> FX_LIMB;
+                        mad_wide(m, A.h, v.l);
+                        mad_wide(m, A.l, v.h);
+                        long long h = m >> FX_LIMB;
+                        mad_wide(h, A.h, v.h);
+                        atomicAdd(Pn + o, (unsigned long long)h);
+                        atomicAdd(Pl + o, ((unsigned)m & ((1u << FX_LIMB) - 1)) >> (FX_LIMB - AD_LO));
+                        atomicAdd(Pd + o, (unsigned long long)c[q]);
+                    }
                 }
-                const int col = q / H, j = r0 + q - col * H;
-                int x = ir + d0 + col;
-                x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
-                if (sd != 0 && j >= 0 && j < nv)
-                    pair_add(acc + 2 * ((size_t)x * nv + j), fx_scale(fx_double(sn), emax - 1079),
-                             fx_scale(fx_double(sd), -57));
+                __syncwarp();
+                for (int q = lane; q < W * H; q += 32) {
+                    long long sn = 0, sd = 0, sl = 0;
+                    for (int t = 0; t < 1 << cs; ++t) {
+                        sn += (long long)Pn[(q << cs) + t];
+                        sd += (long long)Pd[(q << cs) + t];
+                        sl += Pl[(q << cs) + t];
+                    }
+                    sn += sl >> AD_LO;
+                    // as many of the low bits as there is room for
+                    const int z = min(__clzll(sn < 0 ? ~sn : sn) - 1, AD_LO);
+                    sn = sn * (1ll << z) + ((sl & ((1 << AD_LO) - 1)) >> (AD_LO - z));
+                    const int col = q / H, j = r0 + q - col * H;
+                    int x = ir + d0 + col;
+                    x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
+                    if (sd != 0 && j >= 0 && j < nv)
+                        pair_add(acc + 2 * ((size_t)x * nv + j), fx_scale(fx_double(sn), Pe[q] - 1079 - z),
+                                 fx_scale(fx_double(sd), -57));
+                }
+                __syncwarp();
+                ok = ok && !pat;
             }
-            __syncwarp();
-        } else if (ok) {
+        }
+        if (ok) {
             int ia, ib;
             wrap_pair(i0, nx, ia, ib);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int j = j0 + (q >> 1);
                 if (j < 0 || j >= nv) continue;
-                const double cd = fx_scale(fx_double(c[q]), -57);
+                const double cd = fx_scale(weight_of(u, q & 1) * weight_of(w, q & 2), -104);
                 pair_add(acc + 2 * ((size_t)(q & 1 ? ib : ia) * nv + j), cd * fl, cd);
             }
         }

@@ -57,3 +57,44 @@ def test_adjoint_edges(A, nx, nv, lat, nsteps, dt, prec):
     tolJ, tolg = (1e-10, 1e-8) if prec == 0 else (2e-3, 2e-3)
     assert J == pytest.approx(Jo, rel=tolJ)
     assert np.max(np.abs(g - go)) < tolg * np.max(np.abs(go)), (g, go)
+
+
+@pytest.mark.parametrize("w", [1e-3, 1e-4])
+def test_adjoint_cell_of_small_weights(A, w):
+    """After the step a cell of the last velocity row is reached by one marker
+    with weight w alone; there the gradient has terms (f - F) / w.  The mode
+    amplitude that puts the marker there comes from the oracle; a short step
+    and a strong field keep the markers of the row (v near 0) in their columns."""
+    nx, nv, L, seed, jitter, dt, cP = 8, 64, 10.0, 11, 1e-9, 1e-6, 4e5
+    dx, dv = L / nx, 0.125
+    sp = dict(q=-1.0, m=1.0, nv=(nv,), vmin=((1 - nv) * dv,), vmax=(dv,), mobile=True)
+    f0 = lambda amp: dict(beams=[(1.0, (-1.0,), (1.5,))], modes=[(1, amp, 0.3), (2, 0.01, 1.1)])
+
+    def weight(amp):   # of the last row, least over its markers after the push
+        x, v, f = O.init_markers(1, nx, L, O.Species(**sp), (1, 1, 1, 1), O.F0(**f0(amp)), 0, seed, jitter)
+        orc = O.OracleSim(1, nx, L, dt, [O.Species(**sp)], cP, True)
+        orc.set_markers(0, x, v, f)
+        orc.refresh()
+        E, v = orc.E, np.asarray(v).reshape(-1)
+        i0 = np.floor(x / dx - 0.5).astype(int)
+        u = x / dx - 0.5 - i0
+        t = (v - dt * ((1.0 - u) * E[i0 % nx] + u * E[(i0 + 1) % nx]) - sp["vmin"][0]) / dv - 0.5
+        return np.min(t[v > 0.0]) - (nv - 2)
+
+    lo, hi = 0.0, 0.9
+    for _ in range(60):
+        mid = 0.5 * (lo + hi)
+        lo, hi = (mid, hi) if weight(mid) > w else (lo, mid)
+    amp = 0.5 * (lo + hi)
+    assert 0.9 * w < weight(amp) < 1.1 * w
+    sim = A.Simulation(A.make_domain(1, nx, L, dt, cP, True, 0), [A.make_species(**sp)])
+    sim.init_markers(0, (1, 1, 1, 1), A.make_f0(**f0(amp)), seed, jitter)
+    J, ga, gu = sim.adjoint(0, A.make_f0(**f0(amp)), 1, 1)
+    sim.close()
+    Jo, goa, gou, _ = AD.field_energy_gradient(nx, L, dt, [O.Species(**sp)], [O.F0(**f0(amp))], [(1, 1, 1, 1)], seed,
+                                               jitter, 0, 1, cP, True)
+    g, go = np.concatenate([ga, gu]), np.concatenate([goa, gou])
+    # the cell's share of the gradient is about w; its F keeps 2^-52 and w itself
+    # 2^-52 / w, whatever w is, and the sums have some 1e2 roundings
+    assert J == pytest.approx(Jo, rel=1e-13)
+    assert np.max(np.abs(g - go)) < 1e-13 * np.max(np.abs(go)), (g - go, go)
