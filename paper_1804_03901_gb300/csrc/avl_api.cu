@@ -830,9 +830,9 @@ avl_status avl_create(const avl_domain* dom, const avl_species* spec, int32_t ns
             v2[j] = v * v;
             v2f[j] = (float)v * (float)v;
         }
-        e = cudaMemcpy(pv2, dom->precision == AVL_FP32 ? (const void*)v2f.data() : (const void*)v2.data(), nvk * pb,
-                       cudaMemcpyHostToDevice);
-        if (e) {
+        if ((e = cudaMemcpyAsync(pv2, dom->precision == AVL_FP32 ? (const void*)v2f.data() : (const void*)v2.data(),
+                                 nvk * pb, cudaMemcpyHostToDevice, c->st)) ||
+            (e = cudaStreamSynchronize(c->st))) {
             cuda_fail(c, e, "cudaMemcpy(v2)");
             return bail(AVL_ECUDA);
         }
