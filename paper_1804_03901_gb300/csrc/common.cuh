@@ -197,42 +197,37 @@ struct ff {
 };
 
 __device__ __forceinline__ void ff_add(ff& a, float x) { two_sum_add(a.hi, a.lo, x); }
-__device__ __forceinline__ void ff_add(ff& a, ff b)
-{
-    two_sum_add(a.hi, a.lo, b.hi);
-    a.lo = __fadd_rn(a.lo, b.lo);
-}
 
-// Sums of a finalize block, in the accumulators' own arithmetic (FP32 as
-// float-float): an FP64 addition or conversion costs a warp 64 clocks, and the
-// trees of N, W_kin and S, the conversions before them and v^2 of a row took
-// 31 per warp and row pair (now six additions per block warp, v^2 from a
-// table): k_fin1 at 512 x 1024 FP32 48 -> 33 us, 512 x 6600 FP64 114 -> 90,
-// 64 small runs 423 -> 340, k_fin3 at 100 x 24 x 20 x 18 FP64 53 -> 37.
-__device__ __forceinline__ void acc_add(ff& a, ff b) { ff_add(a, b); }
-__device__ __forceinline__ void acc_add(double& a, double b) { a += b; }
-__device__ __forceinline__ ff acc_xor(ff a, int o)
+// Sums of a finalize block in FP64.  An FP64 addition or conversion costs a
+// warp 64 clocks, so the three sums share their tree, v^2 of a row comes from a
+// table and the float-float accumulators of FP32 are widened in integers: nine
+// per warp of a block (FP64 accumulators six) where the trees of N, W_kin and
+// S, the conversions before them and v^2 took 31 per warp and row pair: k_fin1
+// at 512 x 1024 FP32 48 -> 35 us, 512 x 6600 FP64 114 -> 95, 64 small runs
+// 423 -> 352, k_fin3 at 100 x 24 x 20 x 18 FP64 53 -> 37.  (Block sums in
+// float-float take 33 and 340 us, and 48 bits.)
+//
+// sum over eight neighbouring lanes
+__device__ __forceinline__ double sum8(double v)
 {
-    return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
-__device__ __forceinline__ double acc_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
 // the warp's sums of a, b and c, in lanes 0, 8 and 16: half the lanes go on
 // with c, a quarter with b, so that three sums take six additions, not 15
-template <typename S>
-__device__ __forceinline__ S warp_sum3(S a, S b, S c)
+__device__ __forceinline__ double warp_sum3(double a, double b, double c)
 {
     const int lane = threadIdx.x & 31;
     const bool h = lane & 16, q = lane & 8;
-    S x = h ? c : a, y = h ? S{} : b;
-    acc_add(x, acc_xor(h ? a : c, 16));
-    acc_add(y, acc_xor(h ? b : S{}, 16));
-    S z = q ? y : x;
-    acc_add(z, acc_xor(q ? x : y, 8));
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) acc_add(z, acc_xor(z, o));
-    return z;
+    double x = h ? c : a, y = h ? 0.0 : b;
+    x += __shfl_xor_sync(0xffffffffu, h ? a : c, 16);
+    y += __shfl_xor_sync(0xffffffffu, h ? b : 0.0, 16);
+    double z = q ? y : x;
+    z += __shfl_xor_sync(0xffffffffu, q ? x : y, 8);
+    return sum8(z);
 }
-__device__ __forceinline__ double acc_value(ff a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double acc_value(ff a) { return fx_widen(a.hi) + fx_widen(a.lo); }
 __device__ __forceinline__ double acc_value(double a) { return a; }
 
 template <typename T>

@@ -132,6 +132,14 @@ __device__ __forceinline__ double fx_double(long long v)
     return __longlong_as_double(v < 0 ? r | (long long)0x8000000000000000ull : r);
 }
 
+// an FP32 value as FP64, without the FP64 pipe for zeros and normal numbers
+__device__ __forceinline__ double fx_widen(float v)
+{
+    const unsigned b = (unsigned)__float_as_int(v), m = b & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u && m != 0) return (double)v;   // subnormal, Inf, NaN
+    return __hiloint2double((int)((b & 0x80000000u) | (m ? (m >> 3) + (896u << 20) : 0u)), (int)(b << 29));
+}
+
 // lesser of a weight w (a count of 2^-52) and 1 - w, but 1 for w = 0, whose
 // corner takes nothing (at least 0 and less than 2^-32 below)
 __device__ __forceinline__ float lesser_weight(long long w)

@@ -1113,9 +1113,9 @@ __global__ void __launch_bounds__(FIN_THREADS, 4) k_fin1(const StepArgs* __restr
                                                       const BatchMap* __restrict__ bm)
 {
     constexpr int RL = FIN_THREADS / FIN_XB;   // row lanes
-    using Sum = typename ColAcc<T>::Sum;
-    __shared__ Sum col_red[RL][FIN_XB];
-    __shared__ Sum red[3][FIN_THREADS / 32];
+    static_assert(FIN_THREADS == 256 && FIN_XB == 16, "eight warps of two rows");
+    __shared__ double col_red[FIN_XB][8];
+    __shared__ double red[3][8];
     __shared__ int clist[FIN_LIST];
     __shared__ int crow[FIN_LIST];
     __shared__ int ncl;
@@ -1265,26 +1265,24 @@ __global__ void __launch_bounds__(FIN_THREADS, 4) k_fin1(const StepArgs* __restr
             finish(j, any_ovf ? ovf_tag[j] : 0, cs);
         }
     }
-    // charge of this species per column, summed over the row lanes in order
-    col_red[lr][col] = acc.rho;
-    __syncthreads();
-    if (lr == 0 && xok) {
-        Sum r = col_red[0][col];
-        for (int k = 1; k < RL; ++k) acc_add(r, col_red[k][col]);
-        sp.rho_part[(size_t)rqi * nx + x] = sp.q * sp.dv[0] * acc_value(r);
-    }
-    // diagnostics of the block
-    const Sum d = warp_sum3(acc.rho, acc.w, acc.ent);
+    // charge of this species per column and diagnostics of the block, in trees
+    // (an FP64 addition takes 77 clocks: 512 x 1024 FP32 37.5 us with the rows
+    // and warps added one after the other, 35.0 so)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double N = acc_value(acc.rho), d = warp_sum3(N, acc_value(acc.w), acc_value(acc.ent));
+    const double nc = N + __shfl_xor_sync(0xffffffffu, N, FIN_XB);   // the warp's two rows
+    if (lane < FIN_XB) col_red[lane][warp] = nc;
     if ((lane & 7) == 0 && lane < 24) red[lane >> 3][warp] = d;
     __syncthreads();
-    if (threadIdx.x < 3) {   // N, W_kin, S
-        const int k = threadIdx.x;
-        Sum a = red[k][0];
-        for (int w = 1; w < FIN_THREADS / 32; ++w) acc_add(a, red[k][w]);
-        const double cell = sp.dx * sp.dv[0];
-        sp.dpart[(size_t)blk * 4 + k] = acc_value(a) * (k == 1 ? 0.5 * sp.m * cell : cell);
-        if (k == 0) sp.dpart[(size_t)blk * 4 + 3] = 0.0;
+    if (warp < FIN_XB / 4) {   // four columns per warp
+        const int xr = xb * FIN_XB + (threadIdx.x >> 3);
+        const double r = sum8(col_red[threadIdx.x >> 3][lane & 7]);
+        if ((lane & 7) == 0 && xr < nx) sp.rho_part[(size_t)rqi * nx + xr] = sp.q * sp.dv[0] * r;
+    } else if (warp == FIN_XB / 4) {   // N, W_kin, S
+        const int k = min(lane >> 3, 2);
+        const double t = sum8(red[k][lane & 7]), cell = sp.dx * sp.dv[0];
+        if ((lane & 7) == 0)
+            sp.dpart[(size_t)blk * 4 + (lane >> 3)] = lane == 24 ? 0.0 : t * (k == 1 ? 0.5 * sp.m * cell : cell);
     }
 }
 

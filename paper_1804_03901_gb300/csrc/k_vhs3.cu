@@ -1114,10 +1114,9 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
 template <typename T>
 __global__ void __launch_bounds__(FIN3_X * FIN3_R) k_fin3(const StepArgs* __restrict__ A, int all_species)
 {
-    constexpr int NT = FIN3_X * FIN3_R;
-    using Sum = typename ColAcc<T>::Sum;
-    __shared__ Sum col_red[FIN3_R][FIN3_X];
-    __shared__ Sum red[3][NT / 32];
+    static_assert(FIN3_X == 32 && FIN3_R == 8, "eight warps, a row each");
+    __shared__ double col_red[FIN3_X][8];
+    __shared__ double red[3][8];
     const int g = blockIdx.x;
     const int s = species_of_fin3(A, g);
     const SpDev& sp = A->sp[s];
@@ -1171,25 +1170,21 @@ __global__ void __launch_bounds__(FIN3_X * FIN3_R) k_fin3(const StepArgs* __rest
             cell(j, num[o], den[o], v2[j]);
         }
     }
+    // charge per column and diagnostics of the block, in trees (as k_fin1)
     const double dvol = sp.dv[0] * sp.dv[1] * sp.dv[2];
-    col_red[lr][col] = acc.rho;
-    __syncthreads();
-    if (lr == 0 && xok) {
-        Sum r = col_red[0][col];
-        for (int k = 1; k < FIN3_R; ++k) acc_add(r, col_red[k][col]);
-        sp.rho_part[(size_t)rqi * nx + x] = sp.q * dvol * acc_value(r);
-    }
-    const Sum d = warp_sum3(acc.rho, acc.w, acc.ent);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double N = acc_value(acc.rho), d = warp_sum3(N, acc_value(acc.w), acc_value(acc.ent));
+    col_red[col][warp] = N;
     if ((lane & 7) == 0 && lane < 24) red[lane >> 3][warp] = d;
     __syncthreads();
-    if (threadIdx.x < 3) {   // N, W_kin, S
-        const int k = threadIdx.x;
-        Sum t = red[k][0];
-        for (int w = 1; w < NT / 32; ++w) acc_add(t, red[k][w]);
-        const double cell = sp.dx * dvol;
-        sp.dpart[(size_t)blk * 4 + k] = acc_value(t) * (k == 1 ? 0.5 * sp.m * cell : cell);
-        if (k == 0) sp.dpart[(size_t)blk * 4 + 3] = 0.0;
+    const int xr = xb * FIN3_X + (threadIdx.x >> 3);   // four columns per warp
+    const double r = sum8(col_red[threadIdx.x >> 3][lane & 7]);
+    if ((lane & 7) == 0 && xr < nx) sp.rho_part[(size_t)rqi * nx + xr] = sp.q * dvol * r;
+    if (warp == 0) {   // N, W_kin, S
+        const int k = min(lane >> 3, 2);
+        const double t = sum8(red[k][lane & 7]), cell = sp.dx * dvol;
+        if ((lane & 7) == 0)
+            sp.dpart[(size_t)blk * 4 + (lane >> 3)] = lane == 24 ? 0.0 : t * (k == 1 ? 0.5 * sp.m * cell : cell);
     }
 }
 
