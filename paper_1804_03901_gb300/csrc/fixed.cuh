@@ -160,12 +160,12 @@ __device__ __forceinline__ double fx_scale(double d, int k)
 
 // n / d for a normal d > 0, in integers: a 24-bit reciprocal of d's mantissa
 // from the FP32 approximation, one Newton-Raphson step to 30 bits, the
-// quotient's first 29 bits, and one correction by the exact remainder
-// (P. Markstein, "Computation of elementary functions on the IBM RISC
-// System/6000 processor", IBM J. Res. Dev. 34, 1990, the same scheme in
-// floating point).  Within 0.52 units in the last place (0.6 % of quotients
-// are not the nearest).  Operands or quotients that are not normal numbers
-// take the division operator.
+// quotient's first 29 bits, one correction by the exact remainder (P. Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000
+// processor", IBM J. Res. Dev. 34, 1990, the same scheme in floating point),
+// which leaves 0.55 units in the last place, and a second one to the nearest.
+// Operands or quotients that are not normal numbers take the division
+// operator.
 __device__ __forceinline__ double fx_div(double n, double d)
 {
     const long long bn = __double_as_longlong(n), bd = __double_as_longlong(d);
@@ -184,11 +184,14 @@ __device__ __forceinline__ double fx_div(double n, double d)
     const unsigned Q0 = __umulhi((unsigned)(N >> 21), R1);                                  // 2^-30
     const long long rem = (long long)((N << 30) - (unsigned long long)Q0 * D);               // 2^-82, exact
     long long Q = ((long long)Q0 << 32) + (((long long)(int)(rem >> 24) * (int)(R1 >> 1)) >> 26);   // 2^-62
-    if (Q < (1ll << 62)) {
-        Q <<= 1;
-        --ex;
-    }
-    const long long M = (long long)(((unsigned long long)Q + 512ull) >> 10);   // (Q may be just below 2^63)
+    const int below = Q < (1ll << 62) ? 1 : 0;
+    Q <<= below;
+    ex -= below;
+    long long M = (long long)(((unsigned long long)Q + 512ull) >> 10);   // (Q may be just below 2^63)
+    // N 2^(52 + below) - M D, between -D and D, from its low 64 bits
+    const long long left = (long long)((N << (52 + below)) - (unsigned long long)M * D);
+    if (2 * left > (long long)D) ++M;
+    if (2 * left < -(long long)D) --M;
     return __longlong_as_double((((long long)ex << 52) + (M - FX_ONE)) | (bn & (long long)0x8000000000000000ull));
 }
 

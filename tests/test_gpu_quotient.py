@@ -1,5 +1,6 @@
-"""Integer logarithm of the FP64 finalize: the entropy sum f log f where log f is
-small."""
+"""Integer quotient and logarithm of the FP64 finalize: f = num / den rounded
+to nearest where num and den are exact (dyadic weights and values), and the
+entropy sum f log f where log f is small."""
 import math
 
 import numpy as np
@@ -16,6 +17,26 @@ def simulation(nx, nv):
     vmax = tuple(a + n for a, n in zip(vmin, nv))
     return vmin, A.Simulation(A.make_domain(len(nv), nx, float(nx), 0.01, precision=A.AVL_FP64),
                               [A.make_species(-1.0, 1.0, nv, vmin, vmax)])
+
+
+@pytest.mark.parametrize("nx,nv,n", [(256, (128,), 150000), (61, (7,), 3000)])
+def test_quotient_to_nearest(nx, nv, n):
+    vmin, sim = simulation(nx, nv)
+    rng = np.random.default_rng(n)
+    # weights in x of 20 bits, none in v; values of 18 bits: sums of fewer than 2^14
+    # products are exact
+    i, w = rng.integers(0, nx - 1, n), rng.integers(1, 1 << 20, n) / 2.0 ** 20
+    row = rng.integers(0, nv[0], n)
+    f = rng.integers(1 << 17, 1 << 18, n) / 2.0 ** 17
+    sim.set_markers(0, i + 0.5 + w, vmin[0] + row + 0.5, f)
+    num, den = np.zeros((nx, nv[0])), np.zeros((nx, nv[0]))
+    for k, a in ((i, 1.0 - w), (i + 1, w)):
+        np.add.at(num, (k, row), a * f)
+        np.add.at(den, (k, row), a)
+    got, d = sim.get_f(0, with_n=True)
+    assert np.array_equal(d, den)
+    assert np.array_equal(got, np.divide(num, den, out=np.zeros_like(num), where=den > 0))
+    sim.close()
 
 
 @pytest.mark.parametrize("nv", [(24,), (8, 3, 2)])
