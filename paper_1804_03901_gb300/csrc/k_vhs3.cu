@@ -709,6 +709,7 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 3 : (CPT == 2 ? 2 : 1))
 // followed a much larger one: k_pd3x 8.54 -> 8.79 ms), and a value whose
 // exponent the sums do not hold goes with the small corners.
 constexpr float SMALL3 = 1.0f / (1 << 20);
+constexpr int PARK_FEW = 48;
 
 struct FxCol {
     long long d0[4], v0[4];   // row jseg: weights, weighted values of the four planes
@@ -991,7 +992,35 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
             // the parked markers: one thread per (marker, corner) into the
             // global accumulator, so that a chunk's few movers do not hold one
             // warp behind the others at the chunk's barrier
-            for (int t = threadIdx.x; t < nmv * 16; t += NT) {
+            // (many of them: a thread per marker, whose neighbours in the warp
+            // are near it on the grid)
+            for (int t = threadIdx.x; t < nmv && nmv > PARK_FEW; t += NT) {
+                const int o = NB - 1 - t;
+                const int4 id = pqa[o];
+                const longlong2 uw = reinterpret_cast<const longlong2*>(pqb)[o];
+                const longlong2 wyz = reinterpret_cast<const longlong2*>(pa)[o];
+                const double f = __hiloint2double(id.w, id.z);
+                const int x1 = id.x + 1 == nx ? 0 : id.x + 1;
+                double a[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    a[k] = fx_scale(weight_of(uw.x, k & 1) * weight_of(uw.y, k & 2), -104);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const double q = fx_scale(weight_of(wyz.x, c & 1) * weight_of(wyz.y, c & 2), -104);
+                    if (!pl.ok[c] || __double_as_longlong(q) == 0) continue;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int row = id.y + (k >> 1);
+                        if (__double_as_longlong(a[k]) == 0 || row < 0 || row >= nvx) continue;
+                        const double alpha = a[k] * q;
+                        const int at = pl.base[c] + row * nx + (k & 1 ? x1 : id.x);
+                        atomicAdd(gacc + at, alpha * f);
+                        atomicAdd(gacc + cells + at, alpha);
+                    }
+                }
+            }
+            for (int t = threadIdx.x; t < nmv * 16 && nmv <= PARK_FEW; t += NT) {
                 const int o = NB - 1 - (t >> 4);
                 const int4 id = pqa[o];
                 const longlong2 uw = reinterpret_cast<const longlong2*>(pqb)[o];
