@@ -69,6 +69,21 @@ constexpr int GREEN_MAX = 1024;     // largest nx solved by the circulant produc
 // bulk copies of the window need
 __host__ __device__ inline int win_plane(int W, int nx) { return (W * nx + 3) & ~3; }
 
+// log2 of the copies of an FP64 1d1v deposit window, by lane: its reductions
+// are compare-and-swap loops, in which the lanes of a warp that meet in a word
+// take turns.  No more copies than the markers per cell of a chunk's window, so
+// that clearing and adding them up stays small beside the deposit, and as many
+// as shared memory has room for.  524288 markers, deposit without and with:
+// 16 x 32 cells 253 and 50 us, 64 x 32 130 and 71, 256 x 128 194 and 151 (from
+// half as many 150, from a quarter 195).
+__host__ __device__ inline int win_copies_log2(int M, int W, int nx)
+{
+    const long long cells = win_plane(W, nx);
+    int c = 0;
+    while (c < 5 && (1ll << c) * cells <= M && ((2ll << c) + 1) * 16 * cells <= 160 * 1024) ++c;
+    return c;
+}
+
 // device-side error bits (Ctl::err)
 enum : int { ERR_TIMEOUT = 1, ERR_NUMERIC = 2, ERR_CAPACITY = 4 };
 

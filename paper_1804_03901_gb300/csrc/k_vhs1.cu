@@ -280,12 +280,19 @@ static size_t fref_bytes(const SpDev& sp, int prec)
     return prec == AVL_FP32 ? (size_t)4 * win_plane(sp.Wmax, sp.nx) : 0;
 }
 
+// the FP64 window's copies by lane, beside the window that takes their sums
+static size_t copy_bytes(const SpDev& sp, int prec)
+{
+    const int cs = prec == AVL_FP32 ? 0 : win_copies_log2(sp.M, sp.Wmax, sp.nx);
+    return cs ? window_bytes(sp, prec) << cs : 0;
+}
+
 size_t pd1_smem_bytes(const SpDev& sp, int prec)
 {
     size_t eb = (size_t)sp.nx * (prec == AVL_FP32 ? 4 : 8);
     eb = (eb + 15) & ~size_t(15);
     return eb + 32 + (size_t)2 * HIST_S * 4 + (((size_t)4 * sp.nx + 15) & ~size_t(15)) + window_bytes(sp, prec) +
-           fref_bytes(sp, prec);
+           fref_bytes(sp, prec) + copy_bytes(sp, prec);
 }
 
 // ---------------------------------------------------------------------------
@@ -784,7 +791,10 @@ __global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restri
     double* win = reinterpret_cast<double*>(smem + eb + 32 + 2 * HIST_S * 4 + ((4 * nx + 15) & ~15));
     const int plane = win_plane(W, nx);
     const size_t win_bytes = (size_t)2 * 8 * plane;
-    unsigned long long* wden = reinterpret_cast<unsigned long long*>(win + plane);
+    // copies of the window by lane, summed into it at the end
+    const int cs = win_copies_log2(sp.M, W, nx), lc = threadIdx.x & ((1 << cs) - 1);
+    double* wnum = cs ? win + 2 * plane : win;
+    unsigned long long* wden = reinterpret_cast<unsigned long long*>(wnum + ((size_t)plane << cs));
 
     const bool use_bulk = PUSH && nx % 2 == 0;
     if (threadIdx.x == 0) {
@@ -813,8 +823,8 @@ __global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restri
         }
     }
     {   // zero the window while the field is in flight
-        float4* w4 = reinterpret_cast<float4*>(win);
-        const int n4 = (int)(win_bytes / 16);
+        float4* w4 = reinterpret_cast<float4*>(wnum);
+        const int n4 = (int)((win_bytes << cs) / 16);
         for (int i = threadIdx.x; i < n4; i += PD_THREADS) w4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     if (PUSH && !use_bulk)
@@ -896,12 +906,14 @@ __global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restri
                         const long long u = u52 << 5, w = w52 << 5;
                         const long long a3 = fx_mul(fx_split(u), fx_split(w >> 1)), a2 = w - a3, a1 = u - a3;
                         const long long a[4] = {(FX_ONE << 5) - u - a2, a1, a2, a3};
-                        const int cell[4] = {wa * nx + ia, wc * nx + ib, (wa + 1) * nx + ia, (wc + 1) * nx + ib};
+                        const int c0 = wa * nx + ia, c1 = wc * nx + ib;
+                        const int cell[4] = {(c0 << cs) + lc, (c1 << cs) + lc, ((c0 + nx) << cs) + lc,
+                                             ((c1 + nx) << cs) + lc};
                         unsigned long long old[4];
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
                             old[k] = atomicAdd(wden + cell[k], (unsigned long long)a[k]);
-                            atomicAdd(win + cell[k], fx_scale(fx_double(a[k]), -57) * f);
+                            atomicAdd(wnum + cell[k], fx_scale(fx_double(a[k]), -57) * f);
                         }
                         // a weight carries out of a word only from its last 2^57
                         if (max(max(old[0], old[1]), max(old[2], old[3])) >> 57 == 127) {
@@ -939,8 +951,21 @@ __global__ void __launch_bounds__(PD_THREADS, 1) k_pd1x(const StepArgs* __restri
     __syncthreads();
     if (PUSH)
         for (int i = threadIdx.x; i < HIST_S; i += PD_THREADS) sp.cnt[1 - hs][(size_t)c * HIST_S + i] = scnt[i];
-    for (int i = threadIdx.x; i < plane; i += PD_THREADS)
-        win[plane + i] = fx_scale(fx_double(wden[i]), -57);
+    if (cs) {
+        const int nc = 1 << cs;
+        for (int i = threadIdx.x; i < 2 * plane; i += PD_THREADS) {
+            const bool den = i >= plane;
+            const size_t o = (size_t)(den ? i - plane : i) << cs;
+            double sum = 0.0;
+            for (int q = 0; q < nc; ++q) {
+                const size_t k = o + ((q + i) & (nc - 1));   // (the lanes' banks apart)
+                sum += den ? fx_scale(fx_double(wden[k]), -57) : wnum[k];
+            }
+            win[i] = sum;
+        }
+    } else {
+        for (int i = threadIdx.x; i < plane; i += PD_THREADS) win[plane + i] = fx_scale(fx_double(wden[i]), -57);
+    }
     __syncthreads();
     // flush the window to this chunk's partial sums with one bulk copy
     if (threadIdx.x == 0) {

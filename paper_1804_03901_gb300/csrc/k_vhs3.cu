@@ -709,6 +709,9 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 3 : (CPT == 2 ? 2 : 1))
 // followed a much larger one: k_pd3x 8.54 -> 8.79 ms), and a value whose
 // exponent the sums do not hold goes with the small corners.
 constexpr float SMALL3 = 1.0f / (1 << 20);
+// Up to so many of them in a chunk take a thread per corner (8.76 ms at 134 M
+// markers; a thread per marker 11.7), more a thread per marker (16.8 M markers
+// on an unjittered lattice: 2.52 -> 1.96 ms)
 constexpr int PARK_FEW = 48;
 
 struct FxCol {
