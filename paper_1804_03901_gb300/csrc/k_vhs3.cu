@@ -189,7 +189,10 @@ struct Stage3 {
     // take its square root), so that few segments take a second chunk
     static constexpr int NB = 640;
     static constexpr int MPT = (NB + P3_THREADS - 1) / P3_THREADS;
-    static constexpr int NM = 64;                            // movers of a chunk kept in shared memory
+    // movers of a chunk kept in shared memory (the others are deposited by their
+    // own threads; 16.8 M markers, steps of 0.2 and 0.5: 1.16 and 1.58 ms with 64
+    // and one corner at a time, 0.86 and 1.18 ms; 192 cost the third CTA's L1)
+    static constexpr int NM = 128;
     static constexpr int NF = 6;
     static constexpr int AL = 4;                             // markers per 16 bytes
     static constexpr int SLEN = NB + 2 * AL;                 // staged entries per field
@@ -557,7 +560,26 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 3 : (CPT == 2 ? 2 : 1))
                     if (o < S::NM) {
                         mv[2 * o] = make_float4(u, f, w, __int_as_float(bin));
                         mv[2 * o + 1] = make_float4(wy, wz, __int_as_float(jx), 0.f);
-                    } else {
+                    } else if constexpr (PUSH) {
+                        const int x1 = bin + 1 == nx ? 0 : bin + 1;
+#pragma unroll 1
+                        for (int q = 0; q < 4; ++q) {
+                            const bool okq = q == 0 ? pl.ok[0] : q == 1 ? pl.ok[1] : q == 2 ? pl.ok[2] : pl.ok[3];
+                            if (!okq) continue;
+                            const int base = q == 0 ? pl.base[0] : q == 1 ? pl.base[1] : q == 2 ? pl.base[2] : pl.base[3];
+                            const float p = ((q & 1) ? wy : 1.f - wy) * ((q & 2) ? wz : 1.f - wz);
+                            float* g = gacc + base + jx * nx;
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const float al = (k & 1 ? u : 1.f - u) * (k & 2 ? w : 1.f - w) * p;
+                                const int row = jx + (k >> 1);
+                                if (al == 0.f || row < 0 || row >= nvx) continue;
+                                float* const gg = g + (k >> 1) * nx + (k & 1 ? x1 : bin);
+                                atomicAdd(gg, al * f);
+                                atomicAdd(gg + cells, al);
+                            }
+                        }
+                    } else {   // (the instance without the push has hardly any; its registers)
 #pragma unroll 1
                         for (int c = 0; c < 16; ++c)
                             deposit_corner(gacc, cells, pl, nx, nvx, bin, u, jx, w, wy, wz, f, c);
