@@ -559,7 +559,7 @@ def run_ours(args):
         ens = measure_ensemble(A, args, stream)
 
     l2 = {"two_stream": "inputs larger than L2 (markers 16 B each, 268 MB per step read)",
-          "bump_on_tail": "inputs larger than L2 (markers 24 B (FP32) / 40 B (FP64) each, 3.2 / 5.4 GB per step)",
+          "bump_on_tail": "inputs larger than L2 (markers 24 B (FP32) / 40 B (FP64) each read, 3.2 / 5.4 GB per step; an FP64 marker is stored in 56 B)",
           "bernstein": "inputs larger than L2 (markers 24 B each, 3.2 GB per step read)",
           "landau_paper": "inputs larger than L2 (markers 24 B each, 324 MB per step read)",
           "landau": "small workload (fits in L2)"}[args.workload]

@@ -340,7 +340,7 @@ void green_table(int nx, const double* gm, double* G);
 cudaError_t launch_poisson_dense(const double* rho, double* E, int nx, const double* G, cudaStream_t st);
 cudaError_t launch_poisson(const double* rho, double* E, int nx, const double2* tw, const double* gmul,
                            cudaStream_t st);
-// table of the FP64 entropy logarithm: tab[j] = (log c_j, 1 / c_j), c_j = 1 + (j + 1/2) / 128
+// table of the FP64 entropy logarithm: tab[j] = (2^62 / c_j, 2^53 log c_j), c_j = 1 + (j + 1/2) / 2048
 cudaError_t init_log_table(longlong2* tab, cudaStream_t st);
 
 }  // namespace avl

@@ -91,8 +91,8 @@ struct Pos<float> {
 // cells everywhere (a double of the same x resolves 2^-52 x), and the
 // cloud-in-cell reads the weight straight from the bits: the 52 low bits of
 // X - 2^51 are the mantissa of 1 + w, so that w and the lower cell cost one
-// FP64 operation instead of four (the form is limited by the FP64 pipe).
-// The drift converts the displacement once (a multiply and a conversion).
+// FP64 operation instead of four, and none where the weights stay integers
+// (k_pd1x, k_pd3x, k_ad_depx).  The drift converts the displacement once.
 struct PosX {
     long long X;
     static constexpr double ONE = 4503599627370496.0;   // 2^52: one cell

@@ -15,9 +15,14 @@
 // The low limbs are signed, so that the product of two of them, which is
 // left out, is at most a quarter of the sum's unit, of either sign.  The units
 // are absolute, so what would reach a cell with a small weight only, and values
-// outside FX_EMIN .. FX_EMAX, are summed in FP64 instead (k_pd3x, k_pd1x).  Against
-// exact rational sums of 4 to 12 markers with values over one e-fold: f
-// 7e-17 rms, weights 5e-17 (the same sums in FP64: 1.3e-16 and 1e-16).
+// outside FX_EMIN .. FX_EMAX, are summed in FP64 instead (k_pd3x, k_pd1x,
+// k_ad_depx).  Against exact rational sums of 4 to 12 markers with values over
+// one e-fold: f 7e-17 rms, weights 5e-17 (the same sums in FP64: 1.3e-16 and
+// 1e-16).  In the least favourable cell,
+// one reached by one weight just above the kernel's limit, n is within 2^-36
+// (k_pd3x), 2^-33 (k_pd1x) and 2^-41 (k_ad_depx) of itself; f within 2^-36
+// (k_pd3x, whose numerators are rounded apart from its weights), and to FP64's
+// rounding in the other two, which take the same weights above and below.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -76,17 +81,6 @@ struct FxSum {
     }
     // whole units, to nearest
     __device__ __forceinline__ long long units() const { return h + ((m + (1 << (FX_LIMB - 1))) >> FX_LIMB); }
-    // the same value with 0 <= m < 2^28
-    __device__ __forceinline__ void carry()
-    {
-        h += m >> FX_LIMB;
-        m &= (1ll << FX_LIMB) - 1;
-    }
-    __device__ __forceinline__ void shr(int s)
-    {
-        h >>= s;
-        m >>= s;
-    }
 };
 
 // f as mant 2^(e - 1078), |mant| < 2^56, e >= 1 the exponent field of f

@@ -11,8 +11,8 @@
 // The engine keeps its own markers in the fixed lattice order (marker m =
 // cell * ppc + sub, as created), so that the adjoint variables of a marker
 // stay aligned across steps.  Per step n the forward pass deposits with
-// global atomics, forms F = N / D and the charge, solves for E (the shared
-// FFT kernel) and pushes.  Checkpoints of (x, v) every K steps; the backward
+// global atomics, forms F = N / D and the charge, solves for E (the circulant
+// product up to GREEN_MAX cells, beyond that the FFT) and pushes.  Checkpoints of (x, v) every K steps; the backward
 // pass recomputes each segment of K states from its checkpoint, storing
 // positions, velocities, the grids D, F and E of every state, then walks it
 // backwards:

@@ -430,8 +430,8 @@ __global__ void __cluster_dims__(FIELD_CLUSTER, 1, 1) __launch_bounds__(FIELD_TH
     // Grids that are no power of two (and small enough for the Green's
     // function table): the product spread over CTAs 1 .. 7 in place of CTA
     // 0's direct transforms, whose 2 nx^2 FP64 operations one SM takes (nx =
-    // 300: 112 -> 20 us for the kernel, nx = 100: 52 -> 17 us; a power of two
-    // takes the FFT, 18 us at 64 and 27 us at 512).
+    // 300: 112 -> 25 us for the kernel, nx = 100: 53 -> 27 us; a power of two
+    // takes the FFT, 18 us at 64 and 29 us at 512).
     const bool dense = !fd.pow2 && fd.green != nullptr;
     if (dense) {
         if (rank != 0) {

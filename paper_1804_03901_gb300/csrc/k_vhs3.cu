@@ -200,8 +200,9 @@ struct Stage3 {
 
 // FP64 (k_pd3x), markers per chunk: more than a segment of two markers per
 // cell at nx = 256 (512, give or take its square root), so that few segments
-// take a second chunk, and two CTAs per SM with the shared memory it needs
-// (97 KB).  64^3 bump-on-tail: 8.29 ms with 640 or 576, 8.40 with 544.
+// take a second chunk (longer ones, as of larger nx or more markers per cell,
+// walk two or more), and two CTAs per SM with the shared memory it needs
+// (98 KB).  64^3 bump-on-tail: 8.29 ms with 640 or 576, 8.40 with 544.
 constexpr int NB3X = 640;
 constexpr int MPT3X = (NB3X + P3_THREADS - 1) / P3_THREADS;
 
@@ -712,7 +713,8 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 3 : (CPT == 2 ? 2 : 1))
 // Bound by the latency of its phases (16 warps per SM, four barriers per
 // chunk; issue slots 34 % busy, multiply-add pipe 45 %, shared memory 37 %,
 // FP64 pipe 23 %).  134 M markers, 256 x 64^3: 16.95 -> 8.29 ms against the
-// same sums in FP64; measured and left out: balanced columns with the sums in
+// same sums in FP64, 8.76 ms with what keeps small cells right (SMALL3 below);
+// measured and left out: balanced columns with the sums in
 // shared memory (10.3 ms, its random payload reads fill the shared-memory
 // pipe), two threads per column (9.5 ms), the push of the next chunk beside
 // the gather (9.5 ms, its second staging buffer and tables cost more
