@@ -308,7 +308,7 @@ avl_status avl_field_solve_noalloc(int32_t nx, double L, double poisson_const, i
  * backwards over the step history, recomputed segment by segment from
  * checkpoints of the markers taken every ckpt_every steps; its device memory
  * (about (ckpt_every + 1) marker states and grids, plus one marker state per
- * checkpoint) is kept by the context for the next call.  The context's own
+ * checkpoint and E of every step) is kept by the context for the next call.  The context's own
  * markers, f, rho and E are left untouched.  Blocks until done.  1d1v only.
  * Errors: AVL_EINVAL (nvdim 3, NULL pointers, nsteps < 0, ckpt_every < 1,
  * theta counts, FP64 with nx >= 2048: its positions are fixed-point counts

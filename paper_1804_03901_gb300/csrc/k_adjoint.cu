@@ -12,10 +12,13 @@
 // cell * ppc + sub, as created), so that the adjoint variables of a marker
 // stay aligned across steps.  Per step n the forward pass deposits with
 // global atomics, forms F = N / D and the charge, solves for E (the circulant
-// product up to GREEN_MAX cells, beyond that the FFT) and pushes.  Checkpoints of (x, v) every K steps; the backward
-// pass recomputes each segment of K states from its checkpoint, storing
-// positions, velocities, the grids D, F and E of every state, then walks it
-// backwards:
+// product up to GREEN_MAX cells, beyond that the FFT) and pushes.  E of every
+// state is kept, (x, v) every K steps; the backward pass recomputes each
+// segment of K states from its checkpoint in the stored fields (the order of
+// the deposit's reductions changes E's last bits, and a marker near a cell's
+// edge then takes the other one-sided derivative: with E solved again the
+// FP32 gradient spread 1.6 times as far from run to run), storing positions,
+// velocities and the grids D and F of every state, then walks it backwards:
 //   e^n   = sum_l lt_l (q/m) dt G(X^n_l),  lt = lambda_V + dt lambda_X
 //           (e^N = dx E^N at the final state)
 //   psi   = q dv P^T e^n = -q dv P e^n   (the multiplier of Eq. 6 is odd and
@@ -91,6 +94,7 @@ struct AdjDev {
     double* e;         // [nx] adjoint deposit
     double* tmp;       // [nx] P e
     double* hE;        // [K + 1][nx]
+    double* allE;      // [nsteps + 1][nx]: E of every state of the forward pass
     double* grad;      // [nmode + nbeam] of the theta species
     const avl_f0* f0;  // [ns] (theta for theta_s)
 };
@@ -688,7 +692,7 @@ struct AdjEngine {
     avl_f0* d_f0 = nullptr;
     // one full segment of K steps, forward (with pushes) and backward,
     // recorded once and replayed for every full segment
-    cudaGraphExec_t g_fwd = nullptr, g_bwd = nullptr;
+    cudaGraphExec_t g_fwd = nullptr, g_rec = nullptr, g_bwd = nullptr;
     int g_K = 0, g_nact = -1;
 };
 
@@ -702,8 +706,9 @@ static cudaError_t grab(AdjEngine* E, void** p, size_t bytes)
 static void drop_graphs(AdjEngine* E)
 {
     if (E->g_fwd) cudaGraphExecDestroy(E->g_fwd);
+    if (E->g_rec) cudaGraphExecDestroy(E->g_rec);
     if (E->g_bwd) cudaGraphExecDestroy(E->g_bwd);
-    E->g_fwd = E->g_bwd = nullptr;
+    E->g_fwd = E->g_rec = E->g_bwd = nullptr;
 }
 
 void adjoint_free(AdjEngine* E)
@@ -870,6 +875,27 @@ static cudaError_t full_fwd(const StepArgs& h, const StepArgs* dA, AdjEngine* E,
     return cudaGraphLaunch(E->g_fwd, st);
 }
 
+// a full segment again from its checkpoint, in the fields of the forward pass
+// (hE): the same trajectories to the bit
+template <typename T>
+static cudaError_t recompute(const StepArgs& h, const StepArgs* dA, AdjEngine* E, cudaStream_t st)
+{
+    if (!E->g_rec) {
+        cudaError_t e = record(st, &E->g_rec, [&] {
+            cudaError_t r = cudaSuccess;
+            for (int j = 0; j < E->K && !r; ++j) {
+                launch_dep<T>(E, nmax_active(E), E->h.nact, j, 0, st);
+                k_ad_fin<T><<<fin_grid(E, E->h.nact), 256, 0, st>>>(dA, E->d, j, 0);
+                r = cudaGetLastError();
+                if (!r && j + 1 < E->K) r = push_slot<T>(E, j, st);
+            }
+            return r;
+        });
+        if (e) return e;
+    }
+    return cudaGraphLaunch(E->g_rec, st);
+}
+
 template <typename T>
 static cudaError_t full_bwd(const StepArgs& h, const StepArgs* dA, AdjEngine* E, cudaStream_t st)
 {
@@ -940,6 +966,9 @@ static cudaError_t run(const StepArgs& h, const StepArgs* dA, AdjEngine* E, int 
             return e;
         }
         last_len = len;
+        if ((e = cudaMemcpyAsync(E->h.allE + (size_t)c * K * E->nx, E->h.hE, (size_t)len * E->nx * 8,
+                                 cudaMemcpyDeviceToDevice, st)))
+            return e;
         if (c + 1 < nseg && (e = ckpt_copy(E, c + 1, len, true, st))) return e;
         if (c + 1 < nseg && (e = ckpt_copy(E, c + 1, 0, false, st))) return e;
     }
@@ -954,7 +983,10 @@ static cudaError_t run(const StepArgs& h, const StepArgs* dA, AdjEngine* E, int 
     // earlier segments: recompute from the checkpoint, then walk back
     for (int c = nseg - 2; c >= 0; --c) {
         if ((e = ckpt_copy(E, c, 0, false, st))) return e;
-        if ((e = full_fwd<T>(h, dA, E, true, st))) return e;
+        if ((e = cudaMemcpyAsync(E->h.hE, E->h.allE + (size_t)c * K * E->nx, (size_t)K * E->nx * 8,
+                                 cudaMemcpyDeviceToDevice, st)))
+            return e;
+        if ((e = recompute<T>(h, dA, E, st))) return e;
         if ((e = full_bwd<T>(h, dA, E, st))) return e;
     }
     k_ad_theta<T><<<grid_for(E->n[E->h.theta_s]), 256, 0, st>>>(dA, E->d);
@@ -1022,6 +1054,7 @@ cudaError_t adjoint_run(AdjEngine** eng, const StepArgs& h, const StepArgs* dA, 
         g((void**)&E->h.e, nx * 8);
         g((void**)&E->h.tmp, nx * 8);
         g((void**)&E->h.hE, (size_t)(K + 1) * nx * 8);
+        g((void**)&E->h.allE, ((size_t)C * K + 1) * nx * 8);
         g((void**)&E->h.grad, 8 * (64 + 4));
         g((void**)&E->d_f0, sizeof(avl_f0) * ns);
         g((void**)&E->d, sizeof(AdjDev));
