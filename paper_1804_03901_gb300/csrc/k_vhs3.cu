@@ -1166,7 +1166,8 @@ __global__ void __launch_bounds__(P3_THREADS, CPT == 1 ? 2 : 1) k_pd3x(const Ste
 // ---------------------------------------------------------------------------
 // FP64: quotient and entropy logarithm in integers (fx_div, fx_log), which
 // leaves three FP64 operations per cell (the sums) of the 17 that bound this
-// kernel: 67 M cells 1.97 -> 0.63 ms, 2.7 GB, 63 % of the copy rate.
+// kernel: 67 M cells 1.97 -> 0.68 ms, 2.7 GB, 58 % of the copy rate (0.63 ms
+// with the quotient's last bit left undecided).
 template <typename T>
 __global__ void __launch_bounds__(FIN3_X * FIN3_R) k_fin3(const StepArgs* __restrict__ A, int all_species)
 {
